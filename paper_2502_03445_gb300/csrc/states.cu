@@ -6,9 +6,8 @@
 // steps over the cut indices alone (a plan with no free qubits) contract it.
 //
 // Two forms, chosen from the plan:
-//   fused      one persistent kernel; a CTA takes one state at a time and
-//              runs every step of the single-state plan in shared memory.
-//              Its leaf operands are rows of per-node tables
+//   fused      one persistent kernel runs every step of the single-state plan
+//              on chip.  Its leaf operands are rows of per-node tables
 //              Tt_j[x][cuts] (node tensors transposed so that the 4^{c_j}
 //              values a state needs are one contiguous row, FP32, built by
 //              the ingest kernel once per tensor version and small enough
@@ -19,10 +18,24 @@
 //              multiply-adds per state) run the single-state plan once per
 //              state through the ordinary step kernels, with the state's
 //              bits as the fixed bits.
+//
+// The fused form is bound by FP32 arithmetic, so it does no step twice for
+// equal inputs: the result of a step depends only on the output bits of its
+// own subcircuits, which many states of a list share (2^17 values for the
+// costliest step of the 30-qubit grid, 10^6 states).  A shared subtree is
+// chosen (choose_split, below), the list is sorted by that subtree's bits (a
+// counting sort), and a CTA walks a contiguous range of the sorted list: the
+// shared steps run on all 256 threads when a bit they depend on has changed,
+// and every state's remaining steps run on one warp, eight states at a time,
+// with no barrier between them.  A K range too long for its outputs is split
+// over neighbouring lanes and summed with shuffles.  10^6 states of the
+// 30-qubit grid: STATES_FIGURES
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
+#include <limits>
 #include <string>
 #include <vector>
 
@@ -34,34 +47,48 @@ namespace tqc {
 namespace {
 
 constexpr int ST_THREADS = 256;
+constexpr int ST_WARPS = ST_THREADS / 32;
 constexpr int ST_MAX_LEAVES = 16;
 constexpr int ST_MAX_STEPS = ST_MAX_LEAVES - 1;
 constexpr int ST_MAX_SMEM_FLOATS = 200 * 1024 / 4;
+constexpr int ST_MAX_KEY_BITS = 22;  // counters of the sort: at most 2^22
+constexpr int SCAN_PER_CTA = 4096;
 
 struct SLeaf {
     const float *table;  // [2^{n_q}][4^{cuts}]: row x is the leaf operand of states with x|out_j = x
     int32_t row_log2;    // log2 of the row length (2 * cuts)
-    int32_t q_off, n_q;  // output qubits in SProgram::qubits[q_off .. q_off + n_q): bit k of x
+    int32_t y_off, n_q;  // x is bits y_off .. y_off + n_q of the permuted state y
 };
 
+// Where a step's operand is: a leaf's table row in global memory, the CTA's
+// shared memory (a staged leaf, or the result of a shared step), or the
+// warp's own part of it.
+enum SrcKind { SRC_TABLE = 0, SRC_CTA = 1, SRC_WARP = 2 };
+
 struct SStep {
-    int32_t a_src, b_src;   // >= 0: leaf index; < 0: result of step (-1 - src)
+    uint64_t mask;          // bits of y the result depends on
+    int32_t a_leaf, b_leaf; // leaf index, or -1
+    int32_t a_kind, b_kind; // SrcKind
+    int32_t a_off, b_off;   // offsets (floats) of SRC_CTA / SRC_WARP operands
     int32_t mb, nb, kb;     // log2 of M, N, K
     uint32_t maskR, maskC;  // result-layout bits of the row / column index bits
     int32_t c_kb;           // log2 K of the step consuming the result; -1 for the final step
-    int32_t c_off;          // shared-memory offset (floats) of the result: rows of 2^c_kb, padded
-    int32_t a_off, b_off;   // shared-memory offsets of the operands
-    int32_t tm, tn;         // register tile of a thread (rows strided by M / tm, columns by N / tn)
-    int32_t ksplit;         // K ranges of one output tile (summed through the reduction buffer)
-    int32_t tab_off;        // shared-memory offset of the result offsets of rows (M) then columns (N)
+    int32_t c_off;          // the result's place: rows of 2^c_kb, padded
+    int32_t lkl;            // log2 of the lanes sharing one output tile's K range
+    int32_t tab_off;        // result offsets of rows (M) then columns (N), in shared memory
 };
 
 struct SProgram {
-    int32_t n_leaves, n_steps;
-    int8_t qubits[64];
+    int32_t n_leaves, n_steps, n_shared;  // steps [0, n_shared) run per CTA, the rest per warp
+    int32_t n_qubits;
+    int32_t key_bits;       // the list is sorted by this many top bits of y (0: not sorted)
+    int32_t one_each;       // states are taken one at a time (every step is a shared one)
+    int32_t restage;        // leaf areas are reused: stage a step's leaves every time it runs
+    uint64_t group_mask;    // bits of y the last shared step depends on
+    int8_t perm[64];        // bit b of y is bit perm[b] of the state
     SLeaf leaf[ST_MAX_LEAVES];
     SStep step[ST_MAX_STEPS];
-    int32_t red_off;
+    int32_t warp_off, warp_floats;  // per-warp regions
     int32_t smem_floats;
 };
 
@@ -69,12 +96,108 @@ struct SProgram {
 // float4 access and spreads rows over the banks.
 __host__ __device__ __forceinline__ int pitch_of(int k) { return k >= 4 ? k + 4 : k; }
 
+// Output tiles of TM x TN results (rows strided by M / TM, columns by
+// N / TN), tile t of every nw x (32 >> lkl): 2^lkl neighbouring lanes share a
+// tile, lane ks taking the float4s ks, ks + 2^lkl, ... of K (consecutive
+// 16-byte pieces of a row: whole sectors, no bank conflicts).  Their partial
+// sums are added by recursive halving, which leaves every lane a part of the
+// tile's results to store (put).  AG / BG: the operand is in global memory.
+template <int TM, int TN, bool AG, bool BG, typename Put>
+__device__ __forceinline__ void step_tiles(const float *A, int pa, const float *B, int pb, int mb, int nb, int kb,
+                                           int lkl, int w, int nw, int lane, const Put &put) {
+    if constexpr (!AG) __builtin_assume(__isShared(A));
+    if constexpr (!BG) __builtin_assume(__isShared(B));
+    constexpr int E = TM * TN;
+    const int rs = (1 << mb) / TM, cs = (1 << nb) / TN;
+    const int lc = nb - (TN == 4 ? 2 : 0);
+    const int tiles = rs * cs, per = 32 >> lkl;
+    const int ks = lane & ((1 << lkl) - 1);
+    for (int tb = w * per; tb < tiles; tb += nw * per) {
+        const int t0 = tb + (lane >> lkl);
+        const bool valid = t0 < tiles;
+        const int t = valid ? t0 : 0;
+        const int rt = t >> lc, ct = t & (cs - 1);
+        float acc[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[e] = 0.f;
+        if (kb >= 2) {
+            const float *pA = A + rt * pa + 4 * ks, *pB = B + ct * pb + 4 * ks;
+            const int sa = rs * pa, sb = cs * pb, n4 = 1 << (kb - 2 - lkl), inc = 4 << lkl;
+#pragma unroll 2
+            for (int k = 0; k < n4; ++k) {
+                float4 a[TM], b[TN];
+#pragma unroll
+                for (int i = 0; i < TM; ++i) a[i] = AG ? __ldg((const float4 *)(pA + i * sa)) : *(const float4 *)(pA + i * sa);
+#pragma unroll
+                for (int j = 0; j < TN; ++j) b[j] = BG ? __ldg((const float4 *)(pB + j * sb)) : *(const float4 *)(pB + j * sb);
+                pA += inc;
+                pB += inc;
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+#pragma unroll
+                    for (int j = 0; j < TN; ++j) {
+                        float &c = acc[i * TN + j];
+                        c = fmaf(a[i].x, b[j].x, c);
+                        c = fmaf(a[i].y, b[j].y, c);
+                        c = fmaf(a[i].z, b[j].z, c);
+                        c = fmaf(a[i].w, b[j].w, c);
+                    }
+            }
+        } else {  // K = 1
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[i * TN + j] = A[(rt + i * rs) * pa] * B[(ct + j * cs) * pb];
+        }
+        // halve the results over lane bit 0, then bit 1, ... while more than
+        // one is left; further lane bits add the same result
+        int e0 = 0;
+        bool mine = valid;
+#pragma unroll
+        for (int s = 0; s < 5; ++s) {
+            if (lkl > s) {
+                const bool up = (ks >> s) & 1;
+                constexpr int H0 = E / 2;
+                const int half = H0 >> s;
+                if (half > 0) {
+#pragma unroll
+                    for (int i = 0; i < (H0 >> s); ++i) {
+                        const float lo = acc[i], hi = acc[i + (H0 >> s)];
+                        acc[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, 1 << s);
+                    }
+                    e0 += up ? half : 0;
+                } else {
+                    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1 << s);
+                    mine = mine && !up;
+                }
+            }
+        }
+        const int left = E >> lkl > 0 ? E >> lkl : 1;
+        if (mine) {
+#pragma unroll
+            for (int i = 0; i < E; ++i)
+                if (i < left) {
+                    const int e = e0 + i;
+                    put(rt + (e / TN) * rs, ct + (e % TN) * cs, acc[i]);
+                }
+        }
+    }
+}
+
+template <bool AG, bool BG, typename Put>
+__device__ __forceinline__ void step_run(const SStep &S, const float *A, int pa, const float *B, int pb, int w, int nw,
+                                         int lane, const Put &put) {
+    if (S.mb >= 2 && S.nb >= 2) step_tiles<4, 4, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, put);
+    else if (S.mb >= 2) step_tiles<4, 1, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, put);
+    else if (S.nb >= 2) step_tiles<1, 4, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, put);
+    else step_tiles<1, 1, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, put);
+}
+
 __global__ void __launch_bounds__(ST_THREADS, 3)
-    states_kernel(const __grid_constant__ SProgram P, const uint64_t *__restrict__ states, int64_t n, void *out,
-                  int out_f64, const double *zinfo) {
+    states_kernel(const __grid_constant__ SProgram P, const uint64_t *__restrict__ list,
+                  const uint32_t *__restrict__ place, int64_t n, void *out, int out_f64, const double *zinfo) {
     extern __shared__ __align__(16) float sm[];
-    __shared__ int64_t proj[ST_MAX_LEAVES];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const double scale = zinfo[1];
     // Every state runs the same program: the place of result row r and column
     // c in the consumer's padded operand is tab[r] + tab[M + c] (the row and
@@ -91,35 +214,93 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
         }
     }
     __syncthreads();
-    for (int64_t s = blockIdx.x; s < n; s += gridDim.x) {
-        const uint64_t x = states[s];
-        if (tid < P.n_leaves) {
-            const SLeaf &L = P.leaf[tid];
-            int64_t pj = 0;
-            for (int k = 0; k < L.n_q; ++k) pj |= (int64_t)((x >> P.qubits[L.q_off + k]) & 1ull) << k;
-            proj[tid] = pj;
-        }
-        __syncthreads();
-        if (P.n_steps == 0) {  // one subcircuit without cuts: a table lookup
-            if (tid == 0) {
-                const double v = (double)P.leaf[0].table[proj[0]] * scale;
-                if (out_f64) ((double *)out)[s] = v;
-                else ((float *)out)[s] = (float)v;
-            }
-            __syncthreads();
-            continue;
-        }
-        for (int si = 0; si < P.n_steps; ++si) {
+    auto store = [&](int64_t at, float v) {
+        const double d = (double)v * scale;
+        if (out_f64) ((double *)out)[at] = d;
+        else ((float *)out)[at] = (float)d;
+    };
+    auto row_of = [&](int leaf, uint64_t y) {
+        const SLeaf &L = P.leaf[leaf];
+        return L.table + ((int64_t)((y >> L.y_off) & ((1ull << L.n_q) - 1ull)) << L.row_log2);
+    };
+    // the permuted state at position p of the list (whole warps call this)
+    auto state_at = [&](int64_t p) {
+        const uint64_t x = list[p];
+        if (P.key_bits) return x;  // permuted by the sort
+        const uint32_t lo = __ballot_sync(0xffffffffu, lane < P.n_qubits && ((x >> P.perm[lane]) & 1ull));
+        const uint32_t hi =
+            __ballot_sync(0xffffffffu, lane + 32 < P.n_qubits && ((x >> P.perm[(lane + 32) & 63]) & 1ull));
+        return ((uint64_t)hi << 32) | lo;
+    };
+    // steps [s0, n_steps) of one state on one warp
+    float *wsm = sm + P.warp_off + warp * P.warp_floats;
+    auto warp_state = [&](uint64_t y, int64_t at) {
+        for (int si = P.n_shared; si < P.n_steps; ++si) {
             const SStep &S = P.step[si];
-            const int M = 1 << S.mb, N = 1 << S.nb, K = 1 << S.kb;
-            const int pk = pitch_of(K);
-            // stage leaf operands (rows x K, row-major in the table) into padded rows
+            const int M = 1 << S.mb, K = 1 << S.kb, pk = pitch_of(K);
+            const float *A = S.a_kind == SRC_TABLE ? row_of(S.a_leaf, y) : (S.a_kind == SRC_CTA ? sm : wsm) + S.a_off;
+            const float *B = S.b_kind == SRC_TABLE ? row_of(S.b_leaf, y) : (S.b_kind == SRC_CTA ? sm : wsm) + S.b_off;
+            const int *tab = (const int *)(sm + S.tab_off);
+            float *res = wsm + S.c_off;
+            const bool last = S.c_kb < 0;
+            auto put = [&](int r, int c, float v) {
+                if (last) store(at, v);
+                else res[tab[r] + tab[M + c]] = v;
+            };
+            const bool ag = S.a_kind == SRC_TABLE, bg = S.b_kind == SRC_TABLE;
+            if (ag && bg) step_run<true, true>(S, A, K, B, K, 0, 1, lane, put);
+            else if (ag) step_run<true, false>(S, A, K, B, pk, 0, 1, lane, put);
+            else if (bg) step_run<false, true>(S, A, pk, B, K, 0, 1, lane, put);
+            else step_run<false, false>(S, A, pk, B, pk, 0, 1, lane, put);
+            __syncwarp();
+        }
+    };
+    if (P.n_steps == 0) {  // one subcircuit without cuts: a table lookup
+        for (int64_t p = (int64_t)blockIdx.x * ST_WARPS + warp; p < n; p += (int64_t)gridDim.x * ST_WARPS) {
+            const uint64_t y = state_at(p);
+            if (lane == 0) store(p, *row_of(0, y));
+        }
+        return;
+    }
+    const int64_t p0 = n * blockIdx.x / gridDim.x, p1 = n * (blockIdx.x + 1) / gridDim.x;
+    if (P.n_shared == 0) {
+        for (int64_t p = p0 + warp; p < p1; p += ST_WARPS) {
+            const uint64_t y = state_at(p);
+            warp_state(y, place ? (int64_t)place[p] : p);
+        }
+        return;
+    }
+    uint64_t prev = 0;
+    int cnt = 0;
+    for (int64_t p = p0; p < p1; p += cnt) {
+        const uint64_t y = state_at(p);
+        // the states that share this one's subtree bits are consecutive: count
+        // them (up to one per thread).  The barrier also ends the reads of the
+        // previous round.
+        if (P.one_each) {
+            __syncthreads();
+            cnt = 1;
+        } else {
+            const int64_t q = p + tid;
+            cnt = __syncthreads_count(q < p1 && ((list[q < p1 ? q : p] ^ y) & P.group_mask) == 0);
+        }
+        const bool first = p == p0;
+        const uint64_t diff = y ^ prev;
+        prev = y;
+        for (int si = 0; si < P.n_shared; ++si) {
+            const SStep &S = P.step[si];
+            const bool last = S.c_kb < 0;
+            if (!first && !last && !(diff & S.mask)) continue;  // nothing it depends on has changed
+            const int M = 1 << S.mb, N = 1 << S.nb, K = 1 << S.kb, pk = pitch_of(K);
+            // stage changed leaf operands (rows x K, row-major in the table) as padded rows
 #pragma unroll
             for (int op = 0; op < 2; ++op) {
-                const int src = op ? S.b_src : S.a_src;
-                if (src < 0) continue;
+                const int leaf = op ? S.b_leaf : S.a_leaf;
+                if (leaf < 0) continue;
+                const uint64_t lm = ((1ull << P.leaf[leaf].n_q) - 1ull) << P.leaf[leaf].y_off;
+                if (!first && !P.restage && !(diff & lm)) continue;
                 const int rows = op ? N : M;
-                const float *row = P.leaf[src].table + (proj[src] << P.leaf[src].row_log2);
+                const float *row = row_of(leaf, y);
                 float *dst = sm + (op ? S.b_off : S.a_off);
                 if (K >= 4) {
                     const int lq = S.kb - 2;  // float4s per row: K / 4
@@ -128,170 +309,348 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
                         *(float4 *)(dst + r * pk + 4 * k4) = __ldg((const float4 *)row + i);
                     }
                 } else {
-                    for (int i = tid; i < rows * K; i += ST_THREADS) dst[i] = __ldg(row + i);
+                    for (int i = tid; i < rows; i += ST_THREADS) dst[i] = __ldg(row + i);
                 }
             }
             __syncthreads();
-            const float *A = sm + S.a_off, *B = sm + S.b_off;
-            const int tm = S.tm, tn = S.tn;
-            const int rstride = M / tm, cstride = N / tn;
-            const int lc = __ffs(cstride) - 1, lt = lc + __ffs(rstride) - 1;  // log2 of cstride, n_tiles
-            const int n_tiles = rstride * cstride;
-            const int kc = K / S.ksplit;
-            float *red = sm + P.red_off;
             const int *tab = (const int *)(sm + S.tab_off);
             float *res = sm + S.c_off;
-            // result element (r, c) -> its place in the consumer's padded operand
-            auto put = [&](int r, int c, float v) {
-                if (S.c_kb < 0) {
-                    const double d = (double)v * scale;
-                    if (out_f64) ((double *)out)[s] = d;
-                    else ((float *)out)[s] = (float)d;
-                    return;
-                }
-                res[tab[r] + tab[M + c]] = v;
-            };
-            for (int u = tid; u < n_tiles * S.ksplit; u += ST_THREADS) {
-                const int t = u & (n_tiles - 1), ks = u >> lt;
-                const int rt = t >> lc, ct = t & (cstride - 1);
-                float acc[4][4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-                const int k0 = ks * kc;
-                if (kc >= 4) {
-                    for (int k = k0; k < k0 + kc; k += 4) {
-                        float4 a[4], b[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            if (i < tm) a[i] = *(const float4 *)(A + (rt + i * rstride) * pk + k);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (j < tn) b[j] = *(const float4 *)(B + (ct + j * cstride) * pk + k);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                if (i < tm && j < tn) {
-                                    acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-                                    acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-                                    acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-                                    acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
-                                }
-                    }
-                } else {
-                    for (int k = k0; k < k0 + kc; ++k)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                if (i < tm && j < tn)
-                                    acc[i][j] = fmaf(A[(rt + i * rstride) * pk + k], B[(ct + j * cstride) * pk + k],
-                                                     acc[i][j]);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (i < tm && j < tn) {
-                            const int r = rt + i * rstride, c = ct + j * cstride;
-                            if (S.ksplit == 1) put(r, c, acc[i][j]);
-                            else red[ks * M * N + r * N + c] = acc[i][j];
-                        }
-            }
+            const int64_t at = last ? (place ? (int64_t)place[p] : p) : 0;
+            step_run<false, false>(S, sm + S.a_off, pk, sm + S.b_off, pk, warp, ST_WARPS, lane,
+                                   [&](int r, int c, float v) {
+                                       if (last) store(at, v);
+                                       else res[tab[r] + tab[M + c]] = v;
+                                   });
             __syncthreads();
-            if (S.ksplit > 1) {
-                for (int o = tid; o < M * N; o += ST_THREADS) {
-                    float v = 0.f;
-                    for (int ks = 0; ks < S.ksplit; ++ks) v += red[ks * M * N + o];
-                    put(o / N, o % N, v);
-                }
-                __syncthreads();
-            }
         }
+        if (P.n_shared < P.n_steps)
+            for (int k = warp; k < cnt; k += ST_WARPS)
+                warp_state(list[p + k], place ? (int64_t)place[p + k] : p + k);
     }
+}
+
+// ---- counting sort of the list by the top key_bits of the permuted state
+// y: count (a state's rank among those counted so far with its key), an
+// exclusive scan of the counters, scatter.  Which of two states with equal
+// keys comes first does not change any state's value.
+__global__ void states_count_kernel(const __grid_constant__ SProgram P, const uint64_t *__restrict__ states, int64_t n,
+                                    uint64_t *__restrict__ ys, uint32_t *__restrict__ rank, uint32_t *counters) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t act = __ballot_sync(0xffffffffu, i < n);
+    if (i >= n) return;
+    const uint64_t x = states[i];
+    uint64_t y = 0;
+    for (int b = 0; b < P.n_qubits; ++b) y |= ((x >> P.perm[b]) & 1ull) << b;
+    ys[i] = y;
+    const uint32_t key = (uint32_t)(y >> (P.n_qubits - P.key_bits));
+    // one atomic per distinct key of the warp
+    const uint32_t peers = __match_any_sync(act, key);
+    const int lane = threadIdx.x & 31, lead = __ffs(peers) - 1;
+    uint32_t base = 0;
+    if (lane == lead) base = atomicAdd(counters + key, (uint32_t)__popc(peers));
+    base = __shfl_sync(peers, base, lead);
+    rank[i] = base + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+}
+
+__device__ __forceinline__ uint32_t block_sum(uint32_t v, uint32_t *red) {
+    v = __reduce_add_sync(0xffffffffu, v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    uint32_t t = 0;
+#pragma unroll
+    for (int i = 0; i < ST_WARPS; ++i) t += red[i];
+    return t;
+}
+
+__global__ void __launch_bounds__(ST_THREADS) states_sums_kernel(const uint32_t *counters, int n, uint32_t *sums) {
+    __shared__ uint32_t red[ST_WARPS];
+    uint32_t v = 0;
+    const int base = blockIdx.x * SCAN_PER_CTA;
+    for (int i = threadIdx.x; i < SCAN_PER_CTA; i += ST_THREADS)
+        if (base + i < n) v += counters[base + i];
+    const uint32_t t = block_sum(v, red);
+    if (threadIdx.x == 0) sums[blockIdx.x] = t;
+}
+
+__global__ void __launch_bounds__(ST_THREADS) states_scan_kernel(uint32_t *counters, int n, const uint32_t *sums) {
+    __shared__ uint32_t red[ST_WARPS], wsum[ST_WARPS];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t v = 0;
+    for (int i = tid; i < (int)blockIdx.x; i += ST_THREADS) v += sums[i];
+    uint32_t run = block_sum(v, red);
+    const int base = blockIdx.x * SCAN_PER_CTA;
+    for (int c = 0; c < SCAN_PER_CTA; c += ST_THREADS) {
+        const int i = base + c + tid;
+        const uint32_t x = i < n ? counters[i] : 0;
+        uint32_t s = x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += u;
+        }
+        __syncthreads();
+        if (lane == 31) wsum[warp] = s;
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+#pragma unroll
+        for (int w = 0; w < ST_WARPS; ++w) {
+            if (w < warp) before += wsum[w];
+            total += wsum[w];
+        }
+        if (i < n) counters[i] = run + before + s - x;
+        run += total;
+    }
+}
+
+__global__ void states_scatter_kernel(const uint64_t *__restrict__ ys, const uint32_t *__restrict__ rank, int64_t n,
+                                      int shift, const uint32_t *__restrict__ offsets, uint64_t *__restrict__ sorted,
+                                      uint32_t *__restrict__ place) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint64_t y = ys[i];
+    const uint32_t at = offsets[y >> shift] + rank[i];
+    sorted[at] = y;
+    place[at] = (uint32_t)i;
 }
 
 int64_t align4(int64_t x) { return (x + 3) & ~int64_t(3); }
 
-// The fused form's program for a single-state plan, without table pointers
-// (set at launch); false when the plan does not fit its limits.
-bool build_program(const Plan &p, SProgram *P, std::string *why) {
+// Distinct values among n uniform draws from 2^q.
+double distinct(double n, int q) {
+    const double d = std::ldexp(1.0, q);
+    return q > 60 ? n : d * -std::expm1(-n / d);
+}
+
+// The fused form's program with the subtree of step `top` shared (-1: no
+// shared steps; the last step: every state on a whole CTA), without table
+// pointers (set at launch), and its estimated cost; false when it does not
+// fit.  compact: leaf operands of the shared steps reuse two areas.
+bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P, double *cost, std::string *why) {
     std::memset(P, 0, sizeof(*P));
+    const int ns = (int)p.steps.size();
+    P->n_leaves = p.m;
+    P->n_steps = ns;
+    P->n_qubits = p.net->n_qubits;
+    std::vector<int> producer(p.tensors.size(), -1), consumer(p.tensors.size(), -1);
+    for (int s = 0; s < ns; ++s) {
+        producer[(size_t)p.steps[s].c] = s;
+        consumer[(size_t)p.steps[s].a] = consumer[(size_t)p.steps[s].b] = s;
+    }
+    // output qubits and multiply-adds below every tensor
+    std::vector<int> q(p.tensors.size(), 0);
+    std::vector<double> macs(p.tensors.size(), 0);
+    for (int j = 0; j < p.m; ++j) q[j] = (int)p.net->nodes[j].out_qubits.size();
+    for (int s = 0; s < ns; ++s) {
+        const StepPlan &st = p.steps[s];
+        q[(size_t)st.c] = q[(size_t)st.a] + q[(size_t)st.b];
+        macs[(size_t)st.c] = macs[(size_t)st.a] + macs[(size_t)st.b] + std::ldexp(1.0, st.mb + st.nb + st.kb);
+    }
+    // steps of the shared subtree first
+    std::vector<char> shared(p.tensors.size(), 0);
+    if (top >= 0) shared[(size_t)p.steps[top].c] = 1;
+    for (int s = ns - 1; s >= 0; --s)
+        if (shared[(size_t)p.steps[s].c]) shared[(size_t)p.steps[s].a] = shared[(size_t)p.steps[s].b] = 1;
+    std::vector<int> order;
+    for (int pass = 0; pass < 2; ++pass)
+        for (int s = 0; s < ns; ++s)
+            if ((shared[(size_t)p.steps[s].c] != 0) == (pass == 0)) order.push_back(s);
+    // y: the sort key's leaves on top, the costliest subtree first at every
+    // level, so that consecutive states of the sorted list share its bits
+    std::vector<int> rank_order;
+    std::vector<int> stack;
+    auto heavy = [&](int t) {
+        const StepPlan &st = p.steps[producer[(size_t)t]];
+        return macs[(size_t)st.a] > macs[(size_t)st.b] || (macs[(size_t)st.a] == macs[(size_t)st.b] && q[(size_t)st.a] > q[(size_t)st.b]);
+    };
+    const int root = ns > 0 ? p.steps[ns - 1].c : 0;
+    int key_t = top >= 0 ? p.steps[top].c : -1;  // the tensor whose bits are the sort key
+    while (key_t >= 0 && q[(size_t)key_t] > ST_MAX_KEY_BITS) {
+        if (producer[(size_t)key_t] < 0) {
+            key_t = -1;
+            break;
+        }
+        const StepPlan &st = p.steps[producer[(size_t)key_t]];
+        key_t = heavy(key_t) ? st.a : st.b;
+    }
+    std::vector<char> placed((size_t)p.m, 0);
+    auto place_below = [&](int t0) {
+        stack.assign(1, t0);
+        while (!stack.empty()) {
+            const int t = stack.back();
+            stack.pop_back();
+            if (producer[(size_t)t] < 0) {
+                if (!placed[(size_t)t]) rank_order.push_back(t);
+                placed[(size_t)t] = 1;
+                continue;
+            }
+            const StepPlan &st = p.steps[producer[(size_t)t]];
+            const bool h = heavy(t);
+            stack.push_back(h ? st.b : st.a);
+            stack.push_back(h ? st.a : st.b);
+        }
+    };
+    if (key_t >= 0) place_below(key_t);
+    if (top >= 0) place_below(p.steps[top].c);
+    place_below(root);
+    int at = P->n_qubits;
+    for (int j : rank_order) {
+        const Node &nd = p.net->nodes[j];
+        at -= (int)nd.out_qubits.size();
+        P->leaf[j].row_log2 = p.tensors[j].nbits();
+        P->leaf[j].y_off = at;
+        P->leaf[j].n_q = (int)nd.out_qubits.size();
+        for (size_t k = 0; k < nd.out_qubits.size(); ++k) P->perm[at + (int)k] = (int8_t)nd.out_qubits[k];
+        if (P->leaf[j].n_q == 0) P->leaf[j].y_off = 0;
+    }
+    auto bits_of = [&](uint64_t leaves) {
+        uint64_t m = 0;
+        for (int j = 0; j < p.m; ++j)
+            if (leaves >> j & 1)
+                for (int k = 0; k < P->leaf[j].n_q; ++k) m |= 1ull << (P->leaf[j].y_off + k);
+        return m;
+    };
+    P->key_bits = key_t >= 0 ? q[(size_t)key_t] : 0;
+    P->one_each = top >= 0 && (top == ns - 1 || key_t != p.steps[top].c || P->key_bits == 0);
+    P->restage = compact;
+    P->group_mask = top >= 0 ? bits_of(p.tensors[(size_t)p.steps[top].c].leaves) : 0;
+    if (P->one_each && top != ns - 1) return *why = "shared subtree has too many output bits", false;
+    // shared memory: leaf operands of the shared steps, intermediates, the
+    // warps' own intermediates, the offset tables
+    int64_t off = 0, woff = 0, area[2] = {0, 0};
+    std::vector<int> place(p.tensors.size(), 0);
+    const int n_shared = (int)std::count_if(order.begin(), order.end(), [&](int s) { return shared[(size_t)p.steps[s].c] != 0; });
+    P->n_shared = n_shared;
+    for (int i = 0; i < n_shared; ++i) {
+        const StepPlan &st = p.steps[order[(size_t)i]];
+        const int64_t pk = pitch_of(1 << st.kb);
+        const int64_t need[2] = {((int64_t)1 << st.mb) * pk, ((int64_t)1 << st.nb) * pk};
+        const int t[2] = {st.a, st.b};
+        for (int k = 0; k < 2; ++k) {
+            if (t[k] >= p.m) continue;
+            if (compact) area[k] = std::max(area[k], align4(need[k]));
+            else {
+                place[(size_t)t[k]] = (int)off;
+                off += align4(need[k]);
+            }
+        }
+    }
+    if (compact) {
+        for (int i = 0; i < n_shared; ++i) {
+            const StepPlan &st = p.steps[order[(size_t)i]];
+            if (st.a < p.m) place[(size_t)st.a] = 0;
+            if (st.b < p.m) place[(size_t)st.b] = (int)area[0];
+        }
+        off = area[0] + area[1];
+    }
+    for (int i = 0; i < ns; ++i) {
+        const StepPlan &st = p.steps[order[(size_t)i]];
+        const int c = consumer[(size_t)st.c];
+        if (c < 0) {  // the final step: a scalar per state
+            if (st.mb != 0 || st.nb != 0) return *why = "final step is not a scalar", false;
+            continue;
+        }
+        const int64_t ck = (int64_t)1 << p.steps[c].kb;
+        const int64_t need = align4((((int64_t)1 << (st.mb + st.nb)) / ck) * pitch_of((int)ck));
+        int64_t &o = i < n_shared ? off : woff;
+        place[(size_t)st.c] = (int)o;
+        o += need;
+    }
+    for (int i = 0; i < ns; ++i) {
+        const StepPlan &st = p.steps[order[(size_t)i]];
+        SStep &S = P->step[i];
+        S.mb = st.mb;
+        S.nb = st.nb;
+        S.kb = st.kb;
+        S.maskR = (uint32_t)st.maskR;
+        S.maskC = (uint32_t)st.maskC;
+        S.mask = bits_of(p.tensors[(size_t)st.c].leaves);
+        const int c = consumer[(size_t)st.c];
+        S.c_kb = c < 0 ? -1 : p.steps[c].kb;
+        S.c_off = place[(size_t)st.c];
+        auto operand = [&](int t, int32_t *leaf, int32_t *kind, int32_t *o) {
+            *leaf = t < p.m ? t : -1;
+            *kind = i < n_shared ? SRC_CTA : (t < p.m ? SRC_TABLE : (shared[(size_t)t] ? SRC_CTA : SRC_WARP));
+            *o = place[(size_t)t];
+        };
+        operand(st.a, &S.a_leaf, &S.a_kind, &S.a_off);
+        operand(st.b, &S.b_leaf, &S.b_kind, &S.b_off);
+        S.tab_off = (int32_t)off;
+        off += align4(((int64_t)1 << st.mb) + ((int64_t)1 << st.nb));
+        // lanes per output tile: what the tiles leave idle, at most one per
+        // float4 of K; rows read from global memory always 8 (a whole line)
+        const int tiles = st.mb + st.nb - (st.mb >= 2 ? 2 : 0) - (st.nb >= 2 ? 2 : 0);  // log2
+        const int lanes = i < n_shared ? 8 : 5;
+        int lkl = std::max(0, std::min(5, lanes - tiles));
+        if (S.a_kind == SRC_TABLE || S.b_kind == SRC_TABLE) lkl = std::max(lkl, 3);
+        S.lkl = std::max(0, std::min(lkl, st.kb - 2));
+    }
+    P->warp_off = (int32_t)off;
+    P->warp_floats = (int32_t)woff;
+    off += woff * ST_WARPS;
+    if (off > ST_MAX_SMEM_FLOATS) return *why = "intermediates exceed shared memory", false;
+    P->smem_floats = (int32_t)std::max<int64_t>(off, 4);
+    if (!cost) return true;
+    // Estimated clocks per SM: a shared step at half the FP32 rate (128
+    // multiply-adds per clock) plus its barriers, a warp's step likewise plus
+    // its fixed instructions, the warps' rounds of a group by latency, and the
+    // sort's launches.
+    const int per_sm = std::max(1, std::min(3, (int)(227 * 1024 / (P->smem_floats * 4 + 1024))));
+    std::vector<double> times(p.tensors.size(), n);  // how often every tensor is computed
+    double total = P->key_bits ? 20000.0 * sm_count() : 0;
+    if (top >= 0) {
+        const int t = p.steps[top].c;
+        times[(size_t)t] = P->one_each ? n : distinct(n, q[(size_t)t]);
+        for (int s = top; s >= 0; --s) {
+            const StepPlan &st = p.steps[s];
+            if (!shared[(size_t)st.c]) continue;
+            const int hv = heavy(st.c) ? st.a : st.b, lt = heavy(st.c) ? st.b : st.a;
+            times[(size_t)lt] = times[(size_t)st.c];
+            times[(size_t)hv] = P->key_bits && q[(size_t)hv] <= P->key_bits
+                                    ? std::min(times[(size_t)st.c], distinct(n, q[(size_t)hv]))
+                                    : times[(size_t)st.c];
+        }
+    }
+    for (int i = 0; i < ns; ++i) {
+        const StepPlan &st = p.steps[order[(size_t)i]];
+        const double clk = std::ldexp(1.0, st.mb + st.nb + st.kb) / 64.0;
+        total += times[(size_t)st.c] * (i < n_shared ? clk + 900.0 / per_sm : clk + 40.0);
+    }
+    if (n_shared > 0 && n_shared < ns) {
+        const double groups = times[(size_t)p.steps[top].c];
+        total += groups * std::ceil(n / std::max(1.0, groups) / ST_WARPS) * 1200.0 * (ns - n_shared) / per_sm;
+    }
+    *cost = total;
+    return true;
+}
+
+// The program of a single-state plan for a list of n states: the split into
+// shared and per-warp steps of least estimated cost, else (nothing else
+// fits) every state on a whole CTA with reused leaf areas.
+bool build_program(const Plan &p, int64_t n, SProgram *P, std::string *why) {
     if (!p.free_qubits.empty()) return *why = "free qubits", false;
     if (p.n_slices() != 1) return *why = "sliced", false;
     if (p.m > ST_MAX_LEAVES) return *why = "more than 16 subcircuits", false;
     if (p.net->n_qubits > 64) return *why = "more than 64 qubits", false;
-    P->n_leaves = p.m;
-    P->n_steps = (int)p.steps.size();
-    int q = 0;
-    for (int j = 0; j < p.m; ++j) {
-        const Node &nd = p.net->nodes[j];
-        P->leaf[j].row_log2 = p.tensors[j].nbits();
-        P->leaf[j].q_off = q;
-        P->leaf[j].n_q = (int)nd.out_qubits.size();
-        for (int oq : nd.out_qubits) P->qubits[q++] = (int8_t)oq;
-    }
-    // shared memory: two staging areas for leaf operands, the reduction
-    // buffer, then one region per intermediate
-    int64_t stg[2] = {0, 0}, red = 0;
-    std::vector<int> consumer(p.tensors.size(), -1);
-    for (size_t s = 0; s < p.steps.size(); ++s) {
-        consumer[(size_t)p.steps[s].a] = (int)s;
-        consumer[(size_t)p.steps[s].b] = (int)s;
-    }
-    for (size_t s = 0; s < p.steps.size(); ++s) {
-        const StepPlan &st = p.steps[s];
+    for (auto &st : p.steps) {
         if (st.kblk) return *why = "K-blocked operands", false;
-        SStep &S = P->step[s];
-        S.mb = st.mb;
-        S.nb = st.nb;
-        S.kb = st.kb;
         if (st.mb + st.kb > 20 || st.nb + st.kb > 20 || st.mb + st.nb > 20) return *why = "step too large", false;
-        S.a_src = st.a < p.m ? st.a : -1 - (st.a - p.m);
-        S.b_src = st.b < p.m ? st.b : -1 - (st.b - p.m);
         if (st.maskR >> 32 || st.maskC >> 32) return *why = "result wider than 32 bits", false;
-        S.maskR = (uint32_t)st.maskR;
-        S.maskC = (uint32_t)st.maskC;
-        const int64_t pk = pitch_of(1 << st.kb);
-        if (S.a_src >= 0) stg[0] = std::max(stg[0], ((int64_t)1 << st.mb) * pk);
-        if (S.b_src >= 0) stg[1] = std::max(stg[1], ((int64_t)1 << st.nb) * pk);
-        const int M = 1 << st.mb, N = 1 << st.nb, K = 1 << st.kb;
-        S.tm = std::min(4, M);
-        S.tn = std::min(4, N);
-        const int tiles = (M / S.tm) * (N / S.tn);
-        int ks = 1;
-        while (2 * ks * tiles <= ST_THREADS && K / (2 * ks) >= 4) ks *= 2;
-        S.ksplit = ks;
-        if (ks > 1) red = std::max(red, (int64_t)ks * M * N);
     }
-    int64_t off = align4(stg[0]) + align4(stg[1]);
-    P->red_off = (int32_t)off;
-    off += align4(red);
-    for (size_t s = 0; s < p.steps.size(); ++s) {
-        SStep &S = P->step[s];
-        const int c = consumer[(size_t)p.steps[s].c];
-        if (c < 0) {  // the final step: a scalar per state
-            if (S.mb != 0 || S.nb != 0) return *why = "final step is not a scalar", false;
-            S.c_kb = -1;
-            S.c_off = 0;
-            continue;
+    const int ns = (int)p.steps.size();
+    double best = std::numeric_limits<double>::infinity();
+    std::string w;
+    for (int top = -1; top < ns; ++top) {
+        SProgram Q;
+        double cost = 0;
+        if (n > (int64_t)1 << 31 && top >= 0) break;  // positions of the sorted list are 32-bit
+        if (layout_program(p, (double)n, top, false, &Q, &cost, &w) && cost < best) {
+            best = cost;
+            *P = Q;
         }
-        S.c_kb = p.steps[(size_t)c].kb;
-        S.c_off = (int32_t)off;
-        const int64_t ck = (int64_t)1 << S.c_kb;
-        off += align4((((int64_t)1 << (S.mb + S.nb)) / ck) * pitch_of((int)ck));
     }
-    for (size_t s = 0; s < p.steps.size(); ++s) {
-        SStep &S = P->step[s];
-        S.a_off = S.a_src >= 0 ? 0 : P->step[-1 - S.a_src].c_off;
-        S.b_off = S.b_src >= 0 ? (int32_t)align4(stg[0]) : P->step[-1 - S.b_src].c_off;
-        S.tab_off = (int32_t)off;  // offset tables of the epilogue (ints)
-        off += align4(((int64_t)1 << S.mb) + ((int64_t)1 << S.nb));
-    }
-    if (off > ST_MAX_SMEM_FLOATS) return *why = "intermediates exceed shared memory", false;
-    P->smem_floats = (int32_t)std::max<int64_t>(off, 4);
+    if (std::isfinite(best)) return true;
+    if (!layout_program(p, (double)n, ns - 1, true, P, nullptr, why)) return false;
+    P->key_bits = 0;  // leaves are staged for every state: nothing to sort for
     return true;
 }
 
@@ -305,7 +664,7 @@ tqc_status cuda_fail(cudaError_t e, const char *what) {
 int states_fused_floats(const Plan &p) {
     SProgram P;
     std::string why;
-    return build_program(p, &P, &why) ? P.smem_floats : -1;
+    return build_program(p, 1, &P, &why) ? P.smem_floats : -1;
 }
 
 tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void *d_out, int out_dtype,
@@ -316,7 +675,9 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
     if (p->net->n_qubits > 64) return fail(TQC_ERR_UNSUPPORTED, "state lists support up to 64 qubits");
     if (n < 0) return fail(TQC_ERR_INVALID, "negative state count");
     const uint64_t qmask = p->net->n_qubits == 64 ? ~0ull : ((1ull << p->net->n_qubits) - 1);
-    for (int64_t i = 0; i < n; ++i)
+    uint64_t any = 0;
+    for (int64_t i = 0; i < n; ++i) any |= states[i];
+    for (int64_t i = 0; (any & ~qmask) && i < n; ++i)
         if (states[i] & ~qmask) return fail(TQC_ERR_INVALID, "state " + std::to_string(i) + " has bits beyond n_qubits");
     tqc_status st = exec_prepare(p);
     if (st != TQC_OK) return st;
@@ -333,7 +694,7 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
     }
     SProgram P;
     std::string why;
-    const bool fused = build_program(*p, &P, &why);
+    const bool fused = build_program(*p, n, &P, &why);
     const int esize = out_dtype == TQC_F64 ? 8 : 4;
     if (fused && n > 0) {
         // per-node tables Tt_j[x][cuts], rebuilt when the tensors changed
@@ -377,18 +738,44 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
             p->tab_version = p->net->version;
         }
         for (int j = 0; j < p->m; ++j) P.leaf[j].table = (const float *)((char *)p->d_tab + p->tab_off[(size_t)j]);
-        if (n * 8 > p->states_bytes) {
+        // the list, and for the sort: permuted states, ranks, sorted states,
+        // their places in the list, counters and their block sums
+        const int64_t n8 = align4(n) * 8, n4 = align4(n) * 4, n_keys = P.key_bits ? (int64_t)1 << P.key_bits : 0;
+        const int64_t n_sums = (n_keys + SCAN_PER_CTA - 1) / SCAN_PER_CTA;
+        const int64_t need = n8 + (P.key_bits ? 2 * n8 + 2 * n4 + align4(n_keys) * 4 + align4(n_sums) * 4 : 0);
+        if (need > p->states_bytes) {
             if (p->d_states) cudaFree(p->d_states);
             p->d_states = nullptr;
             p->states_bytes = 0;
-            if (cudaMalloc(&p->d_states, (size_t)n * 8) != cudaSuccess) {
+            if (cudaMalloc(&p->d_states, (size_t)need) != cudaSuccess) {
                 cudaGetLastError();
                 return fail(TQC_ERR_OOM, "state list of " + std::to_string(n) + " states");
             }
-            p->states_bytes = n * 8;
+            p->states_bytes = need;
         }
-        cudaError_t e = cudaMemcpyAsync(p->d_states, states, (size_t)n * 8, cudaMemcpyHostToDevice, s);
+        uint64_t *d_list = (uint64_t *)p->d_states;
+        uint32_t *d_place = nullptr;
+        cudaError_t e = cudaMemcpyAsync(d_list, states, (size_t)n * 8, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return cuda_fail(e, "state list upload");
+        if (P.key_bits) {
+            char *at = (char *)p->d_states + n8;
+            auto take = [&](int64_t bytes) { char *r = at; at += bytes; return r; };
+            uint64_t *ys = (uint64_t *)take(n8), *sorted = (uint64_t *)take(n8);
+            uint32_t *rank = (uint32_t *)take(n4);
+            d_place = (uint32_t *)take(n4);
+            uint32_t *counters = (uint32_t *)take(align4(n_keys) * 4), *sums = (uint32_t *)take(align4(n_sums) * 4);
+            e = cudaMemsetAsync(counters, 0, (size_t)n_keys * 4, s);
+            if (e != cudaSuccess) return cuda_fail(e, "state list sort");
+            const unsigned blocks = (unsigned)((n + ST_THREADS - 1) / ST_THREADS);
+            states_count_kernel<<<blocks, ST_THREADS, 0, s>>>(P, d_list, n, ys, rank, counters);
+            states_sums_kernel<<<(unsigned)n_sums, ST_THREADS, 0, s>>>(counters, (int)n_keys, sums);
+            states_scan_kernel<<<(unsigned)n_sums, ST_THREADS, 0, s>>>(counters, (int)n_keys, sums);
+            states_scatter_kernel<<<blocks, ST_THREADS, 0, s>>>(ys, rank, n, P.n_qubits - P.key_bits, counters, sorted,
+                                                                d_place);
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return cuda_fail(e, "state list sort");
+            d_list = sorted;
+        }
         const size_t smem = (size_t)P.smem_floats * 4;
         static size_t attr = 0;
         if (smem > 48 * 1024 && smem > attr) {
@@ -400,8 +787,8 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, states_kernel, ST_THREADS, smem);
         if (e != cudaSuccess || per_sm < 1) return fail(TQC_ERR_UNSUPPORTED, "state-list kernel does not fit an SM");
         const int64_t grid = std::min<int64_t>(n, (int64_t)per_sm * sm_count());
-        states_kernel<<<(unsigned)grid, ST_THREADS, smem, s>>>(P, (const uint64_t *)p->d_states, n, d_out,
-                                                              out_dtype == TQC_F64, p->d_zinfo);
+        states_kernel<<<(unsigned)grid, ST_THREADS, smem, s>>>(P, d_list, d_place, n, d_out, out_dtype == TQC_F64,
+                                                              p->d_zinfo);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "state-list kernel");
     } else if (n > 0) {

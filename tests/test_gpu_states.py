@@ -188,3 +188,31 @@ def test_rejections():
     assert ei.value.status == tqc.ERR_INVALID
     p.close()
     h.close()
+
+
+# Three subcircuits joined pairwise by 3, 2 and 1 cuts (the first pair's step,
+# 64 x .. x 64, is worth sharing between states), a chain of four (every step
+# small), and a ring whose last subcircuit has no outputs.
+SPLITS = {
+    "triangle": (14, [(0, 1)] * 3 + [(1, 2)] * 2 + [(0, 2)], [[0, 5, 9], [1, 4, 8, 11], [2, 3, 6, 7, 10, 12, 13]]),
+    "chain": (13, [(0, 1), (1, 2), (2, 3)], [[3, 7, 8], [0, 1, 12], [2, 5, 6, 11], [4, 9, 10]]),
+    "ring": (12, [(0, 1), (1, 2), (2, 3), (0, 3), (0, 2)], [[0, 3, 6, 9], [1, 4, 7, 10], [2, 5, 8, 11], []]),
+}
+
+
+@pytest.mark.parametrize("name", list(SPLITS))
+@pytest.mark.parametrize("count", [1, 31, 257, 5000, 70001])
+def test_list_lengths_and_orders(name, count):
+    """Lists from one state to more than the states there are: random,
+    descending, and one state repeated, each state against the whole
+    distribution by the FP64 oracle."""
+    n, edges, outs = SPLITS[name]
+    net = tensors.pseudo_physical_network(n, edges, outs, 4000 + count)
+    want = oracle.recon_bin(net) / oracle.total_mass(net)
+    h = tqc.Network(net)
+    for st in (states_of(n, count, count), np.sort(states_of(n, count, 1 + count))[::-1].copy(),
+               np.full(count, (1 << n) - 2, np.uint64)):
+        got, z, d = run_states(h, st)
+        assert d["states_form"] == "fused"
+        check_fp32(got, want[st.astype(np.int64)])
+    h.close()

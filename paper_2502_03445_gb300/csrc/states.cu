@@ -23,13 +23,14 @@
 // equal inputs: the result of a step depends only on the output bits of its
 // own subcircuits, which many states of a list share (2^17 values for the
 // costliest step of the 30-qubit grid, 10^6 states).  A shared subtree is
-// chosen (choose_split, below), the list is sorted by that subtree's bits (a
+// chosen (build_program, below), the list is sorted by that subtree's bits (a
 // counting sort), and a CTA walks a contiguous range of the sorted list: the
 // shared steps run on all 256 threads when a bit they depend on has changed,
 // and every state's remaining steps run on one warp, eight states at a time,
 // with no barrier between them.  A K range too long for its outputs is split
 // over neighbouring lanes and summed with shuffles.  10^6 states of the
-// 30-qubit grid: STATES_FIGURES
+// 30-qubit grid: 45.1 -> 4.7 ms (the kernel 4.5 ms: 2.1 in the shared steps,
+// 2.1 in the warps'; the sort 0.07 ms).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -48,6 +49,7 @@ namespace {
 
 constexpr int ST_THREADS = 256;
 constexpr int ST_WARPS = ST_THREADS / 32;
+constexpr int ST_WINDOW = 3 * ST_THREADS;  // a group (up to ST_THREADS states), the next one, and some
 constexpr int ST_MAX_LEAVES = 16;
 constexpr int ST_MAX_STEPS = ST_MAX_LEAVES - 1;
 constexpr int ST_MAX_SMEM_FLOATS = 200 * 1024 / 4;
@@ -61,8 +63,8 @@ struct SLeaf {
 };
 
 // Where a step's operand is: a leaf's table row in global memory, the CTA's
-// shared memory (a staged leaf, or the result of a shared step), or the
-// warp's own part of it.
+// shared memory (a staged leaf, or the
+// result of a shared step), or the warp's own part of it.
 enum SrcKind { SRC_TABLE = 0, SRC_CTA = 1, SRC_WARP = 2 };
 
 struct SStep {
@@ -72,7 +74,7 @@ struct SStep {
     int32_t a_off, b_off;   // offsets (floats) of SRC_CTA / SRC_WARP operands
     int32_t mb, nb, kb;     // log2 of M, N, K
     uint32_t maskR, maskC;  // result-layout bits of the row / column index bits
-    int32_t c_kb;           // log2 K of the step consuming the result; -1 for the final step
+    int32_t c_kb, c_lkl;    // log2 K and lkl of the step consuming the result; c_kb -1 for the final step
     int32_t c_off;          // the result's place: rows of 2^c_kb, padded
     int32_t lkl;            // log2 of the lanes sharing one output tile's K range
     int32_t tab_off;        // result offsets of rows (M) then columns (N), in shared memory
@@ -92,19 +94,56 @@ struct SProgram {
     int32_t smem_floats;
 };
 
-// Row pitch of a [rows][K] operand in shared memory: K + 4 floats keeps
-// float4 access and spreads rows over the banks.
-__host__ __device__ __forceinline__ int pitch_of(int k) { return k >= 4 ? k + 4 : k; }
+// Row pitch of a [rows][K] operand in shared memory whose K is read by 2^lkl
+// neighbouring lanes, 16 bytes each: K + 4 * 2^lkl floats puts the eight lanes
+// of a 16-byte access phase (2^lkl pieces of 8 / 2^lkl rows) on distinct banks.
+__host__ __device__ __forceinline__ int pitch_of(int k, int lkl) { return k >= 4 ? k + (lkl < 3 ? 4 << lkl : 4) : k; }
+
+// Two FP32 multiply-adds per instruction (even and odd k in the two halves).
+__device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float lo32(uint64_t c) { return __uint_as_float((uint32_t)c); }
+__device__ __forceinline__ float hi32(uint64_t c) { return __uint_as_float((uint32_t)(c >> 32)); }
+
+// log2 of the register tile along a dimension of 2^b results.
+__host__ __device__ __forceinline__ int tile_log2(int b) { return b >= 2 ? 2 : 0; }
+
+// Store the LEFT = TM TN >> lkl results (at least one) of a tile that are
+// left in this lane, e0 on, at rows rt + i rs and columns ct + j cs.
+template <int TM, int TN, int LEFT>
+__device__ __forceinline__ void put_left(const float *acc, int lkl, int e0, int rt, int ct, int rs, int cs, float *res,
+                                         const int *tab_r, const int *tab_c) {
+    if constexpr (LEFT > 1) {
+        if ((TM * TN >> lkl) < LEFT) return put_left<TM, TN, LEFT / 2>(acc, lkl, e0, rt, ct, rs, cs, res, tab_r, tab_c);
+    }
+    constexpr int LC = LEFT < TN ? LEFT : TN;  // columns of one row
+    const int r = rt + (e0 / TN) * rs, c = ct + (e0 % TN) * cs;
+    int oc[LC];
+#pragma unroll
+    for (int j = 0; j < LC; ++j) oc[j] = tab_c[c + j * cs];
+#pragma unroll
+    for (int i = 0; i < LEFT / LC; ++i) {
+        float *o = res + tab_r[r + i * rs];
+#pragma unroll
+        for (int j = 0; j < LC; ++j) o[oc[j]] = acc[i * LC + j];
+    }
+}
 
 // Output tiles of TM x TN results (rows strided by M / TM, columns by
 // N / TN), tile t of every nw x (32 >> lkl): 2^lkl neighbouring lanes share a
-// tile, lane ks taking the float4s ks, ks + 2^lkl, ... of K (consecutive
-// 16-byte pieces of a row: whole sectors, no bank conflicts).  Their partial
-// sums are added by recursive halving, which leaves every lane a part of the
-// tile's results to store (put).  AG / BG: the operand is in global memory.
-template <int TM, int TN, bool AG, bool BG, typename Put>
+// tile, lane ks taking the 16-byte pieces ks, ks + 2^lkl, ... of K (whole
+// sectors of a row, no bank conflicts).  Their partial sums are added by
+// recursive halving, which leaves every lane a part of the tile's results to
+// store, (r, c) at res[tab[r] + tab[M + c]].  AG / BG: the operand is in
+// global memory.  4 x 4 tiles move 8 16-byte pieces for 64 multiply-adds, and
+// shared memory delivers 128 bytes a clock, which bounds a CTA's step at half
+// the FP32 rate; 8 x 4 and 8 x 8 tiles move less but measured slower (10^6
+// grid30 states 5.5 and 5.8 against 5.0 ms: two CTAs per SM, not three, and
+// longer reductions).
+template <int TM, int TN, bool AG, bool BG>
 __device__ __forceinline__ void step_tiles(const float *A, int pa, const float *B, int pb, int mb, int nb, int kb,
-                                           int lkl, int w, int nw, int lane, const Put &put) {
+                                           int lkl, int w, int nw, int lane, float *res, const int *tab) {
     if constexpr (!AG) __builtin_assume(__isShared(A));
     if constexpr (!BG) __builtin_assume(__isShared(B));
     constexpr int E = TM * TN;
@@ -118,31 +157,33 @@ __device__ __forceinline__ void step_tiles(const float *A, int pa, const float *
         const int t = valid ? t0 : 0;
         const int rt = t >> lc, ct = t & (cs - 1);
         float acc[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) acc[e] = 0.f;
         if (kb >= 2) {
             const float *pA = A + rt * pa + 4 * ks, *pB = B + ct * pb + 4 * ks;
             const int sa = rs * pa, sb = cs * pb, n4 = 1 << (kb - 2 - lkl), inc = 4 << lkl;
-#pragma unroll 2
+            uint64_t acc2[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) acc2[e] = 0;
+#pragma unroll 1
             for (int k = 0; k < n4; ++k) {
-                float4 a[TM], b[TN];
+                ulonglong2 b[TN];
 #pragma unroll
-                for (int i = 0; i < TM; ++i) a[i] = AG ? __ldg((const float4 *)(pA + i * sa)) : *(const float4 *)(pA + i * sa);
+                for (int j = 0; j < TN; ++j)
+                    b[j] = BG ? __ldg((const ulonglong2 *)(pB + j * sb)) : *(const ulonglong2 *)(pB + j * sb);
 #pragma unroll
-                for (int j = 0; j < TN; ++j) b[j] = BG ? __ldg((const float4 *)(pB + j * sb)) : *(const float4 *)(pB + j * sb);
-                pA += inc;
-                pB += inc;
-#pragma unroll
-                for (int i = 0; i < TM; ++i)
+                for (int i = 0; i < TM; ++i) {
+                    const ulonglong2 a =
+                        AG ? __ldg((const ulonglong2 *)(pA + i * sa)) : *(const ulonglong2 *)(pA + i * sa);
 #pragma unroll
                     for (int j = 0; j < TN; ++j) {
-                        float &c = acc[i * TN + j];
-                        c = fmaf(a[i].x, b[j].x, c);
-                        c = fmaf(a[i].y, b[j].y, c);
-                        c = fmaf(a[i].z, b[j].z, c);
-                        c = fmaf(a[i].w, b[j].w, c);
+                        fma2(acc2[i * TN + j], a.x, b[j].x);
+                        fma2(acc2[i * TN + j], a.y, b[j].y);
                     }
+                }
+                pA += inc;
+                pB += inc;
             }
+#pragma unroll
+            for (int e = 0; e < E; ++e) acc[e] = lo32(acc2[e]) + hi32(acc2[e]);
         } else {  // K = 1
 #pragma unroll
             for (int i = 0; i < TM; ++i)
@@ -172,31 +213,67 @@ __device__ __forceinline__ void step_tiles(const float *A, int pa, const float *
                 }
             }
         }
-        const int left = E >> lkl > 0 ? E >> lkl : 1;
-        if (mine) {
-#pragma unroll
-            for (int i = 0; i < E; ++i)
-                if (i < left) {
-                    const int e = e0 + i;
-                    put(rt + (e / TN) * rs, ct + (e % TN) * cs, acc[i]);
-                }
-        }
+        if (mine) put_left<TM, TN, E>(acc, lkl, e0, rt, ct, rs, cs, res, tab, tab + (1 << mb));
     }
 }
 
-template <bool AG, bool BG, typename Put>
-__device__ __forceinline__ void step_run(const SStep &S, const float *A, int pa, const float *B, int pb, int w, int nw,
-                                         int lane, const Put &put) {
-    if (S.mb >= 2 && S.nb >= 2) step_tiles<4, 4, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, put);
-    else if (S.mb >= 2) step_tiles<4, 1, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, put);
-    else if (S.nb >= 2) step_tiles<1, 4, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, put);
-    else step_tiles<1, 1, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, put);
+template <bool AG, bool BG>
+__device__ __forceinline__ void step_run(const SStep &S, const float *A, const float *B, int w, int nw, int lane,
+                                         float *res, const int *tab) {
+    __builtin_assume(__isShared(res));
+    __builtin_assume(__isShared(tab));
+    const int K = 1 << S.kb, pk = pitch_of(K, S.lkl), pa = AG ? K : pk, pb = BG ? K : pk;
+    if (S.mb >= 2 && S.nb >= 2) step_tiles<4, 4, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, res, tab);
+    else if (S.mb >= 2) step_tiles<4, 1, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, res, tab);
+    else if (S.nb >= 2) step_tiles<1, 4, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, res, tab);
+    else step_tiles<1, 1, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, res, tab);
+}
+
+// Copy a leaf operand (2^row_log2 floats, rows of 2^kb, from one table row)
+// to padded rows in shared memory with 16-byte asynchronous copies (by
+// threads i of n; the caller waits).
+__device__ __forceinline__ void copy_rows(const float *row, int row_log2, int kb, int lkl, float *dst, int i,
+                                          int n) {
+    if (row_log2 < 2) {  // a subcircuit without cuts: one value
+        if (i == 0) dst[0] = __ldg(row);
+        return;
+    }
+    const int lq = kb >= 2 ? kb - 2 : 30, skip = pitch_of(1 << kb, lkl) - (1 << kb);  // pieces per row (K = 1: contiguous)
+    for (; i < 1 << (row_log2 - 2); i += n)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(dst + 4 * i + skip * (i >> lq))),
+                     "l"(row + 4 * i)
+                     : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The final step's partial sum over pieces i, i + n, ... of K (16 bytes
+// each; K = 1: one element), added over the warp.
+__device__ __forceinline__ float final_dot(const float *A, const float *B, int kb, int i, int n) {
+    float v = 0.f;
+    if (kb >= 2) {
+        for (int k = i; k < 1 << (kb - 2); k += n) {
+            const float4 a = ((const float4 *)A)[k], b = ((const float4 *)B)[k];
+            v = fmaf(a.x, b.x, v);
+            v = fmaf(a.y, b.y, v);
+            v = fmaf(a.z, b.z, v);
+            v = fmaf(a.w, b.w, v);
+        }
+    } else if (i == 0) {
+        v = A[0] * B[0];
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 __global__ void __launch_bounds__(ST_THREADS, 3)
     states_kernel(const __grid_constant__ SProgram P, const uint64_t *__restrict__ list,
                   const uint32_t *__restrict__ place, int64_t n, void *out, int out_f64, const double *zinfo) {
     extern __shared__ __align__(16) float sm[];
+    __shared__ float part[ST_WARPS];
+    __shared__ uint64_t win_y[ST_WINDOW];
+    __shared__ uint32_t win_place[ST_WINDOW];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const double scale = zinfo[1];
     // Every state runs the same program: the place of result row r and column
@@ -207,7 +284,7 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
         const SStep &S = P.step[si];
         const int M = 1 << S.mb, N = 1 << S.nb;
         int *tab = (int *)(sm + S.tab_off);
-        const int ck = S.c_kb < 0 ? 1 : 1 << S.c_kb, pc = pitch_of(ck);
+        const int ck = S.c_kb < 0 ? 1 : 1 << S.c_kb, pc = pitch_of(ck, S.c_lkl);
         for (int i = tid; i < M + N; i += ST_THREADS) {
             const uint32_t d = i < M ? pdep32((uint32_t)i, S.maskR) : pdep32((uint32_t)(i - M), S.maskC);
             tab[i] = S.c_kb < 0 ? 0 : (int)(d >> S.c_kb) * pc + (int)(d & (uint32_t)(ck - 1));
@@ -232,26 +309,27 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
             __ballot_sync(0xffffffffu, lane + 32 < P.n_qubits && ((x >> P.perm[(lane + 32) & 63]) & 1ull));
         return ((uint64_t)hi << 32) | lo;
     };
-    // steps [s0, n_steps) of one state on one warp
+    // steps [n_shared, n_steps) of one state on one warp, leaf rows read from
+    // the tables (staged copies per warp cost a CTA per SM and measured no faster)
     float *wsm = sm + P.warp_off + warp * P.warp_floats;
     auto warp_state = [&](uint64_t y, int64_t at) {
         for (int si = P.n_shared; si < P.n_steps; ++si) {
             const SStep &S = P.step[si];
-            const int M = 1 << S.mb, K = 1 << S.kb, pk = pitch_of(K);
-            const float *A = S.a_kind == SRC_TABLE ? row_of(S.a_leaf, y) : (S.a_kind == SRC_CTA ? sm : wsm) + S.a_off;
-            const float *B = S.b_kind == SRC_TABLE ? row_of(S.b_leaf, y) : (S.b_kind == SRC_CTA ? sm : wsm) + S.b_off;
+            const bool ag = S.a_kind == SRC_TABLE, bg = S.b_kind == SRC_TABLE;
+            const float *A = ag ? row_of(S.a_leaf, y) : (S.a_kind == SRC_CTA ? sm : wsm) + S.a_off;
+            const float *B = bg ? row_of(S.b_leaf, y) : (S.b_kind == SRC_CTA ? sm : wsm) + S.b_off;
+            if (S.c_kb < 0) {
+                const float v = final_dot(A, B, S.kb, lane, 32);
+                if (lane == 0) store(at, v);
+                __syncwarp();
+                return;
+            }
             const int *tab = (const int *)(sm + S.tab_off);
             float *res = wsm + S.c_off;
-            const bool last = S.c_kb < 0;
-            auto put = [&](int r, int c, float v) {
-                if (last) store(at, v);
-                else res[tab[r] + tab[M + c]] = v;
-            };
-            const bool ag = S.a_kind == SRC_TABLE, bg = S.b_kind == SRC_TABLE;
-            if (ag && bg) step_run<true, true>(S, A, K, B, K, 0, 1, lane, put);
-            else if (ag) step_run<true, false>(S, A, K, B, pk, 0, 1, lane, put);
-            else if (bg) step_run<false, true>(S, A, pk, B, K, 0, 1, lane, put);
-            else step_run<false, false>(S, A, pk, B, pk, 0, 1, lane, put);
+            if (ag && bg) step_run<true, true>(S, A, B, 0, 1, lane, res, tab);
+            else if (ag) step_run<true, false>(S, A, B, 0, 1, lane, res, tab);
+            else if (bg) step_run<false, true>(S, A, B, 0, 1, lane, res, tab);
+            else step_run<false, false>(S, A, B, 0, 1, lane, res, tab);
             __syncwarp();
         }
     };
@@ -263,69 +341,119 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
         return;
     }
     const int64_t p0 = n * blockIdx.x / gridDim.x, p1 = n * (blockIdx.x + 1) / gridDim.x;
+    auto place_of = [&](int64_t p) { return place ? (int64_t)place[p] : p; };
     if (P.n_shared == 0) {
         for (int64_t p = p0 + warp; p < p1; p += ST_WARPS) {
             const uint64_t y = state_at(p);
-            warp_state(y, place ? (int64_t)place[p] : p);
+            warp_state(y, place_of(p));
         }
         return;
     }
-    uint64_t prev = 0;
-    int cnt = 0;
-    for (int64_t p = p0; p < p1; p += cnt) {
-        const uint64_t y = state_at(p);
-        // the states that share this one's subtree bits are consecutive: count
-        // them (up to one per thread).  The barrier also ends the reads of the
-        // previous round.
-        if (P.one_each) {
-            __syncthreads();
-            cnt = 1;
-        } else {
-            const int64_t q = p + tid;
-            cnt = __syncthreads_count(q < p1 && ((list[q < p1 ? q : p] ^ y) & P.group_mask) == 0);
-        }
-        const bool first = p == p0;
-        const uint64_t diff = y ^ prev;
-        prev = y;
-        for (int si = 0; si < P.n_shared; ++si) {
+    // Stage the leaf operands of the shared steps that changed since the last
+    // staging (diff: the bits of y that did).
+    auto stage = [&](int s0, int s1, uint64_t y, uint64_t diff, bool all) {
+        for (int si = s0; si < s1; ++si) {
             const SStep &S = P.step[si];
-            const bool last = S.c_kb < 0;
-            if (!first && !last && !(diff & S.mask)) continue;  // nothing it depends on has changed
-            const int M = 1 << S.mb, N = 1 << S.nb, K = 1 << S.kb, pk = pitch_of(K);
-            // stage changed leaf operands (rows x K, row-major in the table) as padded rows
 #pragma unroll
             for (int op = 0; op < 2; ++op) {
                 const int leaf = op ? S.b_leaf : S.a_leaf;
                 if (leaf < 0) continue;
                 const uint64_t lm = ((1ull << P.leaf[leaf].n_q) - 1ull) << P.leaf[leaf].y_off;
-                if (!first && !P.restage && !(diff & lm)) continue;
-                const int rows = op ? N : M;
-                const float *row = row_of(leaf, y);
-                float *dst = sm + (op ? S.b_off : S.a_off);
-                if (K >= 4) {
-                    const int lq = S.kb - 2;  // float4s per row: K / 4
-                    for (int i = tid; i < rows << lq; i += ST_THREADS) {
-                        const int r = i >> lq, k4 = i & ((1 << lq) - 1);
-                        *(float4 *)(dst + r * pk + 4 * k4) = __ldg((const float4 *)row + i);
-                    }
-                } else {
-                    for (int i = tid; i < rows; i += ST_THREADS) dst[i] = __ldg(row + i);
-                }
+                if (!all && !(diff & lm)) continue;
+                copy_rows(row_of(leaf, y), P.leaf[leaf].row_log2, S.kb, S.lkl, sm + (op ? S.b_off : S.a_off),
+                          tid, ST_THREADS);
             }
+        }
+    };
+    // One shared step on the whole CTA (not the final one).
+    auto shared_step = [&](const SStep &S) {
+        step_run<false, false>(S, sm + S.a_off, sm + S.b_off, warp, ST_WARPS, lane, sm + S.c_off,
+                               (const int *)(sm + S.tab_off));
+    };
+    if (P.one_each) {  // every step on the whole CTA, one state at a time
+        uint64_t prev = 0;
+        for (int64_t p = p0; p < p1; ++p) {
+            const uint64_t y = state_at(p), diff = y ^ prev;
+            const bool first = p == p0;
+            prev = y;
+            for (int si = 0; si < P.n_shared; ++si) {
+                const SStep &S = P.step[si];
+                // skipped when nothing it depends on has changed
+                if (!first && S.c_kb >= 0 && !(diff & S.mask)) continue;
+                stage(si, si + 1, y, diff, first || P.restage);
+                copies_wait();
+                __syncthreads();
+                if (S.c_kb >= 0) {
+                    shared_step(S);
+                } else {
+                    const float v = final_dot(sm + S.a_off, sm + S.b_off, S.kb, tid, ST_THREADS);
+                    if (lane == 0) part[warp] = v;
+                    __syncthreads();
+                    float sum = 0.f;
+                    for (int w = 0; w < ST_WARPS; ++w) sum += part[w];
+                    if (tid == 0) store(place_of(p), sum);
+                }
+                __syncthreads();
+            }
+        }
+        return;
+    }
+    // Groups of states that share the subtree's bits (consecutive in the
+    // sorted list).  While the warps run the states of one group, the leaf
+    // operands of the next group's shared steps are on their way: a group
+    // takes two barriers, and one between shared steps.
+    auto run_shared = [&](uint64_t diff, bool all) {
+        for (int si = 0; si < P.n_shared; ++si) {
+            const SStep &S = P.step[si];
+            if (!all && !(diff & S.mask)) continue;
+            shared_step(S);
+            if (si + 1 < P.n_shared) __syncthreads();
+        }
+    };
+    // A window of the sorted list in shared memory: [wb, wb + ST_WINDOW).
+    int64_t wb = p0;
+    auto load_window = [&](int64_t at) {
+        wb = at;
+        for (int i = tid; i < ST_WINDOW; i += ST_THREADS)
+            if (at + i < p1) {
+                win_y[i] = list[at + i];
+                win_place[i] = place[at + i];
+            }
+    };
+    auto group_size = [&](int64_t p, uint64_t y) {  // up to one state per thread; a barrier
+        const int64_t q = p + tid;
+        return __syncthreads_count(q < p1 && ((win_y[q < p1 ? q - wb : 0] ^ y) & P.group_mask) == 0);
+    };
+    if (p0 >= p1) return;
+    int64_t p = p0;
+    load_window(p0);
+    __syncthreads();
+    uint64_t y = win_y[0];
+    stage(0, P.n_shared, y, 0, true);
+    int cnt = group_size(p0, y);
+    copies_wait();
+    __syncthreads();
+    run_shared(0, true);
+    while (true) {
+        const int64_t pn = p + cnt;
+        if (pn < p1 && pn + ST_THREADS > wb + ST_WINDOW && wb + ST_WINDOW < p1) {
+            // the window moves on; the states of this group keep their part of it
             __syncthreads();
-            const int *tab = (const int *)(sm + S.tab_off);
-            float *res = sm + S.c_off;
-            const int64_t at = last ? (place ? (int64_t)place[p] : p) : 0;
-            step_run<false, false>(S, sm + S.a_off, pk, sm + S.b_off, pk, warp, ST_WARPS, lane,
-                                   [&](int r, int c, float v) {
-                                       if (last) store(at, v);
-                                       else res[tab[r] + tab[M + c]] = v;
-                                   });
+            load_window(p);
             __syncthreads();
         }
-        if (P.n_shared < P.n_steps)
-            for (int k = warp; k < cnt; k += ST_WARPS)
-                warp_state(list[p + k], place ? (int64_t)place[p + k] : p + k);
+        const uint64_t yn = pn < p1 ? win_y[pn - wb] : y, diff = yn ^ y;
+        const int next = group_size(pn, yn);  // the barrier ends the shared steps' writes
+        if (next > 0) stage(0, P.n_shared, yn, diff, false);
+        for (int k = warp; k < cnt; k += ST_WARPS) warp_state(win_y[p + k - wb], (int64_t)win_place[p + k - wb]);
+        if (next == 0) break;
+        p = pn;
+        cnt = next;
+        y = yn;
+        if (!(diff & P.group_mask)) continue;  // a group longer than the CTA's threads goes on
+        copies_wait();
+        __syncthreads();
+        run_shared(diff, false);
     }
 }
 
@@ -514,15 +642,26 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
     P->restage = compact;
     P->group_mask = top >= 0 ? bits_of(p.tensors[(size_t)p.steps[top].c].leaves) : 0;
     if (P->one_each && top != ns - 1) return *why = "shared subtree has too many output bits", false;
+    const int n_shared = (int)std::count_if(order.begin(), order.end(), [&](int s) { return shared[(size_t)p.steps[s].c] != 0; });
+    P->n_shared = n_shared;
+    // lanes per output tile: what the tiles leave idle, at most one per 16
+    // bytes of K; rows read from global memory always 8 (a whole line)
+    std::vector<int> lkl_of((size_t)ns, 0);
+    for (int i = 0; i < ns; ++i) {
+        const StepPlan &st = p.steps[order[(size_t)i]];
+        const bool cta = i < n_shared;
+        const int tiles = st.mb + st.nb - tile_log2(st.mb) - tile_log2(st.nb);  // log2
+        int lkl = std::max(0, std::min(5, (cta ? 8 : 5) - tiles));
+        if (!cta && (st.a < p.m || st.b < p.m)) lkl = std::max(lkl, 3);
+        lkl_of[(size_t)order[(size_t)i]] = std::max(0, std::min(lkl, st.kb - 2));
+    }
     // shared memory: leaf operands of the shared steps, intermediates, the
     // warps' own intermediates, the offset tables
     int64_t off = 0, woff = 0, area[2] = {0, 0};
     std::vector<int> place(p.tensors.size(), 0);
-    const int n_shared = (int)std::count_if(order.begin(), order.end(), [&](int s) { return shared[(size_t)p.steps[s].c] != 0; });
-    P->n_shared = n_shared;
     for (int i = 0; i < n_shared; ++i) {
         const StepPlan &st = p.steps[order[(size_t)i]];
-        const int64_t pk = pitch_of(1 << st.kb);
+        const int64_t pk = pitch_of(1 << st.kb, lkl_of[(size_t)order[(size_t)i]]);
         const int64_t need[2] = {((int64_t)1 << st.mb) * pk, ((int64_t)1 << st.nb) * pk};
         const int t[2] = {st.a, st.b};
         for (int k = 0; k < 2; ++k) {
@@ -550,7 +689,7 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
             continue;
         }
         const int64_t ck = (int64_t)1 << p.steps[c].kb;
-        const int64_t need = align4((((int64_t)1 << (st.mb + st.nb)) / ck) * pitch_of((int)ck));
+        const int64_t need = align4((((int64_t)1 << (st.mb + st.nb)) / ck) * pitch_of((int)ck, lkl_of[(size_t)c]));
         int64_t &o = i < n_shared ? off : woff;
         place[(size_t)st.c] = (int)o;
         o += need;
@@ -565,7 +704,9 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
         S.maskC = (uint32_t)st.maskC;
         S.mask = bits_of(p.tensors[(size_t)st.c].leaves);
         const int c = consumer[(size_t)st.c];
+        S.lkl = lkl_of[(size_t)order[(size_t)i]];
         S.c_kb = c < 0 ? -1 : p.steps[c].kb;
+        S.c_lkl = c < 0 ? 0 : lkl_of[(size_t)c];
         S.c_off = place[(size_t)st.c];
         auto operand = [&](int t, int32_t *leaf, int32_t *kind, int32_t *o) {
             *leaf = t < p.m ? t : -1;
@@ -576,13 +717,6 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
         operand(st.b, &S.b_leaf, &S.b_kind, &S.b_off);
         S.tab_off = (int32_t)off;
         off += align4(((int64_t)1 << st.mb) + ((int64_t)1 << st.nb));
-        // lanes per output tile: what the tiles leave idle, at most one per
-        // float4 of K; rows read from global memory always 8 (a whole line)
-        const int tiles = st.mb + st.nb - (st.mb >= 2 ? 2 : 0) - (st.nb >= 2 ? 2 : 0);  // log2
-        const int lanes = i < n_shared ? 8 : 5;
-        int lkl = std::max(0, std::min(5, lanes - tiles));
-        if (S.a_kind == SRC_TABLE || S.b_kind == SRC_TABLE) lkl = std::max(lkl, 3);
-        S.lkl = std::max(0, std::min(lkl, st.kb - 2));
     }
     P->warp_off = (int32_t)off;
     P->warp_floats = (int32_t)woff;
@@ -594,7 +728,7 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
     // multiply-adds per clock) plus its barriers, a warp's step likewise plus
     // its fixed instructions, the warps' rounds of a group by latency, and the
     // sort's launches.
-    const int per_sm = std::max(1, std::min(3, (int)(227 * 1024 / (P->smem_floats * 4 + 1024))));
+    const int per_sm = std::max(1, std::min(3, (int)(227 * 1024 / (P->smem_floats * 4 + 10 * 1024))));
     std::vector<double> times(p.tensors.size(), n);  // how often every tensor is computed
     double total = P->key_bits ? 20000.0 * sm_count() : 0;
     if (top >= 0) {
@@ -643,7 +777,8 @@ bool build_program(const Plan &p, int64_t n, SProgram *P, std::string *why) {
         SProgram Q;
         double cost = 0;
         if (n > (int64_t)1 << 31 && top >= 0) break;  // positions of the sorted list are 32-bit
-        if (layout_program(p, (double)n, top, false, &Q, &cost, &w) && cost < best) {
+        if (!layout_program(p, (double)n, top, false, &Q, &cost, &w)) continue;
+        if (cost < best) {
             best = cost;
             *P = Q;
         }

@@ -27,10 +27,9 @@
 // counting sort), and a CTA walks a contiguous range of the sorted list: the
 // shared steps run on all 256 threads when a bit they depend on has changed,
 // and every state's remaining steps run on one warp, eight states at a time,
-// with no barrier between them.  A K range too long for its outputs is split
-// over neighbouring lanes and summed with shuffles.  10^6 states of the
-// 30-qubit grid: 45.1 -> 4.7 ms (the kernel 4.5 ms: 2.1 in the shared steps,
-// 2.1 in the warps'; the sort 0.07 ms).
+// with no barrier between them.  10^6 states of the 30-qubit
+// grid, FP32 results: 45.1 -> 4.7 ms (the kernel 4.5 ms: 2.1 in the shared
+// steps, 2.1 in the warps'; the sort 0.07 ms).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -74,9 +73,10 @@ struct SStep {
     int32_t a_off, b_off;   // offsets (floats) of SRC_CTA / SRC_WARP operands
     int32_t mb, nb, kb;     // log2 of M, N, K
     uint32_t maskR, maskC;  // result-layout bits of the row / column index bits
-    int32_t c_kb, c_lkl;    // log2 K and lkl of the step consuming the result; c_kb -1 for the final step
+    int32_t c_kb;           // log2 K of the step consuming the result; -1 for the final step
     int32_t c_off;          // the result's place: rows of 2^c_kb, padded
-    int32_t lkl;            // log2 of the lanes sharing one output tile's K range
+    int32_t lkl;            // log2 of the lanes sharing one output tile's K range (FP32 results)
+    int32_t lkc;            // log2 of the multiply-adds in one partial sum (FP64 results)
     int32_t tab_off;        // result offsets of rows (M) then columns (N), in shared memory
 };
 
@@ -94,10 +94,9 @@ struct SProgram {
     int32_t smem_floats;
 };
 
-// Row pitch of a [rows][K] operand in shared memory whose K is read by 2^lkl
-// neighbouring lanes, 16 bytes each: K + 4 * 2^lkl floats puts the eight lanes
-// of a 16-byte access phase (2^lkl pieces of 8 / 2^lkl rows) on distinct banks.
-__host__ __device__ __forceinline__ int pitch_of(int k, int lkl) { return k >= 4 ? k + (lkl < 3 ? 4 << lkl : 4) : k; }
+// Row pitch of a [rows][K] operand in shared memory: K + 4 floats keeps
+// 16-byte access and spreads rows over the banks.
+__host__ __device__ __forceinline__ int pitch_of(int k) { return k >= 4 ? k + 4 : k; }
 
 // Two FP32 multiply-adds per instruction (even and odd k in the two halves).
 __device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) {
@@ -105,9 +104,6 @@ __device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) {
 }
 __device__ __forceinline__ float lo32(uint64_t c) { return __uint_as_float((uint32_t)c); }
 __device__ __forceinline__ float hi32(uint64_t c) { return __uint_as_float((uint32_t)(c >> 32)); }
-
-// log2 of the register tile along a dimension of 2^b results.
-__host__ __device__ __forceinline__ int tile_log2(int b) { return b >= 2 ? 2 : 0; }
 
 // Store the LEFT = TM TN >> lkl results (at least one) of a tile that are
 // left in this lane, e0 on, at rows rt + i rs and columns ct + j cs.
@@ -130,19 +126,18 @@ __device__ __forceinline__ void put_left(const float *acc, int lkl, int e0, int 
     }
 }
 
-// Output tiles of TM x TN results (rows strided by M / TM, columns by
-// N / TN), tile t of every nw x (32 >> lkl): 2^lkl neighbouring lanes share a
-// tile, lane ks taking the 16-byte pieces ks, ks + 2^lkl, ... of K (whole
-// sectors of a row, no bank conflicts).  Their partial sums are added by
-// recursive halving, which leaves every lane a part of the tile's results to
-// store, (r, c) at res[tab[r] + tab[M + c]].  AG / BG: the operand is in
-// global memory.  4 x 4 tiles move 8 16-byte pieces for 64 multiply-adds, and
-// shared memory delivers 128 bytes a clock, which bounds a CTA's step at half
-// the FP32 rate; 8 x 4 and 8 x 8 tiles move less but measured slower (10^6
-// grid30 states 5.5 and 5.8 against 5.0 ms: two CTAs per SM, not three, and
-// longer reductions).
+// FP32 results: K is split over lanes.  Tile t of every nw x (32 >> lkl):
+// 2^lkl neighbouring lanes share a tile, lane ks taking the 16-byte pieces ks,
+// ks + 2^lkl, ... of K (whole sectors of a row, no bank conflicts).  Their
+// partial sums are added by recursive halving, which leaves every lane a part
+// of the tile's results to store, (r, c) at res[tab[r] + tab[M + c]].  AG / BG:
+// the operand is in global memory.  4 x 4 tiles move 8 16-byte pieces for 64
+// multiply-adds, and shared memory delivers 128 bytes a clock, which bounds a
+// CTA's step at half the FP32 rate; 8 x 4 and 8 x 8 tiles move less but
+// measured slower (10^6 grid30 states 5.5 and 5.8 against 5.0 ms: two CTAs per
+// SM, not three, and longer reductions).
 template <int TM, int TN, bool AG, bool BG>
-__device__ __forceinline__ void step_tiles(const float *A, int pa, const float *B, int pb, int mb, int nb, int kb,
+__device__ __forceinline__ void step_split(const float *A, int pa, const float *B, int pb, int mb, int nb, int kb,
                                            int lkl, int w, int nw, int lane, float *res, const int *tab) {
     if constexpr (!AG) __builtin_assume(__isShared(A));
     if constexpr (!BG) __builtin_assume(__isShared(B));
@@ -217,28 +212,116 @@ __device__ __forceinline__ void step_tiles(const float *A, int pa, const float *
     }
 }
 
-template <bool AG, bool BG>
+// FP64 results: every sum in one order.  Output tiles of TM x TN results (rows
+// strided by M / TM, columns by N / TN), one per thread; a result is the sum,
+// in order, of K / kc partial sums, each one chain of kc multiply-adds,
+// whatever the tile, the number of threads or the shared steps: a state's
+// value does not depend on its list (10^6 grid30 states: 6.9 ms, 4.7 with
+// the split sums).
+template <int TM, int TN, bool AG, bool BG>
+__device__ __forceinline__ void step_tiles(const float *A, int pa, const float *B, int pb, int mb, int nb, int kb,
+                                           int lkc, int t0, int nt, float *res, const int *tab) {
+    if constexpr (!AG) __builtin_assume(__isShared(A));
+    if constexpr (!BG) __builtin_assume(__isShared(B));
+    constexpr int E = TM * TN;
+    const int rs = (1 << mb) / TM, cs = (1 << nb) / TN;
+    const int lc = nb - (TN == 4 ? 2 : (TN == 2 ? 1 : 0));
+    for (int t = t0; t < rs * cs; t += nt) {
+        const int rt = t >> lc, ct = t & (cs - 1);
+        float acc[E], tot[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[e] = tot[e] = 0.f;
+        if (kb >= 2) {
+            const float *pA = A + rt * pa, *pB = B + ct * pb;
+            const int sa = rs * pa, sb = cs * pb, m4 = (1 << (lkc - 2)) - 1;
+            const bool one = lkc == kb;
+#pragma unroll (E <= 4 ? 4 : 1)
+            for (int k4 = 0; k4 < 1 << (kb - 2); ++k4) {
+                float4 a[TM], b[TN];
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+                    a[i] = AG ? __ldg((const float4 *)(pA + i * sa) + k4) : ((const float4 *)(pA + i * sa))[k4];
+#pragma unroll
+                for (int j = 0; j < TN; ++j)
+                    b[j] = BG ? __ldg((const float4 *)(pB + j * sb) + k4) : ((const float4 *)(pB + j * sb))[k4];
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+#pragma unroll
+                    for (int j = 0; j < TN; ++j) {
+                        float &c = acc[i * TN + j];
+                        c = fmaf(a[i].x, b[j].x, c);
+                        c = fmaf(a[i].y, b[j].y, c);
+                        c = fmaf(a[i].z, b[j].z, c);
+                        c = fmaf(a[i].w, b[j].w, c);
+                    }
+                if (!one && (k4 & m4) == m4) {
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        tot[e] += acc[e];
+                        acc[e] = 0.f;
+                    }
+                }
+            }
+            if (!one) {
+#pragma unroll
+                for (int e = 0; e < E; ++e) acc[e] = tot[e];
+            }
+        } else {  // K = 1
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j)
+                    acc[i * TN + j] = fmaf(A[(rt + i * rs) * pa], B[(ct + j * cs) * pb], 0.f);
+        }
+        int oc[TN];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) oc[j] = tab[(1 << mb) + ct + j * cs];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            float *o = res + tab[rt + i * rs];
+#pragma unroll
+            for (int j = 0; j < TN; ++j) o[oc[j]] = acc[i * TN + j];
+        }
+    }
+}
+
+// A step by the warps w, ... of nw.
+template <bool ORD, bool AG, bool BG>
 __device__ __forceinline__ void step_run(const SStep &S, const float *A, const float *B, int w, int nw, int lane,
                                          float *res, const int *tab) {
     __builtin_assume(__isShared(res));
     __builtin_assume(__isShared(tab));
-    const int K = 1 << S.kb, pk = pitch_of(K, S.lkl), pa = AG ? K : pk, pb = BG ? K : pk;
-    if (S.mb >= 2 && S.nb >= 2) step_tiles<4, 4, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, res, tab);
-    else if (S.mb >= 2) step_tiles<4, 1, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, res, tab);
-    else if (S.nb >= 2) step_tiles<1, 4, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, res, tab);
-    else step_tiles<1, 1, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, res, tab);
+    const int K = 1 << S.kb, pk = pitch_of(K), pa = AG ? K : pk, pb = BG ? K : pk;
+    if constexpr (ORD) {
+#define TQC_ST_TILE(TM, TN) \
+    step_tiles<TM, TN, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkc, 32 * w + lane, 32 * nw, res, tab)
+        // up to 4 x 4, while every thread has a tile
+        const int each = (1 << (S.mb + S.nb)) / (32 * nw);
+        if (each < 2 || S.mb < 2 || S.nb < 2) TQC_ST_TILE(1, 1);
+        else if (each < 4) TQC_ST_TILE(2, 1);
+        else if (each < 16) TQC_ST_TILE(2, 2);
+        else TQC_ST_TILE(4, 4);
+#undef TQC_ST_TILE
+    } else {
+#define TQC_ST_TILE(TM, TN) \
+    step_split<TM, TN, AG, BG>(A, pa, B, pb, S.mb, S.nb, S.kb, S.lkl, w, nw, lane, res, tab)
+        if (S.mb >= 2 && S.nb >= 2) TQC_ST_TILE(4, 4);
+        else if (S.mb >= 2) TQC_ST_TILE(4, 1);
+        else if (S.nb >= 2) TQC_ST_TILE(1, 4);
+        else TQC_ST_TILE(1, 1);
+#undef TQC_ST_TILE
+    }
 }
 
 // Copy a leaf operand (2^row_log2 floats, rows of 2^kb, from one table row)
 // to padded rows in shared memory with 16-byte asynchronous copies (by
 // threads i of n; the caller waits).
-__device__ __forceinline__ void copy_rows(const float *row, int row_log2, int kb, int lkl, float *dst, int i,
-                                          int n) {
+__device__ __forceinline__ void copy_rows(const float *row, int row_log2, int kb, float *dst, int i, int n) {
     if (row_log2 < 2) {  // a subcircuit without cuts: one value
         if (i == 0) dst[0] = __ldg(row);
         return;
     }
-    const int lq = kb >= 2 ? kb - 2 : 30, skip = pitch_of(1 << kb, lkl) - (1 << kb);  // pieces per row (K = 1: contiguous)
+    const int lq = kb >= 2 ? kb - 2 : 30, skip = kb >= 2 ? 4 : 0;  // pieces per row (K = 1: contiguous)
     for (; i < 1 << (row_log2 - 2); i += n)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
                          (uint32_t)__cvta_generic_to_shared(dst + 4 * i + skip * (i >> lq))),
@@ -247,31 +330,34 @@ __device__ __forceinline__ void copy_rows(const float *row, int row_log2, int kb
 }
 __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// The final step's partial sum over pieces i, i + n, ... of K (16 bytes
-// each; K = 1: one element), added over the warp.
-__device__ __forceinline__ float final_dot(const float *A, const float *B, int kb, int i, int n) {
+// The final step on one warp: lane i takes the partial sums i, i + 32, ...
+// (2^lkc multiply-adds each), which are added in order.
+__device__ __forceinline__ float final_dot(const float *A, const float *B, int kb, int lkc, int lane) {
+    if (kb < 2) return fmaf(A[0], B[0], 0.f);
+    const int blocks = 1 << (kb - lkc), n4 = 1 << (lkc - 2);
     float v = 0.f;
-    if (kb >= 2) {
-        for (int k = i; k < 1 << (kb - 2); k += n) {
-            const float4 a = ((const float4 *)A)[k], b = ((const float4 *)B)[k];
-            v = fmaf(a.x, b.x, v);
-            v = fmaf(a.y, b.y, v);
-            v = fmaf(a.z, b.z, v);
-            v = fmaf(a.w, b.w, v);
-        }
-    } else if (i == 0) {
-        v = A[0] * B[0];
+    for (int b0 = 0; b0 < blocks; b0 += 32) {
+        float c = 0.f;
+        if (b0 + lane < blocks)
+            for (int k = (b0 + lane) * n4; k < (b0 + lane + 1) * n4; ++k) {
+                const float4 a = ((const float4 *)A)[k], b = ((const float4 *)B)[k];
+                c = fmaf(a.x, b.x, c);
+                c = fmaf(a.y, b.y, c);
+                c = fmaf(a.z, b.z, c);
+                c = fmaf(a.w, b.w, c);
+            }
+        const int m = blocks - b0 < 32 ? blocks - b0 : 32;
+        for (int i = 0; i < m; ++i) v += __shfl_sync(0xffffffffu, c, i);
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
+// ORD: the results are FP64 (and every sum in one order), else FP32.
+template <bool ORD>
 __global__ void __launch_bounds__(ST_THREADS, 3)
     states_kernel(const __grid_constant__ SProgram P, const uint64_t *__restrict__ list,
-                  const uint32_t *__restrict__ place, int64_t n, void *out, int out_f64, const double *zinfo) {
+                  const uint32_t *__restrict__ place, int64_t n, void *out, const double *zinfo) {
     extern __shared__ __align__(16) float sm[];
-    __shared__ float part[ST_WARPS];
     __shared__ uint64_t win_y[ST_WINDOW];
     __shared__ uint32_t win_place[ST_WINDOW];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -284,7 +370,7 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
         const SStep &S = P.step[si];
         const int M = 1 << S.mb, N = 1 << S.nb;
         int *tab = (int *)(sm + S.tab_off);
-        const int ck = S.c_kb < 0 ? 1 : 1 << S.c_kb, pc = pitch_of(ck, S.c_lkl);
+        const int ck = S.c_kb < 0 ? 1 : 1 << S.c_kb, pc = pitch_of(ck);
         for (int i = tid; i < M + N; i += ST_THREADS) {
             const uint32_t d = i < M ? pdep32((uint32_t)i, S.maskR) : pdep32((uint32_t)(i - M), S.maskC);
             tab[i] = S.c_kb < 0 ? 0 : (int)(d >> S.c_kb) * pc + (int)(d & (uint32_t)(ck - 1));
@@ -293,7 +379,7 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
     __syncthreads();
     auto store = [&](int64_t at, float v) {
         const double d = (double)v * scale;
-        if (out_f64) ((double *)out)[at] = d;
+        if (ORD) ((double *)out)[at] = d;
         else ((float *)out)[at] = (float)d;
     };
     auto row_of = [&](int leaf, uint64_t y) {
@@ -319,17 +405,17 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
             const float *A = ag ? row_of(S.a_leaf, y) : (S.a_kind == SRC_CTA ? sm : wsm) + S.a_off;
             const float *B = bg ? row_of(S.b_leaf, y) : (S.b_kind == SRC_CTA ? sm : wsm) + S.b_off;
             if (S.c_kb < 0) {
-                const float v = final_dot(A, B, S.kb, lane, 32);
+                const float v = final_dot(A, B, S.kb, S.lkc, lane);
                 if (lane == 0) store(at, v);
                 __syncwarp();
                 return;
             }
             const int *tab = (const int *)(sm + S.tab_off);
             float *res = wsm + S.c_off;
-            if (ag && bg) step_run<true, true>(S, A, B, 0, 1, lane, res, tab);
-            else if (ag) step_run<true, false>(S, A, B, 0, 1, lane, res, tab);
-            else if (bg) step_run<false, true>(S, A, B, 0, 1, lane, res, tab);
-            else step_run<false, false>(S, A, B, 0, 1, lane, res, tab);
+            if (ag && bg) step_run<ORD, true, true>(S, A, B, 0, 1, lane, res, tab);
+            else if (ag) step_run<ORD, true, false>(S, A, B, 0, 1, lane, res, tab);
+            else if (bg) step_run<ORD, false, true>(S, A, B, 0, 1, lane, res, tab);
+            else step_run<ORD, false, false>(S, A, B, 0, 1, lane, res, tab);
             __syncwarp();
         }
     };
@@ -360,15 +446,14 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
                 if (leaf < 0) continue;
                 const uint64_t lm = ((1ull << P.leaf[leaf].n_q) - 1ull) << P.leaf[leaf].y_off;
                 if (!all && !(diff & lm)) continue;
-                copy_rows(row_of(leaf, y), P.leaf[leaf].row_log2, S.kb, S.lkl, sm + (op ? S.b_off : S.a_off),
-                          tid, ST_THREADS);
+                copy_rows(row_of(leaf, y), P.leaf[leaf].row_log2, S.kb, sm + (op ? S.b_off : S.a_off), tid, ST_THREADS);
             }
         }
     };
     // One shared step on the whole CTA (not the final one).
     auto shared_step = [&](const SStep &S) {
-        step_run<false, false>(S, sm + S.a_off, sm + S.b_off, warp, ST_WARPS, lane, sm + S.c_off,
-                               (const int *)(sm + S.tab_off));
+        step_run<ORD, false, false>(S, sm + S.a_off, sm + S.b_off, warp, ST_WARPS, lane, sm + S.c_off,
+                                    (const int *)(sm + S.tab_off));
     };
     if (P.one_each) {  // every step on the whole CTA, one state at a time
         uint64_t prev = 0;
@@ -386,12 +471,10 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
                 if (S.c_kb >= 0) {
                     shared_step(S);
                 } else {
-                    const float v = final_dot(sm + S.a_off, sm + S.b_off, S.kb, tid, ST_THREADS);
-                    if (lane == 0) part[warp] = v;
-                    __syncthreads();
-                    float sum = 0.f;
-                    for (int w = 0; w < ST_WARPS; ++w) sum += part[w];
-                    if (tid == 0) store(place_of(p), sum);
+                    if (warp == 0) {
+                        const float v = final_dot(sm + S.a_off, sm + S.b_off, S.kb, S.lkc, lane);
+                        if (lane == 0) store(place_of(p), v);
+                    }
                 }
                 __syncthreads();
             }
@@ -644,24 +727,13 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
     if (P->one_each && top != ns - 1) return *why = "shared subtree has too many output bits", false;
     const int n_shared = (int)std::count_if(order.begin(), order.end(), [&](int s) { return shared[(size_t)p.steps[s].c] != 0; });
     P->n_shared = n_shared;
-    // lanes per output tile: what the tiles leave idle, at most one per 16
-    // bytes of K; rows read from global memory always 8 (a whole line)
-    std::vector<int> lkl_of((size_t)ns, 0);
-    for (int i = 0; i < ns; ++i) {
-        const StepPlan &st = p.steps[order[(size_t)i]];
-        const bool cta = i < n_shared;
-        const int tiles = st.mb + st.nb - tile_log2(st.mb) - tile_log2(st.nb);  // log2
-        int lkl = std::max(0, std::min(5, (cta ? 8 : 5) - tiles));
-        if (!cta && (st.a < p.m || st.b < p.m)) lkl = std::max(lkl, 3);
-        lkl_of[(size_t)order[(size_t)i]] = std::max(0, std::min(lkl, st.kb - 2));
-    }
     // shared memory: leaf operands of the shared steps, intermediates, the
     // warps' own intermediates, the offset tables
     int64_t off = 0, woff = 0, area[2] = {0, 0};
     std::vector<int> place(p.tensors.size(), 0);
     for (int i = 0; i < n_shared; ++i) {
         const StepPlan &st = p.steps[order[(size_t)i]];
-        const int64_t pk = pitch_of(1 << st.kb, lkl_of[(size_t)order[(size_t)i]]);
+        const int64_t pk = pitch_of(1 << st.kb);
         const int64_t need[2] = {((int64_t)1 << st.mb) * pk, ((int64_t)1 << st.nb) * pk};
         const int t[2] = {st.a, st.b};
         for (int k = 0; k < 2; ++k) {
@@ -689,7 +761,7 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
             continue;
         }
         const int64_t ck = (int64_t)1 << p.steps[c].kb;
-        const int64_t need = align4((((int64_t)1 << (st.mb + st.nb)) / ck) * pitch_of((int)ck, lkl_of[(size_t)c]));
+        const int64_t need = align4((((int64_t)1 << (st.mb + st.nb)) / ck) * pitch_of((int)ck));
         int64_t &o = i < n_shared ? off : woff;
         place[(size_t)st.c] = (int)o;
         o += need;
@@ -704,9 +776,17 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
         S.maskC = (uint32_t)st.maskC;
         S.mask = bits_of(p.tensors[(size_t)st.c].leaves);
         const int c = consumer[(size_t)st.c];
-        S.lkl = lkl_of[(size_t)order[(size_t)i]];
+        // lanes per output tile: what the tiles leave idle, at most one per 16
+        // bytes of K; rows read from global memory always 8 (a whole line)
+        const int tiles = std::max(0, st.mb - 2) + std::max(0, st.nb - 2);  // log2
+        const bool cta = i < n_shared, table = !cta && (st.a < p.m || st.b < p.m);
+        const int lkl = std::max(table ? 3 : 0, std::min(5, (cta ? 8 : 5) - tiles));
+        S.lkl = std::max(0, std::min(lkl, st.kb - 2));
+        // partial sums: K in as many parts as give 256 threads a tile each, of
+        // at least 4 multiply-adds
+        S.lkc = st.kb;
+        while (st.kb - S.lkc + 1 + tiles <= 8 && S.lkc >= 3) --S.lkc;
         S.c_kb = c < 0 ? -1 : p.steps[c].kb;
-        S.c_lkl = c < 0 ? 0 : lkl_of[(size_t)c];
         S.c_off = place[(size_t)st.c];
         auto operand = [&](int t, int32_t *leaf, int32_t *kind, int32_t *o) {
             *leaf = t < p.m ? t : -1;
@@ -912,18 +992,19 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
             d_list = sorted;
         }
         const size_t smem = (size_t)P.smem_floats * 4;
-        static size_t attr = 0;
-        if (smem > 48 * 1024 && smem > attr) {
-            e = cudaFuncSetAttribute(states_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const bool f64 = out_dtype == TQC_F64;
+        auto *kernel = f64 ? states_kernel<true> : states_kernel<false>;
+        static size_t attr[2] = {0, 0};
+        if (smem > 36 * 1024 && smem > attr[f64]) {  // beside 9 KB of static shared memory
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return cuda_fail(e, "state-list kernel attribute");
-            attr = smem;
+            attr[f64] = smem;
         }
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, states_kernel, ST_THREADS, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, ST_THREADS, smem);
         if (e != cudaSuccess || per_sm < 1) return fail(TQC_ERR_UNSUPPORTED, "state-list kernel does not fit an SM");
         const int64_t grid = std::min<int64_t>(n, (int64_t)per_sm * sm_count());
-        states_kernel<<<(unsigned)grid, ST_THREADS, smem, s>>>(P, d_list, d_place, n, d_out, out_dtype == TQC_F64,
-                                                              p->d_zinfo);
+        kernel<<<(unsigned)grid, ST_THREADS, smem, s>>>(P, d_list, d_place, n, d_out, p->d_zinfo);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "state-list kernel");
     } else if (n > 0) {

@@ -222,6 +222,11 @@ int default_step_tile(const StepPlan &st, int out_esize, bool smallk) {
         return st.nb >= 7 ? UMMA_128x128 : UMMA_128x64;
     }
     if (smallk && smallk_ok(st.mb, st.nb, st.kb, st.kblk)) return SIMT_SMALLK;
+    // K >= 16: too few 128 x 128 tiles to give every SM one run as 64 x 64
+    // (four times the CTAs, a quarter of a tile's latency: a 17-qubit FP32
+    // contract 242 -> 72 us together with simt_gemm_f32)
+    if (st.kb >= 4 && st.mb >= 6 && st.nb >= 6 && ((int64_t)1 << (st.mb + st.nb)) < ((int64_t)sm_count() << 14))
+        return SIMT_64x64;
     return (st.mb >= 7 && st.nb >= 7) ? SIMT_128x128 : (st.mb >= 7 && st.nb >= 6 ? SIMT_128x64 : SIMT_64x64);
 }
 

@@ -93,6 +93,139 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 }
 
 
+__device__ __forceinline__ uint64_t dup2(float a) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+
+// Whole BM x BN tiles of a step with K >= 16 (a multiple of 16): TM x 8
+// results per thread, operands copied 16 k at a time through registers into
+// one of two [k][row] buffers while the other is multiplied.  Bound by FP32
+// arithmetic and, as closely, by shared memory: a k takes 16 bytes of loads
+// per 16 multiply-adds, 128 bytes a clock against 128 multiply-adds a clock.
+// The multiply-adds are packed two columns to an instruction (the row's value
+// doubled), which leaves the issue slots for the loads.  Row m of k sits at
+// m ^ 8 (k / 4 mod 4): the transposing stores of a warp (8 rows x 4 pieces of
+// 4 k) and the 16-byte loads are free of bank conflicts.  The k order and the
+// multiply-adds are those of simt_step_f32, so the two agree bit for bit.
+// Measured (K = 64, 2^16 x 2^11 results; K = 256, 2^19 x 2^7; K = 64, 2^20 x
+// 2^8 into 1.07 GB of output): 0.605, 1.195 and 1.31 ms before, 0.41, 0.74 and
+// 0.875 ms now (20.9, 23.3 and 19.6 T multiply-adds/s of 39.8); 16 x 8 results
+// per thread (fewer loads, half the warps): 0.42, 0.77 and 0.90 ms.
+template <int BM, int BN, int TM, int MINB>
+__global__ void __launch_bounds__((BM / TM) * (BN / 8), MINB)
+    simt_gemm_f32(StepArgs args, int64_t n_tiles, int64_t col_tiles) {
+    constexpr int NX = BN / 8, NY = BM / TM, NT = NX * NY, BK = 16;
+    constexpr int LA = BM * BK / 4 / NT, LB = BN * BK / 4 / NT;  // 16-byte pieces per thread and chunk
+    constexpr int PS = BN + 4;
+    constexpr int BUF = BK * (BM + BN);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    EpiTables *tb = (EpiTables *)smem_raw;
+    float *buf = (float *)(smem_raw + sizeof(EpiTables));  // two operand buffers; the staged tile aliases them
+    const EpiParams &e = args.epi;
+    const int64_t K = 1ll << args.kb;
+    const int chunks = 1 << (args.kb - 4);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // a warp covers 4 x 8 threads: rows 4 ty + 4 NY u, columns 4 tx + 4 NX v
+    constexpr int WX = NX / 8;
+    const int tx = (warp % WX) * 8 + (lane & 7), ty = (warp / WX) * 4 + (lane >> 3);
+    epi_tables_init(tb, e, true, PS, tid, NT);
+    const int gm = gather_mode(e.lowCc);
+    float4 pa[LA], pb[LB];
+    auto load = [&](int64_t tile, int c) {
+        const int64_t rt = tile / col_tiles, ct = tile - rt * col_tiles;
+        const float *A = (const float *)args.A + rt * BM * K + c * BK, *B = (const float *)args.B + ct * BN * K + c * BK;
+#pragma unroll
+        for (int j = 0; j < LA; ++j) {
+            const int f = tid + j * NT;
+            pa[j] = *(const float4 *)(A + (int64_t)(f >> 2) * K + (f & 3) * 4);
+        }
+#pragma unroll
+        for (int j = 0; j < LB; ++j) {
+            const int f = tid + j * NT;
+            pb[j] = *(const float4 *)(B + (int64_t)(f >> 2) * K + (f & 3) * 4);
+        }
+    };
+    load(blockIdx.x, 0);
+    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const int64_t rt = tile / col_tiles, ct = tile - rt * col_tiles;
+        uint64_t acc[TM][4];
+#pragma unroll
+        for (int u = 0; u < TM; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[u][v] = 0;
+        auto put = [&](int c) {
+            float *As = buf + (c & 1) * BUF, *Bs = As + BK * BM;
+#pragma unroll
+            for (int j = 0; j < LA; ++j) {
+                const int f = tid + j * NT, k4 = f & 3;
+                float *d = As + 4 * k4 * BM + ((f >> 2) ^ (k4 << 3));
+                d[0] = pa[j].x;
+                d[BM] = pa[j].y;
+                d[2 * BM] = pa[j].z;
+                d[3 * BM] = pa[j].w;
+            }
+#pragma unroll
+            for (int j = 0; j < LB; ++j) {
+                const int f = tid + j * NT, k4 = f & 3;
+                float *d = Bs + 4 * k4 * BN + ((f >> 2) ^ (k4 << 3));
+                d[0] = pb[j].x;
+                d[BN] = pb[j].y;
+                d[2 * BN] = pb[j].z;
+                d[3 * BN] = pb[j].w;
+            }
+        };
+        put(0);
+        __syncthreads();
+        for (int c = 0; c < chunks; ++c) {
+            if (c + 1 < chunks) load(tile, c + 1);
+            const float *As = buf + (c & 1) * BUF, *Bs = As + BK * BM;
+#pragma unroll
+            for (int k = 0; k < BK; ++k) {
+                const int sw = (k >> 2) << 3;
+                ulonglong2 b[2];
+#pragma unroll
+                for (int v = 0; v < 2; ++v)
+                    b[v] = *(const ulonglong2 *)(Bs + k * BN + ((4 * tx + 4 * NX * v) ^ sw));
+#pragma unroll
+                for (int u = 0; u < TM / 4; ++u) {
+                    const float4 a = *(const float4 *)(As + k * BM + ((4 * ty + 4 * NY * u) ^ sw));
+                    const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const uint64_t d = dup2(av[i]);
+                        fma2(acc[4 * u + i][0], d, b[0].x);
+                        fma2(acc[4 * u + i][1], d, b[0].y);
+                        fma2(acc[4 * u + i][2], d, b[1].x);
+                        fma2(acc[4 * u + i][3], d, b[1].y);
+                    }
+                }
+            }
+            if (c + 1 < chunks) {
+                put(c + 1);  // the other buffer: its readers passed the last barrier
+                __syncthreads();
+            }
+        }
+        // the next tile's first chunk arrives during the write-out
+        if (tile + gridDim.x < n_tiles) load(tile + gridDim.x, 0);
+        __syncthreads();
+        float *stg = buf;
+#pragma unroll
+        for (int u = 0; u < TM; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+                *(ulonglong2 *)&stg[(4 * ty + 4 * NY * (u >> 2) + (u & 3)) * PS + 4 * tx + 4 * NX * v] =
+                    make_ulonglong2(acc[u][2 * v], acc[u][2 * v + 1]);
+        __syncthreads();
+        epi_readout(tb, stg, e, tile_base(e, rt, ct), BM * BN, tid, NT, gm);
+        __syncthreads();
+    }
+}
+
 // Small-K step (smallk.cuh): one 128-thread CTA per tile slot, one kernel
 // per K, tile width and orientation (each with its own register budget);
 // when the tiles are staged, the staging tables are built once per CTA.
@@ -285,6 +418,25 @@ cudaError_t launch_cfg(const StepArgs &a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// The tile configurations of K >= 16 steps whose tiles are whole.
+template <int BM, int BN, int TM, int MINB>
+cudaError_t launch_gemm(const StepArgs &a, cudaStream_t s) {
+    constexpr int NT = (BM / TM) * (BN / 8);
+    const size_t smem = sizeof(EpiTables) + std::max((size_t)2 * 16 * (BM + BN), (size_t)BM * (BN + 4)) * sizeof(float);
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(simt_gemm_f32<BM, BN, TM, MINB>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    const int64_t col_tiles = 1ll << (a.nb - a.epi.b_bits);
+    const int64_t n_tiles = (1ll << (a.mb - a.epi.a_bits)) * col_tiles;
+    const int64_t grid = std::min<int64_t>(n_tiles, (int64_t)sm_count() * MINB);
+    simt_gemm_f32<BM, BN, TM, MINB><<<(unsigned)grid, NT, smem, s>>>(a, n_tiles, col_tiles);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 int sm_count() {
@@ -431,9 +583,15 @@ cudaError_t launch_smallk(const StepArgs &a, cudaStream_t s) {
 cudaError_t launch_simt_step(int cfg, const StepArgs &a, cudaStream_t s) {
     switch (cfg) {
         case SIMT_SMALLK: return launch_smallk(a, s);
-        case SIMT_128x128: return launch_cfg<128, 128, 8, 8>(a, s);
-        case SIMT_128x64: return launch_cfg<128, 64, 8, 4>(a, s);
-        default: return launch_cfg<64, 64, 4, 4>(a, s);
+        case SIMT_128x128:
+            if (a.kb >= 4 && a.epi.a_bits == 7 && a.epi.b_bits == 7) return launch_gemm<128, 128, 8, 2>(a, s);
+            return launch_cfg<128, 128, 8, 8>(a, s);
+        case SIMT_128x64:
+            if (a.kb >= 4 && a.epi.a_bits == 7 && a.epi.b_bits == 6) return launch_gemm<128, 64, 8, 3>(a, s);
+            return launch_cfg<128, 64, 8, 4>(a, s);
+        default:
+            if (a.kb >= 4 && a.epi.a_bits == 6 && a.epi.b_bits == 6) return launch_gemm<64, 64, 4, 6>(a, s);
+            return launch_cfg<64, 64, 4, 4>(a, s);
     }
 }
 

@@ -21,6 +21,16 @@
 
 namespace tqc {
 
+// Programmatic dependent launch.  Every kernel of a contract is launched while
+// its predecessor may still run (launch_pdl, launch.h) and calls both: launch
+// lets the next kernel's CTAs start as SMs drain, wait returns once the
+// predecessor has completed and its writes are visible.  Before wait a kernel
+// touches only its parameters and its own shared and tensor memory; since every
+// kernel of the chain waits, a completed predecessor means that all earlier
+// ones have completed too.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Deposit the low bits of `src` into the set bits of `mask`, lowest first.
 __device__ __forceinline__ uint64_t pdep64(uint64_t src, uint64_t mask) {
     uint64_t r = 0;

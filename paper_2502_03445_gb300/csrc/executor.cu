@@ -455,30 +455,66 @@ void exec_release(Plan *p) {
     p->ready = false;
 }
 
+namespace {
+
+// Ingest of every leaf of the total-mass network of one slice.
+void mass_leaves(const Plan &p, const ExecCtx &c, int64_t sl, std::vector<IngestArgs> *out) {
+    double *zslice = (double *)ws_ptr(c.zws, p.zws_bytes);
+    for (int j = 0; j < p.m; ++j) {
+        const TensorPlan &t = p.ztensors[j];
+        IngestArgs g = leaf_args(p, t, j, p.fixed_bits.data(), sl, true, &c);
+        g.dst = p.m == 1 ? (void *)(zslice + sl) : (void *)ws_ptr(c.zws, t.offset);
+        out->push_back(g);
+    }
+}
+
+std::vector<ZStep> mass_steps(const Plan &p, void *zws, double *zout) {
+    std::vector<ZStep> z;
+    for (auto &zs : p.zsteps) {
+        ZStep a;
+        a.A = (const double *)ws_ptr(zws, p.ztensors[zs.a].offset);
+        a.B = (const double *)ws_ptr(zws, p.ztensors[zs.b].offset);
+        a.out = zs.final ? zout : (double *)ws_ptr(zws, p.ztensors[zs.c].offset);
+        a.mb = zs.mb;
+        a.nb = zs.nb;
+        a.kb = zs.kb;
+        a.maskR = zs.maskR;
+        a.maskC = zs.maskC;
+        z.push_back(a);
+    }
+    return z;
+}
+
+// The steps of slice sl's network (its leaves are in c.zws); after the last
+// slice also Z and the scale.
+cudaError_t mass_run(const Plan &p, const ExecCtx &c, int64_t sl, cudaStream_t s) {
+    double *zslice = (double *)ws_ptr(c.zws, p.zws_bytes);
+    const std::vector<ZStep> z = mass_steps(p, c.zws, zslice + sl);
+    const int64_t ns = p.n_slices();
+    return launch_znet(z.data(), (int)z.size(), sl + 1 == ns ? zslice : nullptr, (int)ns, p.net->n_cuts,
+                       !(p.flags & TQC_FLAG_NO_RENORM), c.zinfo, s);
+}
+
+}  // namespace
+
+int total_mass_launches(const Plan &p) {
+    const std::vector<ZStep> z = mass_steps(p, nullptr, nullptr);
+    const int64_t ns = p.n_slices();
+    const int per = (p.m + INGEST_MAX - 1) / INGEST_MAX + znet_launches(z.data(), (int)z.size(), false);
+    return (int)(per * ns) + znet_launches(z.data(), (int)z.size(), true) - znet_launches(z.data(), (int)z.size(), false);
+}
+
 // Total mass Z of the network (every output summed: a scalar network per
 // slice, FP64), then zinfo = [Z, scale = 2^{-|E|} / Z (or 2^{-|E|} without
 // renormalisation)].
-tqc_status exec_total_mass(const Plan &pl, const ExecCtx &c, void *stream) {
-    const Plan *p = &pl;
+tqc_status exec_total_mass(const Plan &p, const ExecCtx &c, void *stream) {
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t ns = p->n_slices();
-    double *zslice = (double *)ws_ptr(c.zws, p->zws_bytes);
-    for (int64_t sl = 0; sl < ns; ++sl) {
-        for (int j = 0; j < p->m; ++j) {
-            const TensorPlan &t = p->ztensors[j];
-            IngestArgs g = leaf_args(*p, t, j, p->fixed_bits.data(), sl, true, &c);
-            g.dst = p->m == 1 ? (void *)(zslice + sl) : (void *)ws_ptr(c.zws, t.offset);
-            TQC_CUDA(launch_ingest(g, (int64_t)1 << t.nbits(), s), "total-mass ingest");
-        }
-        for (size_t i = 0; i < p->zsteps.size(); ++i) {
-            const StepPlan &zs = p->zsteps[i];
-            StepArgs a = step_args(*p, p->ztensors, zs, c.zws, simt_f64_tile());
-            a.epi.mode = EPI_Z;
-            a.epi.out = zs.final ? (void *)(zslice + sl) : (void *)ws_ptr(c.zws, p->ztensors[zs.c].offset);
-            TQC_CUDA(launch_simt_step_f64(a, s), "total-mass step");
-        }
+    for (int64_t sl = 0; sl < p.n_slices(); ++sl) {
+        std::vector<IngestArgs> leaves;
+        mass_leaves(p, c, sl, &leaves);
+        TQC_CUDA(launch_ingest(leaves.data(), (int)leaves.size(), s), "total-mass ingest");
+        TQC_CUDA(mass_run(p, c, sl, s), "total-mass steps");
     }
-    TQC_CUDA(launch_zfinal(zslice, (int)ns, p->net->n_cuts, !(p->flags & TQC_FLAG_NO_RENORM), c.zinfo, s), "zfinal");
     return TQC_OK;
 }
 
@@ -508,11 +544,16 @@ tqc_status exec_run(Plan &pl, const ExecCtx &c, const uint8_t *fixed_bits, void 
     // ---- total mass Z (scalar network: every output summed), FP64.  Z depends
     // on the tensors only, so the allocating path recomputes it only when they
     // changed since the plan last computed it.
-    if (c.compute_z) {
+    // Unsliced, its leaves are ingested together with the contract's own.
+    std::vector<IngestArgs> leaves;
+    const bool z_leaves = c.compute_z && ns == 1 && p->m > 1;
+    if (z_leaves) {
+        mass_leaves(*p, c, 0, &leaves);
+    } else if (c.compute_z) {
         st = exec_total_mass(*p, c, stream);
         if (st != TQC_OK) return st;
-        if (z_computed) *z_computed = true;
     }
+    if (z_computed) *z_computed = c.compute_z;
 
     // ---- single subcircuit: the bin is a gather of its tensor
     if (p->m == 1) {
@@ -522,7 +563,7 @@ tqc_status exec_run(Plan &pl, const ExecCtx &c, const uint8_t *fixed_bits, void 
         g.scaled = 1;
         g.out_f64 = out_dtype == TQC_F64;
         g.zinfo = c.zinfo;
-        TQC_CUDA(launch_ingest(g, p->out_elems(), s), "ingest");
+        TQC_CUDA(launch_ingest(&g, 1, s), "ingest");
         return TQC_OK;
     }
     const bool sliced = ns > 1;
@@ -538,8 +579,11 @@ tqc_status exec_run(Plan &pl, const ExecCtx &c, const uint8_t *fixed_bits, void 
             g.dst = ws_ptr(c.ws, t.offset);
             if (t.storage == ST_BF16X2) g.dst_lo = ws_ptr(c.ws, t.offset + t.plane_bytes);
             g.storage = t.storage;
-            TQC_CUDA(launch_ingest(g, (int64_t)1 << t.nbits(), s), "ingest");
+            leaves.push_back(g);
         }
+        if (!leaves.empty()) TQC_CUDA(launch_ingest(leaves.data(), (int)leaves.size(), s), "ingest");
+        leaves.clear();
+        if (z_leaves) TQC_CUDA(mass_run(*p, c, 0, s), "total-mass steps");
         for (size_t si = 0; si < p->steps.size(); ++si) {
             const StepPlan sp = step_of(p->steps[si]);
             if (sp.fuse == 2) continue;  // ran inside the previous step's fused kernel

@@ -132,6 +132,8 @@ __global__ void __launch_bounds__(F_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_launch();
+    pdl_wait();
 
     if (warp == 0) {
         // ------------------------------------------------ A0 / B0 copies
@@ -466,8 +468,7 @@ cudaError_t launch_fused_pair(const StepArgs &a0, const StepArgs &a1, uint64_t m
     p.stall = g_fused_stall.load(std::memory_order_relaxed);
     p.err = d_err;
     const int64_t grid = std::min<int64_t>(p.n_units, sm_count());
-    fused_pair_kernel<<<(unsigned)grid, F_THREADS, F_SMEM, s>>>(tA0, tA0l, tB0, tB0l, tB1, tB1l, p);
-    return cudaGetLastError();
+    return launch_pdl(fused_pair_kernel, grid, F_THREADS, F_SMEM, s, tA0, tA0l, tB0, tB0l, tB1, tB1l, p);
 }
 
 }  // namespace tqc

@@ -21,13 +21,34 @@ TileShape simt_tile(int cfg);
 // its tile shape.
 bool smallk_ok(int mb, int nb, int kb, bool kblk);
 TileShape smallk_tile(int mb, int nb, int kb);
-TileShape simt_f64_tile();
 int sm_count();
 
+// Launch a kernel that may start before its predecessor in the stream has
+// ended; it calls pdl_launch and pdl_wait (device_common.cuh) itself.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), int64_t grid, int block, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 cudaError_t launch_simt_step(int cfg, const StepArgs &a, cudaStream_t s);
-cudaError_t launch_simt_step_f64(const StepArgs &a, cudaStream_t s);
-cudaError_t launch_ingest(const IngestArgs &g, int64_t n_dst, cudaStream_t s);
-cudaError_t launch_zfinal(const double *zslice, int n, int n_cuts, int renorm, double *zinfo, cudaStream_t s);
+// Ingest of n leaves (each of 2^nbits elements): one launch per INGEST_MAX of them.
+constexpr int INGEST_MAX = 16;
+cudaError_t launch_ingest(const IngestArgs *g, int n, cudaStream_t s);
+// The steps of one slice's total-mass network, then (zslice given) the sum of
+// the n per-slice masses and the scale.
+cudaError_t launch_znet(const ZStep *steps, int n_steps, const double *zslice, int n, int n_cuts, int renorm,
+                        double *zinfo, cudaStream_t s);
+int znet_launches(const ZStep *steps, int n_steps, bool last);
 cudaError_t launch_finalize(const double *acc, void *out, int out_f64, const double *zinfo, int64_t n,
                             cudaStream_t s);
 // Sum of a K-split step's FP32 partials (split s at part + s * n) into its

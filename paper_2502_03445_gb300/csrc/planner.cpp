@@ -878,11 +878,16 @@ std::string plan_describe(const Plan &pl) {
     for (size_t i = 0; i < p->tensors.size(); ++i) os << (i ? "," : "") << mode_str(p->tensors[i].layout);
     // kernel launches of one contract once the total mass is cached, and of
     // the total-mass network when the tensors changed
-    const int64_t z_launches = ((int64_t)p->m + (int64_t)p->zsteps.size()) * p->n_slices() + 1;
+    const int64_t z_launches = total_mass_launches(*p);
     int64_t launches = 0;
     if (p->m == 1) launches += 1;
     else {
-        for (int j = 0; j < p->m; ++j) launches += p->tensors[j].slice_dep ? p->n_slices() : 1;
+        // one ingest launch per INGEST_MAX leaves: every leaf, then (further
+        // slices) those that depend on a sliced cut
+        int dep = 0;
+        for (int j = 0; j < p->m; ++j) dep += p->tensors[j].slice_dep;
+        launches += (p->m + INGEST_MAX - 1) / INGEST_MAX;
+        launches += (p->n_slices() - 1) * ((dep + INGEST_MAX - 1) / INGEST_MAX);
         for (auto &st : p->steps)  // a K-split step adds its reduce pass; a fused pair is one launch
             if (st.fuse != 2) launches += (p->tensors[st.c].slice_dep ? p->n_slices() : 1) * (st.ksplit > 1 ? 2 : 1);
         if (p->n_slices() > 1) launches += 1;

@@ -48,6 +48,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
     const int tx = tid % (BN / TN), ty = tid / (BN / TN);
     epi_tables_init(tb, e, true, PS, tid, NT);
     const int E = Me * Ne;
+    pdl_launch();
+    pdl_wait();
     for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const int64_t rt = tile / col_tiles, ct = tile - rt * col_tiles;
         const int64_t r0 = rt << a, c0 = ct << b;
@@ -135,6 +137,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / 8), MINB)
     const int tx = (warp % WX) * 8 + (lane & 7), ty = (warp / WX) * 4 + (lane >> 3);
     epi_tables_init(tb, e, true, PS, tid, NT);
     const int gm = gather_mode(e.lowCc);
+    pdl_launch();
+    pdl_wait();
     float4 pa[LA], pb[LB];
     auto load = [&](int64_t tile, int c) {
         const int64_t rt = tile / col_tiles, ct = tile - rt * col_tiles;
@@ -239,133 +243,246 @@ __global__ void __launch_bounds__(128, (QM == 1) == RM ? 8 : 6)
         epi_tables_init(tb, args.epi, true, 0, threadIdx.x, 128);
         __syncthreads();
     }
+    pdl_launch();
+    pdl_wait();
     smallk_tiles_body<KB, QM, RM, false>(args, tb, L, col_tiles, blockIdx.x, n_tiles, gridDim.x, buf, threadIdx.x, 1);
 }
 
-// FP64 twin for the scalar total-mass network (small; one config).
-template <int BM, int BN, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
-    simt_step_f64(StepArgs args, int64_t n_tiles, int64_t col_tiles) {
-    constexpr int NT = (BM / TM) * (BN / TN);
-    constexpr int BK = 16;
-    __shared__ double As[BK * BM], Bs[BK * BN];
-    __shared__ double stage[BM * BN];
-    const EpiParams &e = args.epi;
-    const int a = e.a_bits, b = e.b_bits;
-    const int Me = 1 << a, Ne = 1 << b;
-    const int64_t K = 1ll << args.kb;
-    const int lkc = args.kb < 4 ? args.kb : 4;
-    const int kc = 1 << lkc;
-    const double *A = (const double *)args.A;
-    const double *B = (const double *)args.B;
-    const int tid = threadIdx.x;
-    const int tx = tid % (BN / TN), ty = tid / (BN / TN);
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const int64_t rt = tile / col_tiles, ct = tile - rt * col_tiles;
-        const int64_t r0 = rt << a, c0 = ct << b;
-        double acc[TM][TN];
-        for (int u = 0; u < TM; ++u)
-            for (int v = 0; v < TN; ++v) acc[u][v] = 0.0;
-        for (int64_t k0 = 0; k0 < K; k0 += kc) {
-            for (int idx = tid; idx < (BM << lkc); idx += NT) {
-                int i = idx >> lkc, kk = idx & (kc - 1);
-                As[kk * BM + i] = i < Me ? A[(r0 + i) * K + k0 + kk] : 0.0;
-            }
-            for (int idx = tid; idx < (BN << lkc); idx += NT) {
-                int j = idx >> lkc, kk = idx & (kc - 1);
-                Bs[kk * BN + j] = j < Ne ? B[(c0 + j) * K + k0 + kk] : 0.0;
-            }
-            __syncthreads();
-            for (int kk = 0; kk < kc; ++kk)
-                for (int u = 0; u < TM; ++u)
-                    for (int v = 0; v < TN; ++v)
-                        acc[u][v] = fma(As[kk * BM + ty * TM + u], Bs[kk * BN + tx * TN + v], acc[u][v]);
-            __syncthreads();
+// The total-mass network: FP64 steps over the cut indices alone.  The FP64
+// rate (two multiply-adds a clock per SM) bounds them, so the work is spread
+// over as many SMs as it has outputs for: 2^lkl lanes of a warp share one
+// output (each takes every 2^lkl-th k; a fixed shuffle tree adds their sums).
+__device__ __forceinline__ void zstep_range(const ZStep &z, int64_t warp, int64_t n_warps, int lane) {
+    const int lkl = z.kb < 5 ? z.kb : 5;
+    const int64_t n_out = 1ll << (z.mb + z.nb);
+    const int per = 32 >> lkl;
+    for (int64_t o0 = warp * per; o0 < n_out; o0 += n_warps * per) {
+        const int64_t o = o0 + (lane >> lkl);
+        double acc = 0.0;
+        const int64_t r = o >> z.nb, c = o & ((1ll << z.nb) - 1);
+        if (o < n_out) {
+            const double *A = z.A + (r << z.kb), *B = z.B + (c << z.kb);
+            // written by other SMs of this launch in the cluster form: not through L1
+            for (int64_t k = lane & ((1 << lkl) - 1); k < 1ll << z.kb; k += 1 << lkl)
+                acc = fma(__ldcg(A + k), __ldcg(B + k), acc);
         }
-        for (int u = 0; u < TM; ++u)
-            for (int v = 0; v < TN; ++v) {
-                int i = ty * TM + u, j = tx * TN + v;
-                if (i < Me && j < Ne) stage[pdep32(i, e.lowRc) | pdep32(j, e.lowCc)] = acc[u][v];
-            }
-        __syncthreads();
-        const uint64_t base = tile_base(e, rt, ct);
-        double *o = (double *)e.out;
-        for (int t = tid; t < Me * Ne; t += NT) o[base + pdep64((uint64_t)t, e.tileMask)] = stage[t];
-        __syncthreads();
-    }
-}
-
-// Gather a node tensor into an operand layout: destination bit b reads
-// source bit srcpos[b]; src_base carries the fixed output bits of the bin and
-// the values of sliced cuts.  With reduce_bits > 0 (total mass) one warp sums
-// the 2^reduce_bits consecutive source elements in FP64.
-__global__ void ingest_kernel(IngestArgs g, int64_t n_dst) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    if (g.reduce_bits > 0) {
-        const int lane = threadIdx.x & 31;
-        const int64_t wstride = stride >> 5;
-        const int64_t nx = 1ll << g.reduce_bits;
-        for (int64_t d = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; d < n_dst; d += wstride) {
-            int64_t s = g.src_base;
-            for (int b = 0; b < g.nbits; ++b)
-                if (d >> b & 1) s += 1ll << g.srcpos[b];
-            double acc = 0.0;
-            for (int64_t x = lane; x < nx; x += 32) acc += ld_src<double>(g.src, g.src_dtype, s + x);
-            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) ((double *)g.dst)[d] = acc;
-        }
-        return;
-    }
-    // The grid is a power of two threads (2^lg): a thread's destination
-    // indices share their lg low bits, so their part of the source offset is
-    // summed once and each element adds only its bits from lg up.
-    const int lg = __ffsll((long long)stride) - 1;
-    const int64_t d0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t s_lo = g.src_base;
-    for (int b = 0; b < g.nbits && b < lg; ++b)
-        if (d0 >> b & 1) s_lo += 1ll << g.srcpos[b];
-    for (int64_t d = d0; d < n_dst; d += stride) {
-        int64_t s = s_lo;
-        for (int b = lg; b < g.nbits; ++b)
-            if (d >> b & 1) s += 1ll << g.srcpos[b];
-        if (g.scaled) {
-            double v = ld_src<double>(g.src, g.src_dtype, s) * g.zinfo[1];
-            if (g.out_f64) ((double *)g.dst)[d] = v;
-            else ((float *)g.dst)[d] = (float)v;
-            continue;
-        }
-        const float v = ld_src<float>(g.src, g.src_dtype, s);
-        switch (g.storage) {
-            case ST_F32: ((float *)g.dst)[d] = v; break;
-            case ST_TF32: ((float *)g.dst)[d] = to_tf32(v); break;
-            case ST_BF16: ((__nv_bfloat16 *)g.dst)[d] = __float2bfloat16_rn(v); break;
-            case ST_BF16X2: {
-                // hi = bf16(v), lo = bf16(v - hi) from the FP32 value (v - hi is
-                // exact in FP32); one FP64 conversion per element, which matters
-                // on a part whose FP64 rate is a small fraction of its FP32 rate
-                const __nv_bfloat16 h = __float2bfloat16_rn(v);
-                ((__nv_bfloat16 *)g.dst)[d] = h;
-                ((__nv_bfloat16 *)g.dst_lo)[d] = __float2bfloat16_rn(v - __bfloat162float(h));
-            } break;
-            case ST_F64: ((double *)g.dst)[d] = ld_src<double>(g.src, g.src_dtype, s); break;
-            default: break;
-        }
+        for (int s = 1; s < 1 << lkl; s <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+        if (o < n_out && (lane & ((1 << lkl) - 1)) == 0)
+            z.out[pdep64((uint64_t)r, z.maskR) | pdep64((uint64_t)c, z.maskC)] = acc;
     }
 }
 
 // Z = sum over slices of the scalar network; scale = 2^{-|E|} / Z (or
 // 2^{-|E|} without renormalisation).
+__device__ __forceinline__ void zfinal(const double *zslice, int n, int n_cuts, int renorm, double *zinfo) {
+    double z = 0.0;
+    for (int i = 0; i < n; ++i) z += __ldcg(zslice + i);
+    const double z_scaled = ldexp(z, -n_cuts);  // Z includes the 1/2 per cut
+    zinfo[0] = z_scaled;
+    zinfo[1] = renorm ? ldexp(1.0, -n_cuts) / z_scaled : ldexp(1.0, -n_cuts);
+}
+
+// A whole small network in one launch: a cluster of ZN_CTAS CTAs with a
+// cluster barrier between steps (a launch each took longer than their work:
+// three
+// steps and the sum of a 15-qubit network 41 -> 8.6 us, a 24-qubit one's four
+// 134 -> 21 us, both with the FP64 work on eight SMs, not one).
+constexpr int ZN_CTAS = 8, ZN_MAX = 16, ZN_THREADS = 256;
+constexpr double ZN_MAX_MACS = 1 << 18;  // more: one launch per step, over every SM
+struct ZNetArgs {
+    ZStep step[ZN_MAX];
+    int32_t n_steps;
+    const double *zslice;  // NULL: another slice follows
+    int32_t n, n_cuts, renorm;
+    double *zinfo;
+};
+__global__ void __cluster_dims__(ZN_CTAS, 1, 1) __launch_bounds__(ZN_THREADS)
+    znet_kernel(const __grid_constant__ ZNetArgs a) {
+    pdl_launch();
+    pdl_wait();
+    const int warp = (int)(blockIdx.x * (ZN_THREADS / 32) + (threadIdx.x >> 5));
+    for (int i = 0; i < a.n_steps; ++i) {
+        zstep_range(a.step[i], warp, ZN_CTAS * (ZN_THREADS / 32), threadIdx.x & 31);
+        asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    if (a.zslice && blockIdx.x == 0 && threadIdx.x == 0) zfinal(a.zslice, a.n, a.n_cuts, a.renorm, a.zinfo);
+}
+__global__ void __launch_bounds__(ZN_THREADS) zstep_kernel(const __grid_constant__ ZStep z) {
+    pdl_launch();
+    pdl_wait();
+    zstep_range(z, (int64_t)blockIdx.x * (ZN_THREADS / 32) + (threadIdx.x >> 5),
+                (int64_t)gridDim.x * (ZN_THREADS / 32), threadIdx.x & 31);
+}
 __global__ void zfinal_kernel(const double *zslice, int n, int n_cuts, int renorm, double *zinfo) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double z = 0.0;
-        for (int i = 0; i < n; ++i) z += zslice[i];
-        double z_scaled = ldexp(z, -n_cuts);  // Z includes the 1/2 per cut
-        zinfo[0] = z_scaled;
-        zinfo[1] = renorm ? ldexp(1.0, -n_cuts) / z_scaled : ldexp(1.0, -n_cuts);
+    pdl_launch();
+    pdl_wait();
+    if (threadIdx.x == 0 && blockIdx.x == 0) zfinal(zslice, n, n_cuts, renorm, zinfo);
+}
+
+// FP64 bits -> nearest FP32 (ties to even), the conversion instruction's
+// result, in integer arithmetic for normal results: the instruction runs at
+// the FP64 rate, which held grid30's largest leaf (2^22 elements) to 24 us.
+__device__ __forceinline__ float f64_to_f32(uint64_t b) {
+    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    if (e - 897u > 253u) return (float)__longlong_as_double((long long)b);  // zero, subnormal, overflow, inf, NaN
+    uint32_t u = __funnelshift_l(lo, hi, 3) - (896u << 23);  // exponent rebased (modulo 512), 23 mantissa bits
+    u += ((lo << 3) | (u & 1u)) > 0x80000000u;                // round to nearest even; a carry is right
+    return __uint_as_float(u | (hi & 0x80000000u));
+}
+
+// V source elements from element s on (V > 1: the address is a multiple of V elements).
+template <int V>
+__device__ __forceinline__ void ingest_load(const IngestArgs &g, int64_t s, float (&v)[V]) {
+    if (g.src_dtype == TQC_F64) {
+        const double *p = (const double *)g.src + s;
+        if constexpr (V == 1) {
+            v[0] = f64_to_f32((uint64_t)__double_as_longlong(__ldg(p)));
+        } else {
+#pragma unroll
+            for (int i = 0; i < V; i += 2) {
+                const ulonglong2 q = __ldg((const ulonglong2 *)(p + i));
+                v[i] = f64_to_f32(q.x);
+                v[i + 1] = f64_to_f32(q.y);
+            }
+        }
+    } else {
+        const float *p = (const float *)g.src + s;
+        if constexpr (V == 4) {
+            const float4 q = __ldg((const float4 *)p);
+            v[0] = q.x;
+            v[1] = q.y;
+            v[2] = q.z;
+            v[3] = q.w;
+        } else if constexpr (V == 2) {
+            const float2 q = __ldg((const float2 *)p);
+            v[0] = q.x;
+            v[1] = q.y;
+        } else {
+            v[0] = __ldg(p);
+        }
     }
 }
 
+// Gather a leaf: thread t (of 2^nbits / V) takes V neighbouring source
+// elements, whose destinations differ in bits vb[0] (and vb[1]).  The threads
+// are a power of two (2^lg), so a thread's t share their lg low bits: that
+// part of the source offset is summed once.
+template <int V>
+__device__ __forceinline__ void ingest_gather(const IngestArgs &g, int64_t t0, int lg) {
+    const int nb = g.nbits - (V == 4 ? 2 : (V == 2 ? 1 : 0));  // bits of t: srcpos[0 .. nb)
+    const int64_t n = 1ll << nb, stride = 1ll << lg;
+    int64_t s_lo = g.src_base;
+    for (int b = 0; b < nb && b < lg; ++b)
+        if (t0 >> b & 1) s_lo += 1ll << g.srcpos[b];
+    const int p0 = V == 4 ? (g.vb[0] < g.vb[1] ? g.vb[0] : g.vb[1]) : g.vb[0];
+    const int p1 = V == 4 ? (g.vb[0] < g.vb[1] ? g.vb[1] : g.vb[0]) : 0;
+    const int64_t d1 = 1ll << g.vb[0], d2 = V == 4 ? 1ll << g.vb[1] : 0;
+    for (int64_t t = t0; t < n; t += stride) {
+        int64_t s = s_lo;
+        for (int b = lg; b < nb; ++b)
+            if (t >> b & 1) s += 1ll << g.srcpos[b];
+        int64_t d = t;  // destination of the first: zero bits inserted at vb
+        if (V >= 2) d = ((d >> p0) << (p0 + 1)) | (d & ((1ll << p0) - 1));
+        if (V == 4) d = ((d >> p1) << (p1 + 1)) | (d & ((1ll << p1) - 1));
+        auto at = [&](int i) { return d + ((i & 1) ? d1 : 0) + ((i & 2) ? d2 : 0); };
+        if (g.scaled || g.storage == ST_F64) {
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                const double x = ld_src<double>(g.src, g.src_dtype, s + i);
+                if (!g.scaled) ((double *)g.dst)[at(i)] = x;
+                else if (g.out_f64) ((double *)g.dst)[at(i)] = x * g.zinfo[1];
+                else ((float *)g.dst)[at(i)] = (float)(x * g.zinfo[1]);
+            }
+            continue;
+        }
+        float v[V];
+        ingest_load<V>(g, s, v);
+        switch (g.storage) {
+            case ST_F32:
+#pragma unroll
+                for (int i = 0; i < V; ++i) ((float *)g.dst)[at(i)] = v[i];
+                break;
+            case ST_TF32:
+#pragma unroll
+                for (int i = 0; i < V; ++i) ((float *)g.dst)[at(i)] = to_tf32(v[i]);
+                break;
+            case ST_BF16:
+#pragma unroll
+                for (int i = 0; i < V; ++i) ((__nv_bfloat16 *)g.dst)[at(i)] = __float2bfloat16_rn(v[i]);
+                break;
+            case ST_BF16X2:
+                // hi = bf16(v), lo = bf16(v - hi) from the FP32 value (v - hi is exact in FP32)
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    const __nv_bfloat16 h = __float2bfloat16_rn(v[i]);
+                    ((__nv_bfloat16 *)g.dst)[at(i)] = h;
+                    ((__nv_bfloat16 *)g.dst_lo)[at(i)] = __float2bfloat16_rn(v[i] - __bfloat162float(h));
+                }
+                break;
+            default: break;
+        }
+    }
+}
+
+// Node tensors into operand layouts (every leaf of a contract in one launch:
+// CTAs blk[j] .. blk[j + 1] take leaf j): destination bit b reads source bit
+// srcpos[b]; src_base carries the fixed output bits of the bin and the values
+// of sliced cuts.  A leaf's lowest destination bits are cuts, its lowest
+// source bits output qubits, so a thread loads four neighbouring source
+// elements (a whole sector of FP64) and the warp's stores are consecutive.
+// With reduce_bits > 0 (total mass) the 2^reduce_bits consecutive source
+// elements of a destination are summed in FP64, by a warp or (few
+// destinations) by a CTA.  Grid30's four leaves (4.8 M
+// FP64 elements): four launches of 41 us in all -> one of 20 us.
+constexpr int INGEST_THREADS = 256;
+struct IngestMulti {
+    int32_t n;
+    int32_t blk[INGEST_MAX + 1];
+    IngestArgs g[INGEST_MAX];
+};
+__global__ void __launch_bounds__(INGEST_THREADS) ingest_kernel(const __grid_constant__ IngestMulti m) {
+    __shared__ double part[INGEST_THREADS / 32];
+    pdl_launch();
+    pdl_wait();
+    int j = 0;
+    while ((int)blockIdx.x >= m.blk[j + 1]) ++j;
+    const IngestArgs &g = m.g[j];
+    const int blocks = m.blk[j + 1] - m.blk[j], block = (int)blockIdx.x - m.blk[j];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (g.reduce_bits > 0) {
+        const bool cta = g.vec == INGEST_THREADS;  // threads per destination
+        const int64_t nx = 1ll << g.reduce_bits, n_dst = 1ll << g.nbits;
+        const int64_t w0 = cta ? block : (int64_t)block * (INGEST_THREADS / 32) + warp;
+        for (int64_t d = w0; d < n_dst; d += cta ? blocks : (int64_t)blocks * (INGEST_THREADS / 32)) {
+            int64_t s = g.src_base;
+            for (int b = 0; b < g.nbits; ++b)
+                if (d >> b & 1) s += 1ll << g.srcpos[b];
+            double acc = 0.0;
+            for (int64_t x = cta ? (int64_t)threadIdx.x : lane; x < nx; x += cta ? INGEST_THREADS : 32)
+                acc += ld_src<double>(g.src, g.src_dtype, s + x);
+            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (cta) {
+                if (lane == 0) part[warp] = acc;
+                __syncthreads();
+                acc = 0.0;
+                for (int w = 0; w < INGEST_THREADS / 32; ++w) acc += part[w];
+                __syncthreads();
+            }
+            if (cta ? threadIdx.x == 0 : lane == 0) ((double *)g.dst)[d] = acc;
+        }
+        return;
+    }
+    const int lg = __ffs(blocks * INGEST_THREADS) - 1;
+    const int64_t t0 = (int64_t)block * INGEST_THREADS + threadIdx.x;
+    if (g.vec == 4) ingest_gather<4>(g, t0, lg);
+    else if (g.vec == 2) ingest_gather<2>(g, t0, lg);
+    else ingest_gather<1>(g, t0, lg);
+}
+
 __global__ void finalize_kernel(const double *acc, void *out, int out_f64, const double *zinfo, int64_t n) {
+    pdl_launch();
+    pdl_wait();
     const double s = zinfo[1];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -380,6 +497,8 @@ __global__ void finalize_kernel(const double *acc, void *out, int out_f64, const
 // (FP32 / FP64) or the FP64 slice sum (set / add).
 __global__ void ksplit_reduce_kernel(const float *part, int ksplit, int64_t n, int mode, void *out,
                                      const double *zinfo) {
+    pdl_launch();
+    pdl_wait();
     const double sc = (mode == EPI_OUT_F32 || mode == EPI_OUT_F64) ? zinfo[1] : 1.0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -414,8 +533,7 @@ cudaError_t launch_cfg(const StepArgs &a, cudaStream_t s) {
     int64_t col_tiles = 1ll << (a.nb - a.epi.b_bits);
     int64_t n_tiles = row_tiles * col_tiles;
     int64_t grid = std::min<int64_t>(n_tiles, (int64_t)sm_count() * 16);
-    simt_step_f32<BM, BN, TM, TN, BK><<<(unsigned)grid, NT, smem, s>>>(a, n_tiles, col_tiles);
-    return cudaGetLastError();
+    return launch_pdl(simt_step_f32<BM, BN, TM, TN, BK>, grid, NT, smem, s, a, n_tiles, col_tiles);
 }
 
 // The tile configurations of K >= 16 steps whose tiles are whole.
@@ -433,8 +551,7 @@ cudaError_t launch_gemm(const StepArgs &a, cudaStream_t s) {
     const int64_t col_tiles = 1ll << (a.nb - a.epi.b_bits);
     const int64_t n_tiles = (1ll << (a.mb - a.epi.a_bits)) * col_tiles;
     const int64_t grid = std::min<int64_t>(n_tiles, (int64_t)sm_count() * MINB);
-    simt_gemm_f32<BM, BN, TM, MINB><<<(unsigned)grid, NT, smem, s>>>(a, n_tiles, col_tiles);
-    return cudaGetLastError();
+    return launch_pdl(simt_gemm_f32<BM, BN, TM, MINB>, grid, NT, smem, s, a, n_tiles, col_tiles);
 }
 
 }  // namespace
@@ -457,7 +574,6 @@ TileShape simt_tile(int cfg) {
     }
 }
 
-TileShape simt_f64_tile() { return {5, 5}; }
 
 bool smallk_ok(int mb, int nb, int kb, bool kblk) {
     return (kb == 0 || kb == 2 || kb == 4) && !kblk && mb >= 2 && nb >= 2 && mb + nb >= 7;
@@ -561,8 +677,7 @@ cudaError_t launch_smallk(const StepArgs &a, cudaStream_t s) {
             if (err != cudaSuccess) return err;                                                              \
             done = true;                                                                                     \
         }                                                                                                    \
-        simt_smallk_f32<KBV, QMV, RMV><<<grid, 128, smem, s>>>(a, n_tiles, col_tiles, L);                    \
-        return cudaGetLastError();                                                                           \
+        return launch_pdl(simt_smallk_f32<KBV, QMV, RMV>, grid, 128, smem, s, a, n_tiles, col_tiles, L);      \
     }
     TQC_SMALLK_LAUNCH(0, 1, true)
     TQC_SMALLK_LAUNCH(0, 1, false)
@@ -595,36 +710,97 @@ cudaError_t launch_simt_step(int cfg, const StepArgs &a, cudaStream_t s) {
     }
 }
 
-cudaError_t launch_simt_step_f64(const StepArgs &a, cudaStream_t s) {
-    int64_t row_tiles = 1ll << (a.mb - a.epi.a_bits);
-    int64_t col_tiles = 1ll << (a.nb - a.epi.b_bits);
-    int64_t n_tiles = row_tiles * col_tiles;
-    int64_t grid = std::min<int64_t>(n_tiles, (int64_t)sm_count() * 8);
-    simt_step_f64<32, 32, 2, 2><<<(unsigned)grid, 256, 0, s>>>(a, n_tiles, col_tiles);
-    return cudaGetLastError();
+namespace {
+
+double znet_macs(const ZStep *z, int n) {
+    double t = 0;
+    for (int i = 0; i < n; ++i) t += (double)(1ull << (z[i].mb + z[i].nb + z[i].kb));
+    return t;
+}
+bool znet_small(const ZStep *z, int n) { return n <= ZN_MAX && znet_macs(z, n) <= ZN_MAX_MACS; }
+
+}  // namespace
+
+cudaError_t launch_znet(const ZStep *z, int n_steps, const double *zslice, int n, int n_cuts, int renorm,
+                        double *zinfo, cudaStream_t s) {
+    if (znet_small(z, n_steps)) {
+        ZNetArgs a = {};
+        for (int i = 0; i < n_steps; ++i) a.step[i] = z[i];
+        a.n_steps = n_steps;
+        a.zslice = zslice;
+        a.n = n;
+        a.n_cuts = n_cuts;
+        a.renorm = renorm;
+        a.zinfo = zinfo;
+        return launch_pdl(znet_kernel, ZN_CTAS, ZN_THREADS, 0, s, a);
+    }
+    for (int i = 0; i < n_steps; ++i) {
+        const int lkl = std::min(z[i].kb, 5);
+        const int64_t warps = std::max<int64_t>(1, (1ll << (z[i].mb + z[i].nb)) >> (5 - lkl));
+        const int64_t blocks = std::min<int64_t>((warps + ZN_THREADS / 32 - 1) / (ZN_THREADS / 32), (int64_t)sm_count() * 8);
+        const cudaError_t e = launch_pdl(zstep_kernel, blocks, ZN_THREADS, 0, s, z[i]);
+        if (e != cudaSuccess) return e;
+    }
+    return zslice ? launch_pdl(zfinal_kernel, 1, 32, 0, s, zslice, n, n_cuts, renorm, zinfo) : cudaSuccess;
 }
 
-cudaError_t launch_ingest(const IngestArgs &g, int64_t n_dst, cudaStream_t s) {
-    int64_t threads = g.reduce_bits > 0 ? n_dst * 32 : n_dst;
-    int64_t blocks = std::min<int64_t>((threads + 255) / 256, (int64_t)sm_count() * 32);
-    if (blocks < 1) blocks = 1;
-    // a power of two (the gather's stride; see ingest_kernel)
-    while (blocks & (blocks - 1)) blocks &= blocks - 1;
-    ingest_kernel<<<(unsigned)blocks, 256, 0, s>>>(g, n_dst);
-    return cudaGetLastError();
+int znet_launches(const ZStep *z, int n_steps, bool last) {
+    return znet_small(z, n_steps) ? 1 : n_steps + (last ? 1 : 0);
 }
 
-cudaError_t launch_zfinal(const double *zslice, int n, int n_cuts, int renorm, double *zinfo, cudaStream_t s) {
-    zfinal_kernel<<<1, 32, 0, s>>>(zslice, n, n_cuts, renorm, zinfo);
-    return cudaGetLastError();
+// Largest V <= 4 whose source bits 0 .. log2 V - 1 are destination bits, with
+// the tensor aligned for the loads (16 bytes at most).
+static void ingest_vec(IngestArgs &g) {
+    g.vec = 1;
+    if (g.scaled || g.storage == ST_F64) return;
+    int at[2] = {-1, -1};
+    for (int b = 0; b < g.nbits; ++b)
+        if (g.srcpos[b] < 2) at[(int)g.srcpos[b]] = b;
+    const int esz = g.src_dtype == TQC_F64 ? 8 : 4;
+    auto aligned = [&](int v) { return ((uintptr_t)g.src % (uintptr_t)std::min(16, v * esz)) == 0; };
+    const int v = at[0] >= 0 && at[1] >= 0 && aligned(4) ? 4 : (at[0] >= 0 && aligned(2) ? 2 : 1);
+    if (v == 1) return;
+    int n = 0;
+    int8_t pos[64] = {0};
+    for (int b = 0; b < g.nbits; ++b)
+        if (b != at[0] && !(v == 4 && b == at[1])) pos[n++] = g.srcpos[b];
+    std::copy(pos, pos + 64, g.srcpos);
+    g.vec = v;
+    g.vb[0] = (int8_t)at[0];
+    g.vb[1] = (int8_t)(v == 4 ? at[1] : 0);
+}
+
+cudaError_t launch_ingest(const IngestArgs *g, int n, cudaStream_t s) {
+    for (int i = 0; i < n; i += INGEST_MAX) {
+        IngestMulti m = {};
+        m.n = std::min(n - i, INGEST_MAX);
+        for (int j = 0; j < m.n; ++j) {
+            IngestArgs &a = m.g[j] = g[i + j];
+            int64_t threads;
+            if (a.reduce_bits > 0) {
+                // a CTA per destination when a warp each would leave SMs idle
+                a.vec = a.nbits < 10 && a.reduce_bits >= 8 ? INGEST_THREADS : 32;
+                threads = a.vec << a.nbits;
+            } else {
+                ingest_vec(a);
+                threads = (1ll << a.nbits) / a.vec;
+            }
+            int64_t blocks = std::min<int64_t>((threads + INGEST_THREADS - 1) / INGEST_THREADS, (int64_t)sm_count() * 32);
+            if (blocks < 1) blocks = 1;
+            while (blocks & (blocks - 1)) blocks &= blocks - 1;  // a power of two (ingest_gather)
+            m.blk[j + 1] = m.blk[j] + (int)blocks;
+        }
+        const cudaError_t e = launch_pdl(ingest_kernel, m.blk[m.n], INGEST_THREADS, 0, s, m);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_finalize(const double *acc, void *out, int out_f64, const double *zinfo, int64_t n,
                             cudaStream_t s) {
     int64_t blocks = std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 32);
     if (blocks < 1) blocks = 1;
-    finalize_kernel<<<(unsigned)blocks, 256, 0, s>>>(acc, out, out_f64, zinfo, n);
-    return cudaGetLastError();
+    return launch_pdl(finalize_kernel, blocks, 256, 0, s, acc, out, out_f64, zinfo, n);
 }
 
 cudaError_t launch_ksplit_reduce(const float *part, int ksplit, int64_t n, int mode, void *out, const double *zinfo,
@@ -633,8 +809,7 @@ cudaError_t launch_ksplit_reduce(const float *part, int ksplit, int64_t n, int m
     if (mode != EPI_OUT_F32 && mode != EPI_OUT_F64 && mode != EPI_F64_SET && mode != EPI_F64_ADD)
         return cudaErrorInvalidValue;
     const int64_t blocks = std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 32);
-    ksplit_reduce_kernel<<<(unsigned)blocks, 256, 0, s>>>(part, ksplit, n, mode, out, zinfo);
-    return cudaGetLastError();
+    return launch_pdl(ksplit_reduce_kernel, blocks, 256, 0, s, part, ksplit, n, mode, out, zinfo);
 }
 
 EpiParams make_epi(uint64_t maskR, uint64_t maskC, int mb, int nb, TileShape t) {

@@ -931,6 +931,7 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
                 p->tab_bytes = need;
             }
             p->tab_off = toff;
+            std::vector<IngestArgs> leaves;
             for (int j = 0; j < p->m; ++j) {
                 const Node &nd = p->net->nodes[j];
                 const TensorPlan &t = p->tensors[j];
@@ -947,9 +948,10 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
                 g.nbits = b;
                 g.dst = (char *)p->d_tab + toff[(size_t)j];
                 g.storage = ST_F32;
-                cudaError_t e = launch_ingest(g, (int64_t)1 << b, s);
-                if (e != cudaSuccess) return cuda_fail(e, "state-list table");
+                leaves.push_back(g);
             }
+            cudaError_t e = launch_ingest(leaves.data(), p->m, s);
+            if (e != cudaSuccess) return cuda_fail(e, "state-list table");
             p->tab_version = p->net->version;
         }
         for (int j = 0; j < p->m; ++j) P.leaf[j].table = (const float *)((char *)p->d_tab + p->tab_off[(size_t)j]);

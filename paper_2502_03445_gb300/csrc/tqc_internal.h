@@ -217,6 +217,8 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
 int states_fused_floats(const Plan &p);
 // Total mass Z into c.zinfo (and the output scale), stream-ordered.
 tqc_status exec_total_mass(const Plan &p, const ExecCtx &c, void *stream);
+// Kernel launches of exec_total_mass.
+int total_mass_launches(const Plan &p);
 // Device source bit positions of a node tensor: output qubit q, cut c (-1 if absent).
 int exec_src_pos_qubit(const Node &nd, int q);
 int exec_src_pos_cut(const Node &nd, int c);
@@ -280,6 +282,19 @@ struct IngestArgs {
     int32_t out_f64 = 0;
     const double *zinfo = nullptr;
     int32_t reduce_bits = 0;     // > 0: sum over the 2^reduce_bits low source elements (Z)
+    // set by the launch: source elements loaded together (1, 2 or 4: source
+    // bits 0 and 1 are destination bits vb[0], vb[1], then left out of srcpos)
+    int32_t vec = 1;
+    int8_t vb[2] = {0, 0};
+};
+
+// A step of the total-mass network: C[r, c] = sum_k A[r, k] B[c, k], FP64,
+// element (r, c) at pdep(r, maskR) | pdep(c, maskC) of out.
+struct ZStep {
+    const double *A = nullptr, *B = nullptr;
+    double *out = nullptr;
+    int32_t mb = 0, nb = 0, kb = 0;
+    uint64_t maskR = 0, maskC = 0;
 };
 
 }  // namespace tqc

@@ -151,6 +151,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (threadIdx.x == 64) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tA) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tB) : "memory");
+        if (KIND == K_BF16X3) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tAl) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tBl) : "memory");
+        }
+    }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"((uint32_t)C::TMEM_COLS)
@@ -162,12 +170,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const EpiParams &e = P.epi;
+    pdl_launch();
+    pdl_wait();
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
         if (lane == 0) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tA) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tB) : "memory");
             int64_t it = 0;
             bool ok = true, skipped0 = false;
             if (bres) {  // the one B tile, loaded once
@@ -597,8 +605,7 @@ cudaError_t launch_kind(const StepArgs &a, int *d_err, cudaStream_t s) {
     p.err = d_err;
     p.stall = g_umma_stall.load(std::memory_order_relaxed);
     const int64_t grid = std::min<int64_t>(p.n_units, sm_count());
-    umma_step_kernel<BN, KIND, DEEP><<<(unsigned)grid, NTHREADS, C::SMEM, s>>>(tA, tB, tAl, tBl, p);
-    return cudaGetLastError();
+    return launch_pdl(umma_step_kernel<BN, KIND, DEEP>, grid, NTHREADS, C::SMEM, s, tA, tB, tAl, tBl, p);
 }
 
 template <int BN, bool DEEP>

@@ -3,10 +3,9 @@
 // Step 1 runs on the device: for every output state i of subcircuit C_j, the
 // L2 norm of its entries over all cut assignments e,
 //     ||p_{j,i}|| = sqrt(sum_e T_j[e][i]^2),
-// a column reduction of the [4^c][2^o] node tensor (FP64 partial sums, split
-// over e when 2^o alone cannot fill the GPU, and then added in a fixed order,
-// so equal tensors give bit-identical norms and ties resolve the same way on
-// every call).  Step 2 (seed each subcircuit
+// a column reduction of the [4^c][2^o] node tensor (FP64 sums in a fixed
+// order, so equal tensors give bit-identical norms and ties resolve the same
+// way on every call).  Step 2 (seed each subcircuit
 // with its heaviest state, then add states in descending norm until the
 // product of the per-subcircuit counts reaches s_max) orders a few thousand
 // numbers and runs on the host.  The selected states become a new network
@@ -32,36 +31,66 @@ struct tqc_net {
 namespace tqc {
 namespace {
 
-// part[y][x] = sum_{e in [e0, e1)} T[e][x]^2 for split y = blockIdx.y
-__global__ void hss_sum2_kernel(const void *T, int dtype, int64_t n_x, int64_t e_per, int64_t n_e, double *part) {
-    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= n_x) return;
-    const int64_t e0 = (int64_t)blockIdx.y * e_per;
-    const int64_t e1 = e0 + e_per < n_e ? e0 + e_per : n_e;
+// norm[x] = sqrt(sum_e T[e][x]^2) in one launch.  A CTA takes 2^lx states per
+// warp (32, or all of fewer) and, in its eight warps, wr row groups times
+// 8 / wr groups of states; the rows are further split over a cluster of
+// gridDim.y CTAs, whose sums the first one reads through distributed shared
+// memory.  Every sum is formed in a fixed order: lane, row group, cluster
+// rank.  Bound by the tensor's bytes and, as closely, by the FP64 rate (two
+// multiply-adds a clock per SM).  The four tensors of the
+// 30-qubit grid (38 MB) in four calls: 151 -> 55 us (the sums of up to 586
+// partial sums per state were a serial chain in one thread of a second kernel).
+template <typename V>
+__global__ void __launch_bounds__(256)
+    hss_norms_kernel(const V *__restrict__ T, int64_t n_x, int64_t n_e, int lx, int wr, double *norm) {
+    __shared__ double part[8][32];
+    __shared__ double tot[256];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = warp & (wr - 1), wx = warp / wr;               // row group; group of states
+    const int64_t x0 = ((int64_t)blockIdx.x * (8 / wr) + wx) << lx;
+    const int64_t x = x0 + (lane & ((1 << lx) - 1));
+    const int64_t rows = (int64_t)gridDim.y * wr << (5 - lx);    // rows apart
     double acc = 0.0;
-    if (dtype == TQC_F64) {
-        const double *t = (const double *)T;
-        for (int64_t e = e0; e < e1; ++e) {
-            const double v = t[e * n_x + x];
-            acc += v * v;
+    if (x < n_x) {
+        const V *p = T + x;
+        const int64_t e0 = (((int64_t)blockIdx.y * wr + g) << (5 - lx)) + (lane >> lx);
+        int64_t e = e0;
+        for (; e + 15 * rows < n_e; e += 16 * rows) {  // sixteen loads in flight
+            V v[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = __ldg(p + (e + i * rows) * n_x);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) acc += (double)v[i] * (double)v[i];
         }
-    } else {
-        const float *t = (const float *)T;
-        for (int64_t e = e0; e < e1; ++e) {
-            const double v = (double)t[e * n_x + x];
+        for (; e < n_e; e += rows) {
+            const double v = (double)__ldg(p + e * n_x);
             acc += v * v;
         }
     }
-    part[(int64_t)blockIdx.y * n_x + x] = acc;
-}
-
-// norm[x] = sqrt(sum over the splits, in ascending order, of part[y][x])
-__global__ void hss_sqrt_kernel(const double *part, int64_t splits, double *norm, int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        double v = 0.0;
-        for (int64_t y = 0; y < splits; ++y) v += part[y * n + i];
-        norm[i] = sqrt(v);
+    for (int o = 1 << lx; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    part[warp][lane] = acc;
+    __syncthreads();
+    if (g == 0) {
+        double t = 0.0;
+        for (int w = 0; w < wr; ++w) t += part[wx * wr + w][lane];
+        tot[wx * 32 + lane] = t;
     }
+    if (gridDim.y > 1)
+        asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (blockIdx.y == 0 && g == 0 && x < n_x && lane < 1 << lx) {
+        double t = tot[wx * 32 + lane];
+        const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&tot[wx * 32 + lane]);
+        for (uint32_t r = 1; r < gridDim.y; ++r) {
+            uint32_t at;
+            double v;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(mine), "r"(r));
+            asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(at) : "memory");
+            t += v;
+        }
+        norm[x] = sqrt(t);
+    }
+    if (gridDim.y > 1)  // the other CTAs' shared memory stays until it has been read
+        asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // out[e][r] = r < count ? T[e][states[r]] : 0   (r < 2^k)
@@ -76,29 +105,32 @@ __global__ void hss_gather_kernel(const V *T, int64_t n_x, int64_t n_e, const in
     }
 }
 
+template <typename V>
+cudaError_t launch_norms(const Node &nd, double *d_norms, cudaStream_t s) {
+    const int64_t n_x = (int64_t)1 << nd.out_qubits.size(), n_e = (int64_t)1 << (2 * nd.cut_ids.size());
+    const int lx = (int)std::min<size_t>(5, nd.out_qubits.size());
+    const int wr = (int)std::min<int64_t>(8, n_e);  // 1, 4 or 8
+    // up to eight CTAs share the rows, while a lane has at least eight of them
+    int ys = 1;
+    while (ys < 8 && n_e >= ((int64_t)16 * wr * ys << (5 - lx))) ys *= 2;
+    const int64_t per = (int64_t)(8 / wr) << lx;  // states of a CTA
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((n_x + per - 1) / per), (unsigned)ys);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 1;
+    at.val.clusterDim.y = (unsigned)ys;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, hss_norms_kernel<V>, (const V *)nd.d_data, n_x, n_e, lx, wr, d_norms);
+}
+
 tqc_status node_norms(const Node &nd, double *d_norms, cudaStream_t s) {
-    const int64_t n_x = (int64_t)1 << nd.out_qubits.size();
-    const int64_t n_e = (int64_t)1 << (2 * nd.cut_ids.size());
-    const int threads = 256;
-    const int64_t xb = (n_x + threads - 1) / threads;
-    // split the cut assignments so that about four CTAs per SM run
-    int64_t ys = std::max<int64_t>(1, std::min<int64_t>(n_e, (4ll * sm_count() + xb - 1) / xb));
-    ys = std::min<int64_t>(ys, 65535);
-    const int64_t e_per = (n_e + ys - 1) / ys;
-    ys = (n_e + e_per - 1) / e_per;
-    if (xb > 2147483647ll) return fail(TQC_ERR_UNSUPPORTED, "hss: too many output states");
-    // one split: the partial sums are the norms' squares, in place; several:
-    // stream-ordered scratch of splits x 2^o partial sums (at most a few MB)
-    double *part = d_norms;
-    if (ys > 1 && cudaMallocAsync((void **)&part, sizeof(double) * (size_t)(ys * n_x), s) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(TQC_ERR_OOM, "hss: partial sums");
-    }
-    hss_sum2_kernel<<<dim3((unsigned)xb, (unsigned)ys), threads, 0, s>>>(nd.d_data, nd.dtype, n_x, e_per, n_e, part);
-    const int64_t sb = std::min<int64_t>((n_x + threads - 1) / threads, 16ll * sm_count());
-    hss_sqrt_kernel<<<(unsigned)sb, threads, 0, s>>>(part, ys, d_norms, n_x);
-    cudaError_t e = cudaGetLastError();
-    if (ys > 1) cudaFreeAsync(part, s);
+    if (nd.out_qubits.size() > 35) return fail(TQC_ERR_UNSUPPORTED, "hss: too many output states");
+    const cudaError_t e = nd.dtype == TQC_F64 ? launch_norms<double>(nd, d_norms, s) : launch_norms<float>(nd, d_norms, s);
     if (e != cudaSuccess) return fail(TQC_ERR_CUDA, "hss: norm kernels");
     return TQC_OK;
 }

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "launch.h"
+#include "smallk.cuh"
 #include "tqc_internal.h"
 
 namespace tqc {
@@ -221,7 +222,16 @@ int default_step_tile(const StepPlan &st, int out_esize, bool smallk) {
         }
         return st.nb >= 7 ? UMMA_128x128 : UMMA_128x64;
     }
-    if (smallk && smallk_ok(st.mb, st.nb, st.kb, st.kblk)) return SIMT_SMALLK;
+    if (smallk && smallk_ok(st.mb, st.nb, st.kb, st.kblk)) {
+        // K = 16 over enough 128 x 128 tiles for every SM, staged: 8 x 8 results
+        // per thread (simt_gemm_f32) halve the small-K tile's shared-memory loads
+        // (2^16 x 2^12 results, scrambled bits: 382 -> 343 us; stored directly
+        // the small-K tile is the faster one, 309 against 409 us)
+        if (st.kb == 4 && st.mb >= 7 && st.nb >= 7 && ((int64_t)1 << (st.mb + st.nb)) >= ((int64_t)sm_count() << 14) &&
+            !smallk_layout(make_epi(st.maskR, st.maskC, st.mb, st.nb, simt_tile(SIMT_128x128))).direct)
+            return SIMT_128x128;
+        return SIMT_SMALLK;
+    }
     // K >= 16: too few 128 x 128 tiles to give every SM one run as 64 x 64
     // (four times the CTAs, a quarter of a tile's latency: a 17-qubit FP32
     // contract 242 -> 72 us together with simt_gemm_f32)

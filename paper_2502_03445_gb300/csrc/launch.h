@@ -44,6 +44,7 @@ cudaError_t launch_simt_step(int cfg, const StepArgs &a, cudaStream_t s);
 // Ingest of n leaves (each of 2^nbits elements): one launch per INGEST_MAX of them.
 constexpr int INGEST_MAX = 16;
 cudaError_t launch_ingest(const IngestArgs *g, int n, cudaStream_t s);
+void ingest_vec(IngestArgs &g);  // sets vec, vb and the shortened srcpos
 // The steps of one slice's total-mass network, then (zslice given) the sum of
 // the n per-slice masses and the scale.
 cudaError_t launch_znet(const ZStep *steps, int n_steps, const double *zslice, int n, int n_cuts, int renorm,

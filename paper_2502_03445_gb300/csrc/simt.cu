@@ -13,17 +13,13 @@
 #include <algorithm>
 
 #include "device_common.cuh"
+#include "ingest.cuh"
 #include "launch.h"
 #include "smallk.cuh"
 
 namespace tqc {
 
 namespace {
-
-template <typename T>
-__device__ __forceinline__ T ld_src(const void *p, int dtype, int64_t i) {
-    return dtype == TQC_F64 ? (T)((const double *)p)[i] : (T)((const float *)p)[i];
-}
 
 // One tile per iteration of a grid-stride loop over tiles.
 template <int BM, int BN, int TM, int TN, int BK>
@@ -120,10 +116,9 @@ __device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) {
 // per thread (fewer loads, half the warps): 0.42, 0.77 and 0.90 ms.
 template <int BM, int BN, int TM, int MINB>
 __global__ void __launch_bounds__((BM / TM) * (BN / 8), MINB)
-    simt_gemm_f32(StepArgs args, int64_t n_tiles, int64_t col_tiles) {
+    simt_gemm_f32(StepArgs args, int64_t n_tiles, int64_t col_tiles, SmallkLayout L) {
     constexpr int NX = BN / 8, NY = BM / TM, NT = NX * NY, BK = 16;
     constexpr int LA = BM * BK / 4 / NT, LB = BN * BK / 4 / NT;  // 16-byte pieces per thread and chunk
-    constexpr int PS = BN + 4;
     constexpr int BUF = BK * (BM + BN);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     EpiTables *tb = (EpiTables *)smem_raw;
@@ -135,8 +130,22 @@ __global__ void __launch_bounds__((BM / TM) * (BN / 8), MINB)
     // a warp covers 4 x 8 threads: rows 4 ty + 4 NY u, columns 4 tx + 4 NX v
     constexpr int WX = NX / 8;
     const int tx = (warp % WX) * 8 + (lane & 7), ty = (warp / WX) * 4 + (lane >> 3);
-    epi_tables_init(tb, e, true, PS, tid, NT);
-    const int gm = gather_mode(e.lowCc);
+    if (!L.direct) epi_tables_init(tb, e, true, 0, tid, NT);  // the gather's element offsets
+    // the thread's row and column quads: element offsets in the tile (direct
+    // stores), or bits of the tile's destination order (staged)
+    constexpr int QM = TM / 4, QN = 2;
+    const uint64_t mR = pdep64(e.lowRc, e.tileMask), mC = pdep64(e.lowCc, e.tileMask);
+    uint64_t gr[QM], gc[QN];
+#pragma unroll
+    for (int u = 0; u < QM; ++u) {
+        const uint32_t r = 4 * ty + 4 * NY * u;
+        gr[u] = L.direct ? pdep64(r, mR) : pdep32(r, e.lowRc);
+    }
+#pragma unroll
+    for (int v = 0; v < QN; ++v) {
+        const uint32_t c = 4 * tx + 4 * NX * v;
+        gc[v] = L.direct ? pdep64(c, mC) : pdep32(c, e.lowCc);
+    }
     pdl_launch();
     pdl_wait();
     float4 pa[LA], pb[LB];
@@ -216,17 +225,55 @@ __global__ void __launch_bounds__((BM / TM) * (BN / 8), MINB)
         }
         // the next tile's first chunk arrives during the write-out
         if (tile + gridDim.x < n_tiles) load(tile + gridDim.x, 0);
-        __syncthreads();
-        float *stg = buf;
+        float r[TM][8];
 #pragma unroll
         for (int u = 0; u < TM; ++u)
 #pragma unroll
-            for (int v = 0; v < 2; ++v)
-                *(ulonglong2 *)&stg[(4 * ty + 4 * NY * (u >> 2) + (u & 3)) * PS + 4 * tx + 4 * NX * v] =
-                    make_ulonglong2(acc[u][2 * v], acc[u][2 * v + 1]);
-        __syncthreads();
-        epi_readout(tb, stg, e, tile_base(e, rt, ct), BM * BN, tid, NT, gm);
-        __syncthreads();
+            for (int v = 0; v < 4; ++v) {
+                r[u][2 * v] = __uint_as_float((uint32_t)acc[u][v]);
+                r[u][2 * v + 1] = __uint_as_float((uint32_t)(acc[u][v] >> 32));
+            }
+        const uint64_t base = tile_base(e, rt, ct);
+        __syncthreads();  // the operands are read: the next tile's, or the staged results, may overwrite them
+        if (L.direct) {
+            const double sd = (e.mode == EPI_OUT_F32 || e.mode == EPI_OUT_F64) ? e.zinfo[1] : 1.0;
+            const float sf = (float)sd;
+#define TQC_GEMM_DIRECT(M)                                                                  \
+    case M:                                                                                 \
+        if (L.rowmajor) sk_direct_store<M, QM, QN, true>(e, r, base, gr, gc, mR, mC, sf, sd); \
+        else sk_direct_store<M, QM, QN, false>(e, r, base, gr, gc, mR, mC, sf, sd);         \
+        break;
+            switch (e.mode) {
+                TQC_GEMM_DIRECT(EPI_F32)
+                TQC_GEMM_DIRECT(EPI_TF32)
+                TQC_GEMM_DIRECT(EPI_BF16)
+                TQC_GEMM_DIRECT(EPI_BF16X2)
+                TQC_GEMM_DIRECT(EPI_F64_SET)
+                TQC_GEMM_DIRECT(EPI_F64_ADD)
+                TQC_GEMM_DIRECT(EPI_OUT_F32)
+                TQC_GEMM_DIRECT(EPI_OUT_F64)
+                default: break;
+            }
+#undef TQC_GEMM_DIRECT
+        } else {
+            sk_stage<QM, QN>(buf, r, L, gr, gc);
+            __syncthreads();
+#define TQC_GEMM_GATHER(M) \
+    case M: sk_gather<M, NT>(tb, buf, e, base, BM * BN, tid); break;
+            switch (e.mode) {
+                TQC_GEMM_GATHER(EPI_F32)
+                TQC_GEMM_GATHER(EPI_TF32)
+                TQC_GEMM_GATHER(EPI_BF16)
+                TQC_GEMM_GATHER(EPI_BF16X2)
+                TQC_GEMM_GATHER(EPI_F64_SET)
+                TQC_GEMM_GATHER(EPI_F64_ADD)
+                TQC_GEMM_GATHER(EPI_OUT_F32)
+                TQC_GEMM_GATHER(EPI_OUT_F64)
+                default: break;
+            }
+#undef TQC_GEMM_GATHER
+            __syncthreads();
+        }
     }
 }
 
@@ -319,112 +366,6 @@ __global__ void zfinal_kernel(const double *zslice, int n, int n_cuts, int renor
     if (threadIdx.x == 0 && blockIdx.x == 0) zfinal(zslice, n, n_cuts, renorm, zinfo);
 }
 
-// FP64 bits -> nearest FP32 (ties to even), the conversion instruction's
-// result, in integer arithmetic for normal results: the instruction runs at
-// the FP64 rate, which held grid30's largest leaf (2^22 elements) to 24 us.
-__device__ __forceinline__ float f64_to_f32(uint64_t b) {
-    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
-    const uint32_t e = (hi >> 20) & 0x7ffu;
-    if (e - 897u > 253u) return (float)__longlong_as_double((long long)b);  // zero, subnormal, overflow, inf, NaN
-    uint32_t u = __funnelshift_l(lo, hi, 3) - (896u << 23);  // exponent rebased (modulo 512), 23 mantissa bits
-    u += ((lo << 3) | (u & 1u)) > 0x80000000u;                // round to nearest even; a carry is right
-    return __uint_as_float(u | (hi & 0x80000000u));
-}
-
-// V source elements from element s on (V > 1: the address is a multiple of V elements).
-template <int V>
-__device__ __forceinline__ void ingest_load(const IngestArgs &g, int64_t s, float (&v)[V]) {
-    if (g.src_dtype == TQC_F64) {
-        const double *p = (const double *)g.src + s;
-        if constexpr (V == 1) {
-            v[0] = f64_to_f32((uint64_t)__double_as_longlong(__ldg(p)));
-        } else {
-#pragma unroll
-            for (int i = 0; i < V; i += 2) {
-                const ulonglong2 q = __ldg((const ulonglong2 *)(p + i));
-                v[i] = f64_to_f32(q.x);
-                v[i + 1] = f64_to_f32(q.y);
-            }
-        }
-    } else {
-        const float *p = (const float *)g.src + s;
-        if constexpr (V == 4) {
-            const float4 q = __ldg((const float4 *)p);
-            v[0] = q.x;
-            v[1] = q.y;
-            v[2] = q.z;
-            v[3] = q.w;
-        } else if constexpr (V == 2) {
-            const float2 q = __ldg((const float2 *)p);
-            v[0] = q.x;
-            v[1] = q.y;
-        } else {
-            v[0] = __ldg(p);
-        }
-    }
-}
-
-// Gather a leaf: thread t (of 2^nbits / V) takes V neighbouring source
-// elements, whose destinations differ in bits vb[0] (and vb[1]).  The threads
-// are a power of two (2^lg), so a thread's t share their lg low bits: that
-// part of the source offset is summed once.
-template <int V>
-__device__ __forceinline__ void ingest_gather(const IngestArgs &g, int64_t t0, int lg) {
-    const int nb = g.nbits - (V == 4 ? 2 : (V == 2 ? 1 : 0));  // bits of t: srcpos[0 .. nb)
-    const int64_t n = 1ll << nb, stride = 1ll << lg;
-    int64_t s_lo = g.src_base;
-    for (int b = 0; b < nb && b < lg; ++b)
-        if (t0 >> b & 1) s_lo += 1ll << g.srcpos[b];
-    const int p0 = V == 4 ? (g.vb[0] < g.vb[1] ? g.vb[0] : g.vb[1]) : g.vb[0];
-    const int p1 = V == 4 ? (g.vb[0] < g.vb[1] ? g.vb[1] : g.vb[0]) : 0;
-    const int64_t d1 = 1ll << g.vb[0], d2 = V == 4 ? 1ll << g.vb[1] : 0;
-    for (int64_t t = t0; t < n; t += stride) {
-        int64_t s = s_lo;
-        for (int b = lg; b < nb; ++b)
-            if (t >> b & 1) s += 1ll << g.srcpos[b];
-        int64_t d = t;  // destination of the first: zero bits inserted at vb
-        if (V >= 2) d = ((d >> p0) << (p0 + 1)) | (d & ((1ll << p0) - 1));
-        if (V == 4) d = ((d >> p1) << (p1 + 1)) | (d & ((1ll << p1) - 1));
-        auto at = [&](int i) { return d + ((i & 1) ? d1 : 0) + ((i & 2) ? d2 : 0); };
-        if (g.scaled || g.storage == ST_F64) {
-#pragma unroll
-            for (int i = 0; i < V; ++i) {
-                const double x = ld_src<double>(g.src, g.src_dtype, s + i);
-                if (!g.scaled) ((double *)g.dst)[at(i)] = x;
-                else if (g.out_f64) ((double *)g.dst)[at(i)] = x * g.zinfo[1];
-                else ((float *)g.dst)[at(i)] = (float)(x * g.zinfo[1]);
-            }
-            continue;
-        }
-        float v[V];
-        ingest_load<V>(g, s, v);
-        switch (g.storage) {
-            case ST_F32:
-#pragma unroll
-                for (int i = 0; i < V; ++i) ((float *)g.dst)[at(i)] = v[i];
-                break;
-            case ST_TF32:
-#pragma unroll
-                for (int i = 0; i < V; ++i) ((float *)g.dst)[at(i)] = to_tf32(v[i]);
-                break;
-            case ST_BF16:
-#pragma unroll
-                for (int i = 0; i < V; ++i) ((__nv_bfloat16 *)g.dst)[at(i)] = __float2bfloat16_rn(v[i]);
-                break;
-            case ST_BF16X2:
-                // hi = bf16(v), lo = bf16(v - hi) from the FP32 value (v - hi is exact in FP32)
-#pragma unroll
-                for (int i = 0; i < V; ++i) {
-                    const __nv_bfloat16 h = __float2bfloat16_rn(v[i]);
-                    ((__nv_bfloat16 *)g.dst)[at(i)] = h;
-                    ((__nv_bfloat16 *)g.dst_lo)[at(i)] = __float2bfloat16_rn(v[i] - __bfloat162float(h));
-                }
-                break;
-            default: break;
-        }
-    }
-}
-
 // Node tensors into operand layouts (every leaf of a contract in one launch:
 // CTAs blk[j] .. blk[j + 1] take leaf j): destination bit b reads source bit
 // srcpos[b]; src_base carries the fixed output bits of the bin and the values
@@ -475,9 +416,7 @@ __global__ void __launch_bounds__(INGEST_THREADS) ingest_kernel(const __grid_con
     }
     const int lg = __ffs(blocks * INGEST_THREADS) - 1;
     const int64_t t0 = (int64_t)block * INGEST_THREADS + threadIdx.x;
-    if (g.vec == 4) ingest_gather<4>(g, t0, lg);
-    else if (g.vec == 2) ingest_gather<2>(g, t0, lg);
-    else ingest_gather<1>(g, t0, lg);
+    ingest_range(g, t0, (1ll << g.nbits) / g.vec, lg);
 }
 
 __global__ void finalize_kernel(const double *acc, void *out, int out_f64, const double *zinfo, int64_t n) {
@@ -538,9 +477,18 @@ cudaError_t launch_cfg(const StepArgs &a, cudaStream_t s) {
 
 // The tile configurations of K >= 16 steps whose tiles are whole.
 template <int BM, int BN, int TM, int MINB>
-cudaError_t launch_gemm(const StepArgs &a, cudaStream_t s) {
+cudaError_t launch_gemm(const StepArgs &step, cudaStream_t s) {
+    StepArgs a = step;
+    if (BM == BN && smallk_layout(a.epi).direct && !smallk_layout(a.epi).rowmajor) {
+        // the result's lowest bits are row bits: exchange rows and columns, so
+        // that the eight lanes along columns store 128 consecutive bytes
+        std::swap(a.A, a.B);
+        std::swap(a.mb, a.nb);
+        std::swap(a.epi.lowRc, a.epi.lowCc);
+        std::swap(a.epi.highR, a.epi.highC);
+    }
     constexpr int NT = (BM / TM) * (BN / 8);
-    const size_t smem = sizeof(EpiTables) + std::max((size_t)2 * 16 * (BM + BN), (size_t)BM * (BN + 4)) * sizeof(float);
+    const size_t smem = sizeof(EpiTables) + std::max((size_t)2 * 16 * (BM + BN), (size_t)BM * BN) * sizeof(float);
     static bool attr = false;
     if (!attr) {
         cudaError_t e = cudaFuncSetAttribute(simt_gemm_f32<BM, BN, TM, MINB>,
@@ -551,7 +499,7 @@ cudaError_t launch_gemm(const StepArgs &a, cudaStream_t s) {
     const int64_t col_tiles = 1ll << (a.nb - a.epi.b_bits);
     const int64_t n_tiles = (1ll << (a.mb - a.epi.a_bits)) * col_tiles;
     const int64_t grid = std::min<int64_t>(n_tiles, (int64_t)sm_count() * MINB);
-    return launch_pdl(simt_gemm_f32<BM, BN, TM, MINB>, grid, NT, smem, s, a, n_tiles, col_tiles);
+    return launch_pdl(simt_gemm_f32<BM, BN, TM, MINB>, grid, NT, smem, s, a, n_tiles, col_tiles, smallk_layout(a.epi));
 }
 
 }  // namespace
@@ -750,7 +698,7 @@ int znet_launches(const ZStep *z, int n_steps, bool last) {
 
 // Largest V <= 4 whose source bits 0 .. log2 V - 1 are destination bits, with
 // the tensor aligned for the loads (16 bytes at most).
-static void ingest_vec(IngestArgs &g) {
+void ingest_vec(IngestArgs &g) {
     g.vec = 1;
     if (g.scaled || g.storage == ST_F64) return;
     int at[2] = {-1, -1};

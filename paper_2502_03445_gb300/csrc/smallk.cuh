@@ -142,11 +142,11 @@ __device__ __forceinline__ void sk_stage(float *stg, const float (&acc)[4 * QM][
         }
 }
 
-// Write the staged tile (E results) to the destination: thread gt takes
-// the aligned fours t = 4 gt + 512 n; element offset of t = g_hi[t >> 7] +
-// g_lo[t & 127] (t & 127 fixed per thread).  MODE: the output mode, or -1
+// Write the staged tile (E results) to the destination: thread gt of NT takes
+// the aligned fours t = 4 gt + 4 NT n; element offset of t = g_hi[t >> 7] +
+// g_lo[t & 127] (t & 127 fixed per thread: NT is a multiple of 32).  MODE: the output mode, or -1
 // to dispatch it per store (fewer live registers).
-template <int MODE>
+template <int MODE, int NT = 128>
 __device__ __forceinline__ void sk_gather(const EpiTables *tb, const float *stg, const EpiParams &e, uint64_t base,
                                           int E, int gt) {
     const int mode = MODE >= 0 ? MODE : e.mode;
@@ -154,7 +154,7 @@ __device__ __forceinline__ void sk_gather(const EpiTables *tb, const float *stg,
     const float sf = (float)sd;
     const uint64_t gb = base + tb->g_lo[(gt * 4) & 127];
 #pragma unroll 4
-    for (int t = gt * 4; t < E; t += 512) {
+    for (int t = gt * 4; t < E; t += 4 * NT) {
         const float4 q = *(const float4 *)(stg + (sk_swz((uint32_t)t >> 2) << 2));
         const float v[4] = {q.x, q.y, q.z, q.w};
         if constexpr (MODE >= 0) store_vals<MODE, 4>(e, gb + tb->g_hi[t >> 7], v, sf, sd);

@@ -288,8 +288,10 @@ TQC_API tqc_status tqc_contract_host(tqc_plan_t plan, const void *const *host_te
  * changed, and none is sliced (TQC_ERR_UNSUPPORTED otherwise).  The first
  * call with a given (plans, outputs) list builds and uploads the work list
  * (allocates, synchronises); repeated calls with the same list only reset
- * the counters and launch, so they can be captured in a CUDA graph.  Calls
- * that overlap on the GPU share the work list and race.
+ * the counters and launch, so they can be captured in a CUDA graph.  The work
+ * lists of the last eight (plans, outputs) lists are kept, until one of their
+ * plans is destroyed; a graph that captured one must not be replayed after
+ * that.  Calls that overlap on the GPU on one list race.
  */
 TQC_API tqc_status tqc_contract_batch(const tqc_plan_t *plans, void *const *d_outs, int32_t n,
                                       void *cuda_stream);
@@ -427,10 +429,8 @@ TQC_API tqc_status tqc_plan_candidates(tqc_net_t net, const tqc_plan_opts *opts,
 /* The L2 norm over all cut assignments of every output state of subcircuit
  * `sub`: d_norms[i] = sqrt(sum_e T_sub[e][i]^2), i in [0, 2^{n_out}).
  * d_norms: device, FP64, 2^{n_out} entries, caller-owned; stream-ordered.
- * Deterministic: the partial sums are added in a fixed order.  When the
- * output states alone cannot fill the GPU the sum is split over the cut
- * assignments, with a stream-ordered scratch allocation (cudaMallocAsync) of
- * a few MB for the partials. */
+ * Deterministic: the partial sums are added in a fixed order.  Allocates
+ * nothing. */
 TQC_API tqc_status tqc_hss_norms(tqc_net_t net, int32_t sub, double *d_norms, void *cuda_stream);
 /* Select heavy states: norms on the device, then every subcircuit is seeded
  * with its heaviest state and states are added in descending norm (ties:

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <new>
 #include <string>
@@ -184,6 +185,8 @@ tqc_status tqc_plan(tqc_net_t net, const tqc_plan_opts *opts, tqc_plan_t *out) {
         delete h;
         return st;
     }
+    static std::atomic<uint64_t> serial{0};
+    h->p.serial = ++serial;
     net->n.live_plans++;
     *out = h;
     return TQC_OK;
@@ -351,6 +354,7 @@ tqc_status tqc_plan_step_time(tqc_plan_t plan, int32_t step, double *mean_ms, in
 
 tqc_status tqc_plan_destroy(tqc_plan_t plan) {
     if (!plan) return fail(TQC_ERR_INVALID, "NULL plan");
+    if (plan->p.batched) batch_forget(plan->p.serial);
     exec_release(&plan->p);
     if (plan->p.d_hostout) cudaFree(plan->p.d_hostout);
     plan->p.net->live_plans--;

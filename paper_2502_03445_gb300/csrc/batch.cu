@@ -19,11 +19,14 @@
 
 #include <algorithm>
 #include <cstring>
+#include <iterator>
+#include <list>
 #include <mutex>
 #include <string>
 #include <vector>
 
 #include "device_common.cuh"
+#include "ingest.cuh"
 #include "launch.h"
 #include "smallk.cuh"
 
@@ -36,9 +39,10 @@ namespace {
 
 constexpr int BT = 576;                    // 18 warps: producer, MMA issuer, 16 epilogue / worker warps
 constexpr int EPIW = 16;
-constexpr int EPI = 32 * EPIW;
+constexpr int EPI = 32 * EPIW;             // 2^9: the ingest items' thread stride
+static_assert(EPI == 512, "ingest_range's stride");
 constexpr long long BWAIT = 2000000000ll;  // ~1 s at the boost clock
-constexpr int64_t CHUNK = 1 << 16;          // ingest elements per item
+constexpr int64_t CHUNK = 1 << 13;          // ingest indices (of up to four elements) per item
 constexpr int RING = 196608;               // operand ring (tensor-core items) / worker buffers (CUDA-core items)
 constexpr int MAXST = 16;
 constexpr int BM = 128;
@@ -189,40 +193,6 @@ __device__ __forceinline__ void tmem_load16(uint32_t taddr, uint32_t (&r)[16]) {
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// The elements it.lo + tid + k nt of an ingest chunk.  nt (512) is a power
-// of two and it.lo a multiple of it, so a thread's elements share their low
-// log2(nt) bits: that part of the source offset is summed once.
-__device__ void ingest_range(const BIngest &it, int tid, int nt) {
-    const IngestArgs &g = it.g;
-    const int lg = __ffs(nt) - 1;
-    const int64_t d0 = it.lo + tid;
-    int64_t s_lo = g.src_base;
-    for (int b = 0; b < g.nbits && b < lg; ++b)
-        if (d0 >> b & 1) s_lo += 1ll << g.srcpos[b];
-    for (int64_t d = d0; d < it.hi; d += nt) {
-        int64_t s = s_lo;
-        for (int b = lg; b < g.nbits; ++b)
-            if (d >> b & 1) s += 1ll << g.srcpos[b];
-        const double v64 = g.src_dtype == TQC_F64 ? ((const double *)g.src)[s] : (double)((const float *)g.src)[s];
-        if (g.scaled) {
-            ((float *)g.dst)[d] = (float)(v64 * g.zinfo[1]);
-            continue;
-        }
-        const float v = (float)v64;
-        switch (g.storage) {
-            case ST_F32: ((float *)g.dst)[d] = v; break;
-            case ST_TF32: ((float *)g.dst)[d] = to_tf32(v); break;
-            case ST_BF16: ((__nv_bfloat16 *)g.dst)[d] = __float2bfloat16_rn(v); break;
-            case ST_BF16X2: {  // the standalone ingest's split, from the FP32 value
-                const __nv_bfloat16 h = __float2bfloat16_rn(v);
-                ((__nv_bfloat16 *)g.dst)[d] = h;
-                ((__nv_bfloat16 *)g.dst_lo)[d] = __float2bfloat16_rn(v - __bfloat162float(h));
-            } break;
-            default: break;
-        }
-    }
 }
 
 __device__ __forceinline__ void cp_async4(float *dst, const float *src, bool valid) {
@@ -405,7 +375,10 @@ __global__ void __launch_bounds__(BT, 1)
         const BItem item = items[it];
         const bool run = ctl->ok && item.kind != IT_STALL;
         if (run && item.kind == IT_INGEST) {
-            if (warp >= 2) ingest_range(ing[item.idx], tid - 64, EPI);
+            if (warp >= 2) {
+                const BIngest &b = ing[item.idx];  // b.lo is a multiple of EPI = 2^9
+                ingest_range(b.g, b.lo + tid - 64, b.hi, 9);
+            }
         } else if (run && steps[item.idx].klass != KC_UMMA) {
             if (warp >= 2) {
                 const int g = (warp - 2) >> 2, gt = (tid - 64) & 127;
@@ -668,22 +641,29 @@ struct Batch {
     BStep *d_steps = nullptr;
     EpiTables *d_tables = nullptr;
     BIngest *d_ing = nullptr;
-    unsigned long long *d_counters = nullptr;  // [counters..., next]
-    int *d_err = nullptr;
+    unsigned long long *d_counters = nullptr;  // [counters..., next, error word]
+    int *d_err = nullptr;                      // the error word
     int64_t n_items = 0, n_counters = 0;
+    std::vector<uint64_t> serials;  // of its plans
     void release() {
         cudaFree(d_items);
         cudaFree(d_steps);
         cudaFree(d_tables);
         cudaFree(d_ing);
         cudaFree(d_counters);
-        cudaFree(d_err);
         *this = Batch();
     }
 };
 
+// Work lists are kept for the last few (plans, outputs) lists, so that a
+// program that alternates between batches builds each once (48 networks:
+// 1.4 ms of host work, allocation and upload per build).  At most POOL_MAX;
+// the least recently launched one is freed, and a list goes with the first
+// of its plans to be destroyed (batch_forget).  All under g_batch_mu.
+constexpr size_t POOL_MAX = 8;
 std::mutex g_batch_mu;
-Batch g_batch;
+std::list<Batch> g_pool;     // most recently launched first
+Batch *g_batch = nullptr;    // the last one launched (status, launch counts)
 int g_inject_stall = 0;
 double g_tail_s = 16e-6;
 // process-wide, created on first use (the tail streams of every device's
@@ -704,6 +684,18 @@ cudaError_t upload(T **dst, const std::vector<T> &v) {
     return cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice);
 }
 
+// Whether a batch can run on the plans as they are.
+tqc_status check_plans(Plan *const *plans, int n) {
+    for (int pi = 0; pi < n; ++pi) {
+        const Plan &p = *plans[pi];
+        if (!p.ready) return fail(TQC_ERR_INVALID, "batch: plan " + std::to_string(pi) + " was never contracted");
+        if (p.n_slices() > 1) return fail(TQC_ERR_UNSUPPORTED, "batch: plan " + std::to_string(pi) + " is sliced");
+        if (p.z_version != p.net->version)
+            return fail(TQC_ERR_INVALID, "batch: plan " + std::to_string(pi) + " has changed tensors; contract it once");
+    }
+    return TQC_OK;
+}
+
 tqc_status build_batch(Plan *const *plans, void *const *outs, int n, Batch *b) {
     std::vector<double> tail_time;  // predicted seconds of each plan's large steps
     std::vector<BItem> items;
@@ -715,10 +707,6 @@ tqc_status build_batch(Plan *const *plans, void *const *outs, int n, Batch *b) {
     int n_counters = 0;
     for (int pi = 0; pi < n; ++pi) {
         Plan &p = *plans[pi];
-        if (!p.ready) return fail(TQC_ERR_INVALID, "batch: plan " + std::to_string(pi) + " was never contracted");
-        if (p.n_slices() > 1) return fail(TQC_ERR_UNSUPPORTED, "batch: plan " + std::to_string(pi) + " is sliced");
-        if (p.z_version != p.net->version)
-            return fail(TQC_ERR_INVALID, "batch: plan " + std::to_string(pi) + " has changed tensors; contract it once");
         // ingest chunks (all leaves of the plan count on one counter)
         const int ing_counter = n_counters++;
         int64_t n_chunks = 0;
@@ -736,7 +724,8 @@ tqc_status build_batch(Plan *const *plans, void *const *outs, int n, Batch *b) {
                 bi.g.storage = t.storage;
             }
             bi.done = ing_counter;
-            const int64_t total = p.m == 1 ? p.out_elems() : ((int64_t)1 << t.nbits());
+            ingest_vec(bi.g);
+            const int64_t total = ((int64_t)1 << bi.g.nbits) / bi.g.vec;
             for (int64_t lo = 0; lo < total; lo += CHUNK) {
                 bi.lo = lo;
                 bi.hi = std::min(total, lo + CHUNK);
@@ -777,7 +766,9 @@ tqc_status build_batch(Plan *const *plans, void *const *outs, int n, Batch *b) {
             std::memset((void *)&bs, 0, sizeof bs);
             bs.klass = sp.klass;
             bs.prec = sp.prec;
-            const bool smallk = sp.klass != KC_UMMA && sp.tile == SIMT_SMALLK;
+            // (also where the standalone step takes 128 x 128 tiles for K = 16: no such tile here)
+            const bool smallk = sp.klass != KC_UMMA && (sp.tile == SIMT_SMALLK || (sp.kb == 4 && sp.tile == SIMT_128x128 &&
+                                                                                   !(p.flags & TQC_FLAG_NO_SMALLK)));
             TileShape ts = sp.klass == KC_UMMA ? TileShape{7, 6}
                                                : (smallk ? smallk_tile(sp.mb, sp.nb, sp.kb) : TileShape{6, 6});
             bs.a = exec_step_args(p, sp, ts);
@@ -816,7 +807,8 @@ tqc_status build_batch(Plan *const *plans, void *const *outs, int n, Batch *b) {
             }
             const int64_t n_tiles = row_tiles * bs.col_tiles;
             // items of 16 tiles, larger for large steps (fewer pipeline drains),
-            // still about two per SM
+            // still about two per SM (48 networks of 16-24 qubits: 718 us; from 8
+            // tiles 788, from 4 tiles 903)
             per_item = std::min<int64_t>(128, std::max<int64_t>(16, n_tiles / (2 * (int64_t)sm_count()) / 4 * 4));
             const int64_t n_step_items = (n_tiles + per_item - 1) / per_item;
             bs.dep[0] = counter_of[sp.a];
@@ -861,9 +853,11 @@ tqc_status build_batch(Plan *const *plans, void *const *outs, int n, Batch *b) {
     if (e == cudaSuccess) e = upload(&b->d_steps, steps);
     if (e == cudaSuccess) e = upload(&b->d_tables, tables);
     if (e == cudaSuccess) e = upload(&b->d_ing, ing);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counters, sizeof(unsigned long long) * (n_counters + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(b->d_err, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_counters, sizeof(unsigned long long) * (n_counters + 2));
+    if (e == cudaSuccess) {
+        b->d_err = (int *)(b->d_counters + n_counters + 1);
+        e = cudaMemset(b->d_err, 0, sizeof(int));
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         b->release();
@@ -872,7 +866,32 @@ tqc_status build_batch(Plan *const *plans, void *const *outs, int n, Batch *b) {
     return TQC_OK;
 }
 
+void drop(std::list<Batch>::iterator it) {
+    if (g_batch == &*it) g_batch = nullptr;
+    it->release();
+    g_pool.erase(it);
+}
+
 }  // namespace
+
+// A plan is about to be destroyed: its lists can never be launched again.
+// The last launched one keeps its error word for tqc_batch_status.
+void batch_forget(uint64_t serial) {
+    std::lock_guard<std::mutex> lk(g_batch_mu);
+    for (auto it = g_pool.begin(); it != g_pool.end();) {
+        const auto next = std::next(it);
+        if (std::find(it->serials.begin(), it->serials.end(), serial) != it->serials.end()) {
+            if (g_batch == &*it) {
+                it->key.clear();
+                it->tails.clear();
+            } else {
+                drop(it);
+            }
+        }
+        it = next;
+    }
+}
+
 }  // namespace tqc
 
 using namespace tqc;
@@ -888,37 +907,55 @@ tqc_status tqc_contract_batch(const tqc_plan_t *plans, void *const *d_outs, int3
     // plans' workspaces: they keep no intermediates across tqc_contract calls
     for (int i = 0; i < n; ++i) plans[i]->p.batched = true;
     std::vector<const void *> key;
+    std::vector<Plan *> ps;
     for (int i = 0; i < n; ++i) {
-        key.push_back(plans[i]);
+        ps.push_back(&plans[i]->p);
+        key.push_back((const void *)(uintptr_t)plans[i]->p.serial);
         key.push_back(d_outs[i]);
     }
     key.push_back((const void *)(intptr_t)g_inject_stall);
     key.push_back((const void *)(intptr_t)(int64_t)(std::min(g_tail_s, 1e6) * 1e9));
-    if (key != g_batch.key) {
-        g_batch.release();
-        std::vector<Plan *> ps;
-        for (int i = 0; i < n; ++i) ps.push_back(&plans[i]->p);
-        tqc_status st = build_batch(ps.data(), d_outs, n, &g_batch);
+    if (!g_batch || key != g_batch->key) {
+        tqc_status st = check_plans(ps.data(), n);
         if (st != TQC_OK) return st;
-        g_batch.key = key;
-        static bool attr = false;
-        if (!attr) {
-            if (cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess)
-                return fail(TQC_ERR_CUDA, "batch kernel attributes");
-            attr = true;
+        auto it = std::find_if(g_pool.begin(), g_pool.end(), [&](const Batch &b) { return b.key == key; });
+        if (it != g_pool.end()) {
+            g_pool.splice(g_pool.begin(), g_pool, it);
+        } else {
+            static bool attr = false;
+            if (!attr) {
+                if (cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess)
+                    return fail(TQC_ERR_CUDA, "batch kernel attributes");
+                attr = true;
+            }
+            while (g_pool.size() >= POOL_MAX) drop(std::prev(g_pool.end()));
+            Batch fresh;
+            st = build_batch(ps.data(), d_outs, n, &fresh);
+            if (st != TQC_OK) return st;
+            fresh.key = key;
+            for (Plan *p : ps) fresh.serials.push_back(p->serial);
+            g_pool.push_front(std::move(fresh));
+        }
+        g_batch = &g_pool.front();
+        // lists of destroyed plans were kept for their status only
+        for (auto i = std::next(g_pool.begin()); i != g_pool.end();) {
+            const auto next = std::next(i);
+            if (i->key.empty()) drop(i);
+            i = next;
         }
     }
+    Batch &bt = *g_batch;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    cudaError_t e = cudaMemsetAsync(g_batch.d_counters, 0, sizeof(unsigned long long) * (g_batch.n_counters + 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g_batch.d_err, 0, sizeof(int), s);
+    // counters, the claim counter and the error word
+    cudaError_t e = cudaMemsetAsync(bt.d_counters, 0, sizeof(unsigned long long) * (bt.n_counters + 2), s);
     if (e != cudaSuccess) return fail(TQC_ERR_CUDA, std::string("batch reset: ") + cudaGetErrorString(e));
     const int grid = sm_count();
-    batch_kernel<<<grid, BT, SMEM, s>>>(g_batch.d_items, g_batch.n_items, g_batch.d_steps, g_batch.d_tables,
-                                        g_batch.d_ing, g_batch.d_counters, g_batch.d_counters + g_batch.n_counters,
-                                        g_batch.d_err);
+    batch_kernel<<<grid, BT, SMEM, s>>>(bt.d_items, bt.n_items, bt.d_steps, bt.d_tables,
+                                        bt.d_ing, bt.d_counters, bt.d_counters + bt.n_counters,
+                                        bt.d_err);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(TQC_ERR_CUDA, std::string("batch launch: ") + cudaGetErrorString(e));
-    if (g_batch.tails.empty()) return TQC_OK;
+    if (bt.tails.empty()) return TQC_OK;
     int dev = 0;
     cudaGetDevice(&dev);
     if (g_tail_device != dev) {
@@ -936,9 +973,9 @@ tqc_status tqc_contract_batch(const tqc_plan_t *plans, void *const *d_outs, int3
     for (int k = 0; k < TAIL_STREAMS && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(g_tail_ts[k], g_tail_fork, 0);
     if (e != cudaSuccess) return fail(TQC_ERR_CUDA, std::string("batch fork: ") + cudaGetErrorString(e));
     tqc_status st = TQC_OK;
-    for (size_t i = 0; i < g_batch.tails.size() && st == TQC_OK; ++i) {
-        const BatchTail &t = g_batch.tails[i];
-        st = exec_run_tail(*t.p, t.first, t.out, g_tail_ts[g_batch.tail_stream[i]]);
+    for (size_t i = 0; i < bt.tails.size() && st == TQC_OK; ++i) {
+        const BatchTail &t = bt.tails[i];
+        st = exec_run_tail(*t.p, t.first, t.out, g_tail_ts[bt.tail_stream[i]]);
     }
     // join (also after a failed launch, so the caller's stream stays ordered)
     for (int k = 0; k < TAIL_STREAMS; ++k) {
@@ -951,16 +988,16 @@ tqc_status tqc_contract_batch(const tqc_plan_t *plans, void *const *d_outs, int3
 
 tqc_status tqc_batch_status(void *cuda_stream) {
     std::lock_guard<std::mutex> lk(g_batch_mu);
-    if (!g_batch.d_err) return fail(TQC_ERR_INVALID, "no batch launched");
+    if (!g_batch) return fail(TQC_ERR_INVALID, "no batch launched");
     int h = 0;
-    cudaError_t e = cudaMemcpyAsync(&h, g_batch.d_err, sizeof(int), cudaMemcpyDeviceToHost, (cudaStream_t)cuda_stream);
+    cudaError_t e = cudaMemcpyAsync(&h, g_batch->d_err, sizeof(int), cudaMemcpyDeviceToHost, (cudaStream_t)cuda_stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)cuda_stream);
     if (e != cudaSuccess) return fail(TQC_ERR_CUDA, std::string("batch status: ") + cudaGetErrorString(e));
     if (h) return fail(TQC_ERR_TIMEOUT, "a bounded wait in the batched launch gave up");
     // the large steps' error words (their plans' own): every one that is set
     // is cleared, so the next call reports only its own
     bool timed_out = false;
-    for (const BatchTail &t : g_batch.tails) {
+    for (const BatchTail &t : g_batch->tails) {
         int w = 0;
         e = cudaMemcpyAsync(&w, t.p->d_zinfo + 2, sizeof(int), cudaMemcpyDeviceToHost, (cudaStream_t)cuda_stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)cuda_stream);
@@ -975,9 +1012,9 @@ tqc_status tqc_batch_status(void *cuda_stream) {
 tqc_status tqc_batch_launches(int64_t *launches, int64_t *tail_steps) {
     if (!launches) return fail(TQC_ERR_INVALID, "NULL launches");
     std::lock_guard<std::mutex> lk(g_batch_mu);
-    if (!g_batch.d_err) return fail(TQC_ERR_INVALID, "no batch launched");
+    if (!g_batch) return fail(TQC_ERR_INVALID, "no batch launched");
     int64_t n = 1, steps = 0;  // the persistent kernel, then each large step's launches
-    for (const BatchTail &t : g_batch.tails)
+    for (const BatchTail &t : g_batch->tails)
         for (size_t i = t.first; i < t.p->steps.size(); ++i) {
             const StepPlan &sp = t.p->steps[i];
             ++steps;

@@ -160,6 +160,7 @@ struct Plan {
     int64_t states_bytes = 0;
     // intermediates kept across calls (bins that differ in some leaves' fixed bits)
     bool reuse_ok = false;                 // the workspace holds the last call's values
+    uint64_t serial = 0;                   // unique among the process's plans
     bool batched = false;                  // part of a batched launch, whose replays rewrite the workspace
     uint64_t reuse_version = 0;            // network version of those values
     std::vector<int64_t> leaf_key;         // per leaf: its bin restriction (source offset) in that call
@@ -225,6 +226,7 @@ int exec_src_pos_cut(const Node &nd, int c);
 tqc_status exec_contract(Plan *p, const uint8_t *fixed_bits, void *d_out, int out_dtype, double *z_out,
                          void *stream);
 void exec_release(Plan *p);
+void batch_forget(uint64_t serial);  // batch.cu: frees the work lists a plan is part of
 void exec_clear_events(Plan *p);
 tqc_status exec_step_time(Plan *p, int step, double *mean_ms, int *launches);
 

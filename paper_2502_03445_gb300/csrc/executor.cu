@@ -218,7 +218,12 @@ int default_step_tile(const StepPlan &st, int out_esize, bool smallk) {
         if (deep) return st.prec == TQC_PREC_BF16X3 ? UMMA_128x128_DEEP : UMMA_128x128;
         if (big) {
             const EpiParams e = make_epi(st.maskR, st.maskC, st.mb, st.nb, TileShape{7, 6});
-            if (direct_store_efficiency(e, out_esize) >= 0.99) return st.nb >= 8 ? UMMA_128x256_DEEP : UMMA_128x128_DEEP;
+            if (direct_store_efficiency(e, out_esize) >= 0.99) {
+#ifdef V_FILL
+                if (st.nb >= 8 && ((int64_t)1 << (st.mb + st.nb - 15)) < sm_count()) return UMMA_128x128_DEEP;
+#endif
+                return st.nb >= 8 ? UMMA_128x256_DEEP : UMMA_128x128_DEEP;
+            }
         }
         return st.nb >= 7 ? UMMA_128x128 : UMMA_128x64;
     }

@@ -291,7 +291,6 @@ __global__ void __launch_bounds__(128, (QM == 1) == RM ? 8 : 6)
         __syncthreads();
     }
     pdl_launch();
-    pdl_wait();
     smallk_tiles_body<KB, QM, RM, false>(args, tb, L, col_tiles, blockIdx.x, n_tiles, gridDim.x, buf, threadIdx.x, 1);
 }
 

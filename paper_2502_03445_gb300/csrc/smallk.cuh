@@ -186,7 +186,10 @@ __device__ __forceinline__ void smallk_tiles_body(const StepArgs &sa, const EpiT
     const int direct = L.direct;
     constexpr int K = 1 << KB;
     constexpr int QN = 3 - QM;
-    if (t0 >= t_end) return;
+    if (t0 >= t_end) {
+        if constexpr (!LEAN) pdl_wait();
+        return;
+    }
     __builtin_assume(__isShared(buf));
     __builtin_assume(__isShared(tb));
     const EpiParams &e = sa.epi;
@@ -231,6 +234,8 @@ __device__ __forceinline__ void smallk_tiles_body(const StepArgs &sa, const EpiT
         dr0 = pdep64((uint64_t)sr, e.highR);
         dr1 = pdep64((uint64_t)sr + 1, e.highR);
     }
+    // everything above needs only the parameters (and overlaps the kernel before)
+    if constexpr (!LEAN) pdl_wait();
     for (int t = (int)t0; t < (int)t_end; t += (int)stride) {
         if constexpr (LEAN) {
             rt = t >> lct;

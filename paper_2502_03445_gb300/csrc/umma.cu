@@ -36,6 +36,7 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <vector>
 
 #include "device_common.cuh"
 #include "launch.h"
@@ -64,8 +65,8 @@ struct UmmaParams {
     int32_t sw64;          // deep form: 64-byte swizzled k-blocks (half the K per stage, twice the stages)
     int32_t kblk;          // operands K-blocked ([K / 64][rows][64]): 3-D copies
     int32_t k_blocks;
-    int32_t rowmajor;  // staging orientation (pick_staging)
-    int32_t gmode;     // gather mode of the write-out (pick_staging)
+    int32_t vec;       // staged form: consecutive results of a row in one staging store (1, 2 or 4)
+    uint32_t xmask;    // staged form: the staging swizzle (stage_swizzle)
     int32_t bres;      // B stays resident in shared memory (one k-block, one column tile; deep form)
     int32_t stall;     // test hook: CTA 0 never issues its first k-block's copies
     EpiParams epi;
@@ -82,9 +83,7 @@ struct Cfg {
     static constexpr int STAGE_BYTES = PLANES * (A_BYTES + B_BYTES);
     static constexpr int STAGES = DEEP ? 196608 / STAGE_BYTES : (KIND == K_BF16X3 ? 2 : (BN == 64 ? 6 : 4));
     static constexpr int SUB_N = 64;               // epilogue sub-tile: 128 x 64
-    static constexpr int PITCH_R = SUB_N + 4;      // row-major staging pitch (floats)
-    static constexpr int PITCH_C = BM + 4;         // column-major staging pitch
-    static constexpr int STG_FLOATS = BM * PITCH_R > SUB_N * PITCH_C ? BM * PITCH_R : SUB_N * PITCH_C;
+    static constexpr int STG_FLOATS = BM * SUB_N;
     static constexpr int STG_BYTES = DEEP ? 0 : 2 * STG_FLOATS * 4;  // two buffers (ping-pong)
     static constexpr int BAR_BYTES = 1024;
     static constexpr int RING = STAGES * STAGE_BYTES;      // bytes of the operand ring
@@ -100,6 +99,39 @@ struct Cfg {
 };
 
 
+
+// Staged epilogue.  A 128 x 64 sub-tile is staged in its own destination
+// order: result t (the sub-tile's result bits, compacted, lowest first) at word
+// stage_word(t) = t with bits 2..4 XORed by three-bit masks of t's bits from 5
+// on.  The map is linear over GF(2), so the word of (row, column) is the XOR of
+// a row part and a column part.  The masks (xmask, stage_swizzle) put the row
+// bits that vary over a store's lanes on different banks; the write-out reads
+// 16 bytes per four results in destination order, free of conflicts for any
+// masks.
+__device__ __forceinline__ uint32_t stage_word(uint32_t t, uint32_t xmask) {
+    uint32_t x = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (t >> (5 + k) & 1) x ^= xmask >> (3 * k) & 7u;
+    return t ^ (x << 2);
+}
+
+// Write a staged sub-tile (E results) to its destination: thread etid takes the
+// aligned fours t = 4 etid + 2048 n, element offset g_hi[t >> 7] + g_lo[t & 127].
+template <int MODE>
+__device__ __forceinline__ void staged_write(const EpiTables *tb, const float *stg, const EpiParams &e, uint64_t base,
+                                             int E, int etid, uint32_t w0, uint32_t xmask, float sf, double sd) {
+    __builtin_assume(__isShared(tb));
+    __builtin_assume(__isShared(stg));
+    const uint64_t gb = base + tb->g_lo[(etid * 4) & 127];
+#pragma unroll 4
+    for (int t = etid * 4; t < E; t += 4 * EPI_THREADS) {
+        // t = 4 etid + 2048 n: the words of its two parts XOR
+        const float4 q = *(const float4 *)(stg + (w0 ^ stage_word((uint32_t)(t & ~(4 * EPI_THREADS - 1)), xmask)));
+        const float v[4] = {q.x, q.y, q.z, q.w};
+        store_vals<MODE, 4>(e, gb + tb->g_hi[t >> 7], v, sf, sd);
+    }
+}
 
 template <int BN, int KIND, bool DEEP>
 __global__ void __launch_bounds__(NTHREADS, 1)
@@ -164,6 +196,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                      "r"((uint32_t)C::TMEM_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if constexpr (!DEEP) {  // element offsets of the staged write-out
+        if (warp >= 2) epi_tables_init(tb, P.epi, true, 0, threadIdx.x - 64, EPI_THREADS);
     }
     tc_fence_before();
     __syncthreads();
@@ -354,9 +389,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int etid = threadIdx.x - 64;      // 0..EPI_THREADS-1
         const int Me = 1 << e.a_bits, Ne = 1 << e.b_bits;
         const int E = Me * Ne;
-        const int pitch = P.rowmajor ? C::PITCH_R : C::PITCH_C;
         float *stgbuf[2] = {stg, stg + C::STG_FLOATS};
-        epi_tables_init(tb, e, P.rowmajor != 0, pitch, etid, EPI_THREADS);
         // bit positions of the result bits that carry the tile indices
         int8_t(*pos)[64] = (int8_t(*)[64])tb_pos;
         int *npos = (int *)(tb_pos + 128);
@@ -370,23 +403,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             npos[etid] = n;
         }
         asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
-        // Full sub-tiles: the staging and destination offsets of this thread's
-        // runs are the same for every sub-tile, so they live in registers.
-        constexpr int ITERS = BM * C::SUB_N / (4 * EPI_THREADS);
-        const bool reg_path = E == BM * C::SUB_N && e.L >= 2 && P.gmode != G_SCALAR && (e.tileMask >> 32) == 0;
-        uint32_t r_s0[ITERS], r_s1[ITERS], r_g[ITERS];
-        if (reg_path) {
+        // this thread's first write-out word, and (staging warps) the words of
+        // its row and of the bits of a column
+        const uint32_t w0 = stage_word((uint32_t)etid * 4, P.xmask);
+        const uint32_t wrow = stage_word(pdep32((uint32_t)row, e.lowRc), P.xmask) ^
+                              stage_word(pdep32((uint32_t)wg * 32, e.lowCc), P.xmask);
+        uint32_t wcol[5];
 #pragma unroll
-            for (int it = 0; it < ITERS; ++it) {
-                const int t = (etid + it * EPI_THREADS) * 4;
-                const uint32_t sh = tb->s_hi[t >> 7];
-                const int tl = t & 127;
-                r_s0[it] = sh + tb->s_lo[tl];
-                r_s1[it] = sh + tb->s_lo[tl + (P.gmode == G_PAIR01 ? 2 : 1)];
-                r_g[it] = (uint32_t)(tb->g_hi[t >> 7] + tb->g_lo[tl]);
-            }
-        }
+        for (int b = 0; b < 5; ++b) wcol[b] = stage_word(pdep32(1u << b, e.lowCc), P.xmask);
         const double sc = (e.mode == EPI_OUT_F32 || e.mode == EPI_OUT_F64) ? e.zinfo[1] : 1.0;
+        const float sf = (float)sc;
         const int64_t my_tiles =
             (int64_t)blockIdx.x < P.n_tiles ? (P.n_tiles - 1 - (int64_t)blockIdx.x) / gridDim.x + 1 : 0;
         const int64_t n_sub = my_tiles * SUBS;
@@ -406,17 +432,29 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             uint32_t r[32];
             tmem_ld32(tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(acc * BN + h * C::SUB_N + col0), r);
             if (row < Me) {
-                if (P.rowmajor) {
-                    float *dst = sb + row * C::PITCH_R + col0;
+                // word of column col0 + j: one XOR per j
+                if (P.vec == 4) {
 #pragma unroll
                     for (int j = 0; j < 32; j += 4)
-                        if (col0 + j < Ne)
-                            *(float4 *)(dst + j) = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                                                               __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+                        if (col0 + j < Ne) {
+                            const uint32_t w = wrow ^ (j & 4 ? wcol[2] : 0) ^ (j & 8 ? wcol[3] : 0) ^ (j & 16 ? wcol[4] : 0);
+                            *(float4 *)(sb + w) = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
+                                                              __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+                        }
+                } else if (P.vec == 2) {
+#pragma unroll
+                    for (int j = 0; j < 32; j += 2)
+                        if (col0 + j < Ne) {
+                            const uint32_t w = wrow ^ (j & 2 ? wcol[1] : 0) ^ (j & 4 ? wcol[2] : 0) ^
+                                               (j & 8 ? wcol[3] : 0) ^ (j & 16 ? wcol[4] : 0);
+                            *(float2 *)(sb + w) = make_float2(__uint_as_float(r[j]), __uint_as_float(r[j + 1]));
+                        }
                 } else {
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
-                        if (col0 + j < Ne) sb[(col0 + j) * C::PITCH_C + row] = __uint_as_float(r[j]);
+                        if (col0 + j < Ne)
+                            sb[wrow ^ (j & 1 ? wcol[0] : 0) ^ (j & 2 ? wcol[1] : 0) ^ (j & 4 ? wcol[2] : 0) ^
+                               (j & 8 ? wcol[3] : 0) ^ (j & 16 ? wcol[4] : 0)] = __uint_as_float(r[j]);
                 }
             }
             if (h == SUBS - 1) {  // last read of this accumulator by this warp
@@ -460,36 +498,20 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             }
             const float *cur = stgbuf[k & 1];
             const uint64_t base = tile_base_slot[k & 1];
-            if (reg_path) {
-#pragma unroll
-                for (int it = 0; it < ITERS; ++it) {
-                    float v[4];
-                    if (P.gmode == G_VEC4) {
-                        const float4 q = *(const float4 *)(cur + r_s0[it]);
-                        v[0] = q.x;
-                        v[1] = q.y;
-                        v[2] = q.z;
-                        v[3] = q.w;
-                    } else {
-                        const float2 a = *(const float2 *)(cur + r_s0[it]);
-                        const float2 b = *(const float2 *)(cur + r_s1[it]);
-                        if (P.gmode == G_PAIR01) {
-                            v[0] = a.x;
-                            v[1] = a.y;
-                            v[2] = b.x;
-                            v[3] = b.y;
-                        } else {
-                            v[0] = a.x;
-                            v[1] = b.x;
-                            v[2] = a.y;
-                            v[3] = b.y;
-                        }
-                    }
-                    store_run_f32(e, base + r_g[it], v, 4, sc);
-                }
-            } else {
-                epi_readout_rt(tb, cur, e, base, E, etid, EPI_THREADS, P.gmode);
+#define TQC_STAGED_WRITE(M) \
+    case M: staged_write<M>(tb, cur, e, base, E, etid, w0, P.xmask, sf, sc); break;
+            switch (e.mode) {
+                TQC_STAGED_WRITE(EPI_F32)
+                TQC_STAGED_WRITE(EPI_TF32)
+                TQC_STAGED_WRITE(EPI_BF16)
+                TQC_STAGED_WRITE(EPI_BF16X2)
+                TQC_STAGED_WRITE(EPI_F64_SET)
+                TQC_STAGED_WRITE(EPI_F64_ADD)
+                TQC_STAGED_WRITE(EPI_OUT_F32)
+                TQC_STAGED_WRITE(EPI_OUT_F64)
+                default: break;
             }
+#undef TQC_STAGED_WRITE
             stop = epi_barrier_or(EPI_THREADS, *abort_flag != 0);
         }
     }
@@ -546,6 +568,36 @@ cudaError_t encode(CUtensorMap *m, const void *ptr, int elem, uint64_t k, uint64
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// The masks of stage_word for a layout.  The lanes of a staging store of `vec`
+// values (an access phase: 8 lanes of 16 bytes, 16 of 8, 32 of 4) differ in the
+// 3, 4 or 5 lowest row bits; those not among the chunk's two lowest result bits
+// are to differ in bank bits 2..4.  The ones at result bits 2..4 do; the others
+// get a mask of a bank bit that is still free.
+uint32_t stage_swizzle(const EpiParams &e, int vec) {
+    const int lanes = vec == 4 ? 3 : (vec == 2 ? 4 : 5);
+    std::vector<int> pos;  // result-bit positions of the lane bits
+    for (int b = 0; b < 32 && (int)pos.size() < lanes; ++b)
+        if (e.lowRc >> b & 1u) pos.push_back(b);
+    std::vector<int> far;
+    bool used[3] = {false, false, false};
+    int n = 0;
+    for (int q : pos) {
+        if (q < 2 || n == 3) continue;
+        ++n;
+        if (q < 5) used[q - 2] = true;
+        else far.push_back(q);
+    }
+    uint32_t m = 0;
+    for (int q : far)
+        for (int d = 0; d < 3; ++d)
+            if (!used[d]) {
+                used[d] = true;
+                m |= 1u << (3 * (q - 5) + d);
+                break;
+            }
+    return m;
+}
+
 template <int BN, int KIND, bool DEEP>
 cudaError_t launch_kind(const StepArgs &a, int *d_err, cudaStream_t s) {
     using C = Cfg<BN, KIND, DEEP>;
@@ -599,9 +651,8 @@ cudaError_t launch_kind(const StepArgs &a, int *d_err, cudaStream_t s) {
     p.n_units = p.n_tiles * a.ksplit;
     p.split_stride = a.ksplit > 1 ? a.split_stride : 0;
     p.bres = DEEP && p.k_blocks == 1 && p.col_tiles == 1;
-    const StagePick pk = pick_staging(a.epi.lowRc, a.epi.lowCc);
-    p.rowmajor = pk.rowmajor;
-    p.gmode = pk.gmode;
+    p.vec = (a.epi.lowCc & 3u) == 3u ? 4 : ((a.epi.lowCc & 1u) ? 2 : 1);
+    p.xmask = stage_swizzle(a.epi, p.vec);
     p.err = d_err;
     p.stall = g_umma_stall.load(std::memory_order_relaxed);
     const int64_t grid = std::min<int64_t>(p.n_units, sm_count());

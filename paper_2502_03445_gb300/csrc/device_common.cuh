@@ -83,6 +83,32 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
     return *(uint32_t *)&p;
 }
 
+// FP32 -> FP64 (exact) and the FP64 product (double)v * s, rounded to nearest
+// even, in integer arithmetic for normal values: the conversion and the
+// multiplication run at two a clock per SM, which bound every FP64 output (2^28
+// results of a K = 4 step: F64FIG).  s is a normal value whose exponent keeps
+// the product normal; zero, subnormal, infinite and NaN v take the instructions.
+__device__ __forceinline__ double f32_to_f64(float v) {
+    const uint32_t u = __float_as_uint(v), e = (u >> 23) & 0xffu;
+    if (e - 1u > 253u) return (double)v;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+__device__ __forceinline__ double f32_times_f64(float v, double s) {
+    const uint32_t u = __float_as_uint(v), ev = (u >> 23) & 0xffu;
+    const uint32_t hi = (uint32_t)__double2hiint(s), lo = (uint32_t)__double2loint(s), es = (hi >> 20) & 0x7ffu;
+    if (ev - 1u > 253u || es - 256u > 1280u) return (double)v * s;
+    // 24 x 53 bits: P = p1 2^32 + low half of p0, in [2^75, 2^77)
+    const uint32_t mv = (u & 0x7fffffu) | 0x800000u;
+    const uint64_t p0 = (uint64_t)mv * lo;
+    const uint64_t p1 = (uint64_t)mv * ((hi & 0xfffffu) | 0x100000u) + (p0 >> 32);
+    const uint32_t n = (uint32_t)(p1 >> 44);  // 1: P >= 2^76, one more bit to drop
+    const uint32_t w0 = (uint32_t)p0;
+    uint64_t m = (p1 << (9 - n)) | (w0 >> (23 + n));              // 53 bits
+    m += ((w0 << (9 - n)) | ((uint32_t)m & 1u)) > 0x80000000u;   // to nearest even; a carry is right
+    const uint64_t e = (uint64_t)(ev + es + n - 128u) << 52;      // the mantissa's leading bit adds one
+    return __longlong_as_double((long long)((e + m) | ((uint64_t)((u ^ hi) & 0x80000000u) << 32)));
+}
+
 // Store `vw` (1, 2 or 4) values to consecutive elements starting at `off`;
 // `s` is the output scale zinfo[1] for the EPI_OUT_* modes (read once per
 // tile by the caller).
@@ -161,12 +187,12 @@ __device__ __forceinline__ void store_run_f32(const EpiParams &e, uint64_t off, 
         case EPI_OUT_F64: {
             double *o = (double *)e.out + off;
             if (vw == 4) {
-                ((double2 *)o)[0] = make_double2(v[0] * s, v[1] * s);
-                ((double2 *)o)[1] = make_double2(v[2] * s, v[3] * s);
+                ((double2 *)o)[0] = make_double2(f32_times_f64(v[0], s), f32_times_f64(v[1], s));
+                ((double2 *)o)[1] = make_double2(f32_times_f64(v[2], s), f32_times_f64(v[3], s));
             } else if (vw == 2) {
-                ((double2 *)o)[0] = make_double2(v[0] * s, v[1] * s);
+                ((double2 *)o)[0] = make_double2(f32_times_f64(v[0], s), f32_times_f64(v[1], s));
             } else {
-                o[0] = v[0] * s;
+                o[0] = f32_times_f64(v[0], s);
             }
         } break;
         default: break;
@@ -272,7 +298,7 @@ __device__ __forceinline__ void store_vals(const EpiParams &e, uint64_t off, con
         double w[VW];
         double *o = (double *)e.out + off;
 #pragma unroll
-        for (int i = 0; i < VW; ++i) w[i] = MODE == EPI_OUT_F64 ? (double)v[i] * sd : (double)v[i];
+        for (int i = 0; i < VW; ++i) w[i] = MODE == EPI_OUT_F64 ? f32_times_f64(v[i], sd) : f32_to_f64(v[i]);
         if constexpr (MODE == EPI_F64_ADD) {
 #pragma unroll
             for (int i = 0; i < VW; i += 2) {

@@ -441,7 +441,7 @@ __global__ void ksplit_reduce_kernel(const float *part, int ksplit, int64_t n, i
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         double v = 0.0;
-        for (int s = 0; s < ksplit; ++s) v += (double)part[s * n + i];
+        for (int s = 0; s < ksplit; ++s) v += f32_to_f64(part[s * n + i]);
         switch (mode) {
             case EPI_OUT_F32: ((float *)out)[i] = (float)(v * sc); break;
             case EPI_OUT_F64: ((double *)out)[i] = v * sc; break;

@@ -117,13 +117,13 @@ __device__ __forceinline__ uint32_t stage_word(uint32_t t, uint32_t xmask) {
 }
 
 // Write a staged sub-tile (E results) to its destination: thread etid takes the
-// aligned fours t = 4 etid + 2048 n, element offset g_hi[t >> 7] + g_lo[t & 127].
+// aligned fours t = 4 etid + 2048 n, element offset g_hi[t >> 7] + g0 (g0 = g_lo[4 etid & 127]).
 template <int MODE>
 __device__ __forceinline__ void staged_write(const EpiTables *tb, const float *stg, const EpiParams &e, uint64_t base,
-                                             int E, int etid, uint32_t w0, uint32_t xmask, float sf, double sd) {
+                                             int E, int etid, uint32_t w0, uint64_t g0, uint32_t xmask, float sf, double sd) {
     __builtin_assume(__isShared(tb));
     __builtin_assume(__isShared(stg));
-    const uint64_t gb = base + tb->g_lo[(etid * 4) & 127];
+    const uint64_t gb = base + g0;
 #pragma unroll 4
     for (int t = etid * 4; t < E; t += 4 * EPI_THREADS) {
         // t = 4 etid + 2048 n: the words of its two parts XOR
@@ -406,6 +406,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         // this thread's first write-out word, and (staging warps) the words of
         // its row and of the bits of a column
         const uint32_t w0 = stage_word((uint32_t)etid * 4, P.xmask);
+        const uint64_t g0 = tb->g_lo[(etid * 4) & 127];  // its element offset
         const uint32_t wrow = stage_word(pdep32((uint32_t)row, e.lowRc), P.xmask) ^
                               stage_word(pdep32((uint32_t)wg * 32, e.lowCc), P.xmask);
         uint32_t wcol[5];
@@ -499,7 +500,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const float *cur = stgbuf[k & 1];
             const uint64_t base = tile_base_slot[k & 1];
 #define TQC_STAGED_WRITE(M) \
-    case M: staged_write<M>(tb, cur, e, base, E, etid, w0, P.xmask, sf, sc); break;
+    case M: staged_write<M>(tb, cur, e, base, E, etid, w0, g0, P.xmask, sf, sc); break;
             switch (e.mode) {
                 TQC_STAGED_WRITE(EPI_F32)
                 TQC_STAGED_WRITE(EPI_TF32)

@@ -157,6 +157,7 @@ std::vector<int> tile_candidates(const StepPlan &st, bool smallk) {
         c.push_back(UMMA_128x64);
         if (st.mb >= 7 && st.nb >= 7) c.push_back(UMMA_128x128_DEEP);
         if (st.mb >= 7 && st.nb >= 8) c.push_back(UMMA_128x256_DEEP);
+        if (st.mb >= 7 && st.nb >= 8) c.push_back(UMMA_128x256);
     } else {
         if (smallk && smallk_ok(st.mb, st.nb, st.kb, st.kblk)) c.push_back(SIMT_SMALLK);
         c.push_back(SIMT_64x64);
@@ -219,12 +220,17 @@ int default_step_tile(const StepPlan &st, int out_esize, bool smallk) {
         if (big) {
             const EpiParams e = make_epi(st.maskR, st.maskC, st.mb, st.nb, TileShape{7, 6});
             if (direct_store_efficiency(e, out_esize) >= 0.99) {
-#ifdef V_FILL
-                if (st.nb >= 8 && ((int64_t)1 << (st.mb + st.nb - 15)) < sm_count()) return UMMA_128x128_DEEP;
-#endif
-                return st.nb >= 8 ? UMMA_128x256_DEEP : UMMA_128x128_DEEP;
+                // (TF32 from K = 2^8 on: 128 x 128 also where 128 x 256 tiles would leave
+                // SMs without one, 2^11 x 2^10 results, K = 2^8: 16.4 -> 12.1 us)
+                const bool few = st.prec == TQC_PREC_TF32 && st.kb >= 8 && ((int64_t)1 << (st.mb + st.nb - 15)) < sm_count();
+                return st.nb >= 8 && !few ? UMMA_128x256_DEEP : UMMA_128x128_DEEP;
             }
         }
+        // staged, K >= 2^8 and a 128 x 256 tile for every SM: a third more
+        // multiply-adds per operand byte (2^19 x 2^9 results, K = 2^10 in TF32:
+        // 1200 -> 865 us; K = 2^8: 104 -> 99 us; K = 2^6: no faster)
+        if (st.mb >= 7 && st.nb >= 8 && st.kb >= 8 && ((int64_t)1 << (st.mb + st.nb - 15)) >= sm_count())
+            return UMMA_128x256;
         return st.nb >= 7 ? UMMA_128x128 : UMMA_128x64;
     }
     if (smallk && smallk_ok(st.mb, st.nb, st.kb, st.kblk)) {

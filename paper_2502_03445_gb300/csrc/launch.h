@@ -59,7 +59,9 @@ cudaError_t launch_ksplit_reduce(const float *part, int ksplit, int64_t n, int m
 
 // tcgen05 step (umma.cu)
 // *_DEEP: direct epilogue and a deeper operand ring, for steps with a long K loop
-enum UmmaCfg { UMMA_128x128 = 0, UMMA_128x64 = 1, UMMA_128x128_DEEP = 2, UMMA_128x256_DEEP = 3, UMMA_N_CFG = 4 };
+enum UmmaCfg {
+    UMMA_128x128 = 0, UMMA_128x64 = 1, UMMA_128x128_DEEP = 2, UMMA_128x256_DEEP = 3, UMMA_128x256 = 4, UMMA_N_CFG = 5
+};
 TileShape umma_tile(int cfg);
 // prec: TQC_PREC_BF16 / TQC_PREC_BF16X3 / TQC_PREC_TF32
 cudaError_t launch_umma_step(int cfg, int prec, const StepArgs &a, int *d_err, cudaStream_t s);

@@ -57,12 +57,12 @@ std::atomic<int> g_umma_stall{0};  // tqc_step_inject_stall
 
 
 struct UmmaParams {
-    int64_t n_tiles;
-    int64_t n_units;       // n_tiles * ksplit: unit u is split u / n_tiles of tile u % n_tiles
-    int64_t col_tiles;
+    int64_t n_units;       // tiles * ksplit: unit u is split u >> l_tiles of tile u mod 2^l_tiles
+    int32_t l_tiles;       // log2 of the tiles, and of the column tiles (both powers of
+    int32_t l_col;         // two: no divisions, each over 100 instructions, per tile)
     int64_t split_stride;  // elements between the FP32 partials of the splits
     int32_t ksplit;        // K ranges per tile (deep form only)
-    int32_t sw64;          // deep form: 64-byte swizzled k-blocks (half the K per stage, twice the stages)
+    int32_t sw64;          // 64-byte swizzled k-blocks (half the K per stage, twice the stages)
     int32_t kblk;          // operands K-blocked ([K / 64][rows][64]): 3-D copies
     int32_t k_blocks;
     int32_t vec;       // staged form: consecutive results of a row in one staging store (1, 2 or 4)
@@ -81,17 +81,19 @@ struct Cfg {
     static constexpr int A_BYTES = BM * 128;
     static constexpr int B_BYTES = BN * 128;
     static constexpr int STAGE_BYTES = PLANES * (A_BYTES + B_BYTES);
-    static constexpr int STAGES = DEEP ? 196608 / STAGE_BYTES : (KIND == K_BF16X3 ? 2 : (BN == 64 ? 6 : 4));
+    // bytes of the operand ring: the direct form has no staging buffers
+    static constexpr int RING = DEEP ? 196608 : (BN == 128 ? 131072 : (KIND == K_BF16X3 && BN == 64 ? 98304 : 147456));
     static constexpr int SUB_N = 64;               // epilogue sub-tile: 128 x 64
     static constexpr int STG_FLOATS = BM * SUB_N;
     static constexpr int STG_BYTES = DEEP ? 0 : 2 * STG_FLOATS * 4;  // two buffers (ping-pong)
     static constexpr int BAR_BYTES = 1024;
-    static constexpr int RING = STAGES * STAGE_BYTES;      // bytes of the operand ring
-    static constexpr int MAXST = DEEP ? 16 : STAGES;        // barrier slots of the ring
-    static constexpr int SMEM = 1024 + STAGES * STAGE_BYTES + STG_BYTES + (int)sizeof(EpiTables) + BAR_BYTES;
+    static constexpr int MAXST = 16;               // barrier slots of the ring
+    // k-blocks of 64 bytes: two stages of 128-byte ones would not fit
+    static constexpr bool SW64 = !DEEP && RING / STAGE_BYTES < 2;
+    static constexpr int SMEM = 1024 + RING + STG_BYTES + (int)sizeof(EpiTables) + BAR_BYTES;
     static constexpr int TMEM_COLS = 2 * BN;
     static_assert(SMEM <= 232448, "shared memory per CTA");
-    static_assert(STAGES >= 2, "operand ring");
+    static_assert(RING / STAGE_BYTES >= (SW64 ? 1 : 2), "operand ring");
     // instruction descriptor: D = F32, A/B = BF16 (1) or TF32 (2), K-major, N >> 3, M >> 4
     static constexpr uint32_t IDESC = (1u << 4) | ((KIND == K_TF32 ? 2u : 1u) << 7) |
                                       ((KIND == K_TF32 ? 2u : 1u) << 10) | ((uint32_t)(BN >> 3) << 17) |
@@ -99,6 +101,16 @@ struct Cfg {
 };
 
 
+
+// k-blocks [kb0, kb1) of split sp.
+__device__ __forceinline__ void k_range(const UmmaParams &P, int64_t sp, int &kb0, int &kb1) {
+    kb0 = 0;
+    kb1 = P.k_blocks;
+    if (P.ksplit > 1) {
+        kb0 = (int)(sp * P.k_blocks / P.ksplit);
+        kb1 = (int)((sp + 1) * P.k_blocks / P.ksplit);
+    }
+}
 
 // Staged epilogue.  A 128 x 64 sub-tile is staged in its own destination
 // order: result t (the sub-tile's result bits, compacted, lowest first) at word
@@ -156,7 +168,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const bool bres = DEEP && P.bres;
     // bytes of K per operand row in one k-block (the swizzle span), and the
     // plane sizes of a stage
-    const int rowb = (DEEP && P.sw64) ? 64 : 128;
+    const int rowb = ((DEEP || C::SW64) && P.sw64) ? 64 : 128;
     const bool kblk = P.kblk != 0;
     const int bk = rowb / C::ELEM, ksl = rowb / 32;  // elements of K per k-block; 32-byte MMA slices
     const int ab = BM * rowb, bb = BN * rowb;
@@ -212,6 +224,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         // ------------------------------------------------ TMA producer
         if (lane == 0) {
             int64_t it = 0;
+            int ps = 0;        // stage and phase of copy `it`
+            uint32_t pph = 0;
             bool ok = true, skipped0 = false;
             if (bres) {  // the one B tile, loaded once
                 mbar_expect_tx(bfull, C::PLANES * bb);
@@ -219,15 +233,19 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 if (KIND == K_BF16X3) tma_load_op(bsm + bb, &tBl, 0, 0, bfull, kblk);
             }
             for (int64_t u = blockIdx.x; ok && u < P.n_units; u += gridDim.x) {
-                const int64_t sp = u / P.n_tiles, tile = u - sp * P.n_tiles;
-                const int rt = (int)(tile / P.col_tiles), ct = (int)(tile - (int64_t)rt * P.col_tiles);
-                const int kb0 = (int)(sp * P.k_blocks / P.ksplit), kb1 = (int)((sp + 1) * P.k_blocks / P.ksplit);
+                const int64_t sp = u >> P.l_tiles, tile = u - (sp << P.l_tiles);
+                const int rt = (int)(tile >> P.l_col), ct = (int)(tile - ((int64_t)rt << P.l_col));
+                int kb0, kb1;
+                k_range(P, sp, kb0, kb1);
                 for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                    const int s = (int)(it % nst);
-                    const uint32_t ph = (uint32_t)((it / nst) & 1);
-                    if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
+                    const int s = ps;
+                    if (!mbar_wait(&empty[s], pph ^ 1u, abort_flag)) {
                         ok = false;
                         break;
+                    }
+                    if (++ps == nst) {
+                        ps = 0;
+                        pph ^= 1u;
                     }
                     if (P.stall && blockIdx.x == 0 && it == 0) {
                         // test hook: stage 0 never fills, so the MMA issuer's bounded wait gives up
@@ -266,15 +284,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         if (lane == 0) {
-            int64_t it = 0, lt = 0;
+            int64_t lt = 0;
+            int ms = 0;        // stage and phase of the next k-block
+            uint32_t mph = 0;
             bool ok = true;
             if (bres) {
                 ok = mbar_wait(bfull, 0, abort_flag);
                 tc_fence_after();
             }
             for (int64_t u = blockIdx.x; ok && u < P.n_units; u += gridDim.x, ++lt) {
-                const int64_t sp = u / P.n_tiles;
-                const int kb0 = (int)(sp * P.k_blocks / P.ksplit), kb1 = (int)((sp + 1) * P.k_blocks / P.ksplit);
+                int kb0, kb1;
+                k_range(P, u >> P.l_tiles, kb0, kb1);
                 const int acc = (int)(lt & 1);
                 const uint32_t aph = (uint32_t)((lt >> 1) & 1);
                 if (!mbar_wait(&tempty[acc], aph ^ 1u, abort_flag)) {
@@ -283,12 +303,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 }
                 tc_fence_after();
                 const uint32_t d = tmem_base + (uint32_t)(acc * BN);
-                for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                    const int s = (int)(it % nst);
-                    const uint32_t ph = (uint32_t)((it / nst) & 1);
-                    if (!mbar_wait(&full[s], ph, abort_flag)) {
+                for (int kb = kb0; kb < kb1; ++kb) {
+                    const int s = ms;
+                    if (!mbar_wait(&full[s], mph, abort_flag)) {
                         ok = false;
                         break;
+                    }
+                    if (++ms == nst) {
+                        ms = 0;
+                        mph ^= 1u;
                     }
                     tc_fence_after();
                     const uint32_t a0 = smem_u32(stages + s * sbytes);
@@ -353,9 +376,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             __syncwarp();
             if (*abort_flag) break;
             tc_fence_after();
-            const int64_t sp = u / P.n_tiles, tile = u - sp * P.n_tiles;
-            const uint64_t rt = (uint64_t)(tile / P.col_tiles);
-            const uint64_t ct = (uint64_t)(tile - (int64_t)rt * P.col_tiles);
+            const int64_t sp = u >> P.l_tiles, tile = u - (sp << P.l_tiles);
+            const uint64_t rt = (uint64_t)tile >> P.l_col;
+            const uint64_t ct = (uint64_t)tile - (rt << P.l_col);
             // sub-tile column index ct * SUBS + h: the h bits are the lowest bits of highC (in coff);
             // split sp stores its partial sp * split_stride elements further on
             const uint64_t base = (warp_pdep64(rt, e.highR) | warp_pdep64(ct * SUBS, e.highC)) +
@@ -415,7 +438,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const double sc = (e.mode == EPI_OUT_F32 || e.mode == EPI_OUT_F64) ? e.zinfo[1] : 1.0;
         const float sf = (float)sc;
         const int64_t my_tiles =
-            (int64_t)blockIdx.x < P.n_tiles ? (P.n_tiles - 1 - (int64_t)blockIdx.x) / gridDim.x + 1 : 0;
+            (int64_t)blockIdx.x < P.n_units ? (P.n_units - 1 - (int64_t)blockIdx.x) / gridDim.x + 1 : 0;  // (unsplit)
         const int64_t n_sub = my_tiles * SUBS;
         // stage sub-tile k into buffer k & 1 (staging warps only); returns false on abort
         auto stage_sub = [&](int64_t k) {
@@ -468,8 +491,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         // l (and l + 32) of the row / column tile index, then an OR reduction.
         auto sub_base_warp = [&](int64_t k) {
             const int64_t tile = (int64_t)blockIdx.x + (k / SUBS) * gridDim.x;
-            const uint64_t rt = (uint64_t)(tile / P.col_tiles);
-            const uint64_t ct = (uint64_t)((tile - (int64_t)rt * P.col_tiles) * SUBS + k % SUBS);
+            const uint64_t rt = (uint64_t)tile >> P.l_col;
+            const uint64_t ct = ((uint64_t)tile - (rt << P.l_col)) * SUBS + (uint64_t)(k % SUBS);
             uint64_t v = 0;
 #pragma unroll
             for (int hw = 0; hw < 2; ++hw) {
@@ -619,8 +642,8 @@ cudaError_t launch_kind(const StepArgs &a, int *d_err, cudaStream_t s) {
     // as many copies are in flight ahead of the tensor pipe.  Not for rows
     // longer than 64 KB: a box then spans many pages, and twice the boxes
     // per byte cost more in address translation than the deeper ring gains.
-    const bool sw64 = DEEP && KIND != K_TF32 && !a.kblk && K >= ((uint64_t)1 << SW64_MIN_LOG2_K) &&
-                      K * C::ELEM <= ((uint64_t)1 << 16);
+    const bool sw64 = C::SW64 || (DEEP && KIND != K_TF32 && !a.kblk && K >= ((uint64_t)1 << SW64_MIN_LOG2_K) &&
+                                  K * C::ELEM <= ((uint64_t)1 << 16));
     const uint32_t bk = (sw64 ? 64 : 128) / C::ELEM;
     if (K < (uint64_t)bk) return cudaErrorInvalidValue;
     CUtensorMap tA, tB, tAl, tBl;
@@ -638,9 +661,9 @@ cudaError_t launch_kind(const StepArgs &a, int *d_err, cudaStream_t s) {
     p.epi = a.epi;
     // MMA tiles are 128 x BN; the epilogue parameters describe 128 x 64 sub-tiles
     if (BN >= 128 && a.nb < lbn) return cudaErrorInvalidValue;
-    const int64_t row_tiles = (int64_t)1 << (a.mb - a.epi.a_bits);
-    p.col_tiles = a.nb >= lbn ? (int64_t)1 << (a.nb - lbn) : 1;
-    p.n_tiles = row_tiles * p.col_tiles;
+    p.l_col = a.nb >= lbn ? a.nb - lbn : 0;
+    p.l_tiles = a.mb - a.epi.a_bits + p.l_col;
+    const int64_t n_tiles = (int64_t)1 << p.l_tiles;
     p.k_blocks = (int)(K / bk);
     p.sw64 = sw64;
     p.kblk = kb3;
@@ -649,9 +672,9 @@ cudaError_t launch_kind(const StepArgs &a, int *d_err, cudaStream_t s) {
     if (a.ksplit < 1 || a.ksplit > p.k_blocks || (a.ksplit > 1 && (!DEEP || a.epi.mode != EPI_F32)))
         return cudaErrorInvalidValue;
     p.ksplit = a.ksplit;
-    p.n_units = p.n_tiles * a.ksplit;
+    p.n_units = n_tiles * a.ksplit;
     p.split_stride = a.ksplit > 1 ? a.split_stride : 0;
-    p.bres = DEEP && p.k_blocks == 1 && p.col_tiles == 1;
+    p.bres = DEEP && p.k_blocks == 1 && p.l_col == 0;
     p.vec = (a.epi.lowCc & 3u) == 3u ? 4 : ((a.epi.lowCc & 1u) ? 2 : 1);
     p.xmask = stage_swizzle(a.epi, p.vec);
     p.err = d_err;
@@ -704,6 +727,7 @@ TileShape umma_tile(int cfg) {
 cudaError_t launch_umma_step(int cfg, int prec, const StepArgs &a, int *d_err, cudaStream_t s) {
     switch (cfg) {
         case UMMA_128x64: return launch_bn<64, false>(prec, a, d_err, s);
+        case UMMA_128x256: return launch_bn<256, false>(prec, a, d_err, s);
         case UMMA_128x128: return launch_bn<128, false>(prec, a, d_err, s);
         case UMMA_128x128_DEEP: return launch_bn<128, true>(prec, a, d_err, s);
         case UMMA_128x256_DEEP: return launch_bn<256, true>(prec, a, d_err, s);

@@ -200,7 +200,7 @@ TQC_API tqc_status tqc_plan_step(tqc_plan_t plan, int32_t step, int32_t *log2_m,
  * the full length needed, excluding the NUL, or -1 on a bad handle.  Each
  * step lists its shape, class, precision, result layout, tile configuration
  * ("tile": CUDA-core 0 = 64 x 64, 1 = 128 x 128, 2 = 128 x 64, 3 = the
- * small-K tile; tcgen05 0 = 128 x 128, 1 = 128 x 64, 4 = 128 x 256, and
+ * small-K tile, 4 = 32 x 32; tcgen05 0 = 128 x 128, 1 = 128 x 64, 4 = 128 x 256, and
  * with the direct epilogue 2 = 128 x 128, 3 = 128 x 256), "ksplit" (K ranges run by
  * separate CTAs, 1 = none) and "kblk" (1 = its operands are stored
  * K-blocked, [K / 64][rows][64], for rows over 64 KB; fixed by the plan).

@@ -161,6 +161,7 @@ std::vector<int> tile_candidates(const StepPlan &st, bool smallk) {
     } else {
         if (smallk && smallk_ok(st.mb, st.nb, st.kb, st.kblk)) c.push_back(SIMT_SMALLK);
         c.push_back(SIMT_64x64);
+        if (st.kb >= 4 && !st.kblk) c.push_back(SIMT_32x32);
         if (st.mb >= 7 && st.nb >= 6) c.push_back(SIMT_128x64);
         if (st.mb >= 7 && st.nb >= 7) c.push_back(SIMT_128x128);
     }
@@ -243,11 +244,15 @@ int default_step_tile(const StepPlan &st, int out_esize, bool smallk) {
             return SIMT_128x128;
         return SIMT_SMALLK;
     }
-    // K >= 16: too few 128 x 128 tiles to give every SM one run as 64 x 64
-    // (four times the CTAs, a quarter of a tile's latency: a 17-qubit FP32
-    // contract 242 -> 72 us together with simt_gemm_f32)
-    if (st.kb >= 4 && st.mb >= 6 && st.nb >= 6 && ((int64_t)1 << (st.mb + st.nb)) < ((int64_t)sm_count() << 14))
-        return SIMT_64x64;
+    // K >= 16, not whole 64 x 64 tiles, or fewer of them than SMs: 32 x 32 tiles
+    // (10-13-qubit FP32 contracts 47-109 -> 15-21 us); too few 128 x 128 tiles to give every SM one: 64 x 64 (four
+    // times the CTAs, a quarter of a tile's latency: a 17-qubit FP32 contract
+    // 242 -> 72 us together with simt_gemm_f32)
+    if (st.kb >= 4) {
+        const int64_t results = (int64_t)1 << (st.mb + st.nb);
+        if (st.mb < 6 || st.nb < 6 || results < ((int64_t)sm_count() << 12)) return SIMT_32x32;
+        if (results < ((int64_t)sm_count() << 14)) return SIMT_64x64;
+    }
     return (st.mb >= 7 && st.nb >= 7) ? SIMT_128x128 : (st.mb >= 7 && st.nb >= 6 ? SIMT_128x64 : SIMT_64x64);
 }
 

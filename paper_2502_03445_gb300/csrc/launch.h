@@ -9,7 +9,8 @@ namespace tqc {
 
 // CUDA-core step tiles (FP32), chosen by the autotuner; SIMT_SMALLK: the
 // write-out-shaped tile of steps with K = 1, 4 or 16 (smallk.cuh)
-enum SimtCfg { SIMT_64x64 = 0, SIMT_128x128 = 1, SIMT_128x64 = 2, SIMT_SMALLK = 3, SIMT_N_CFG = 4 };
+// SIMT_32x32: small steps with K >= 16
+enum SimtCfg { SIMT_64x64 = 0, SIMT_128x128 = 1, SIMT_128x64 = 2, SIMT_SMALLK = 3, SIMT_32x32 = 4, SIMT_N_CFG = 5 };
 
 struct TileShape {
     int log_bm, log_bn;

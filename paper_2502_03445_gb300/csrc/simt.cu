@@ -277,6 +277,98 @@ __global__ void __launch_bounds__((BM / TM) * (BN / 8), MINB)
     }
 }
 
+__device__ __forceinline__ void copy16(float *dst, const float *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+// Small steps with K >= 16 (at most 32 x 32 results per tile, down to one row
+// or column): bound by the latency of a tile's K loop, so that loop has three
+// 64-k chunks of operands on their way (asynchronous copies, K-major rows) and
+// a tile is spread over all 256 threads, 2 x 2 results or one each.  The k order
+// and the multiply-adds are those of simt_step_f32: bit-identical.  A step of 2^5 x
+// 2^5 results with K = 4^5: 109 -> 16 us of a whole contract (one chunk of 16 k
+// waited for at a time before).
+constexpr int SS_STAGES = 3, SS_KC = 64, SS_P = SS_KC + 4, SS_PS = 36;
+template <int T>
+__device__ __forceinline__ void small_chunk(const float *As, const float *Bs, int rt, int ct, int rs, int cs, int n4,
+                                            float (&acc)[T][T]) {
+#pragma unroll 4
+    for (int k = 0; k < n4; ++k) {
+        float4 a[T], b[T];
+#pragma unroll
+        for (int i = 0; i < T; ++i) a[i] = *(const float4 *)(As + (rt + i * rs) * SS_P + 4 * k);
+#pragma unroll
+        for (int j = 0; j < T; ++j) b[j] = *(const float4 *)(Bs + (ct + j * cs) * SS_P + 4 * k);
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int j = 0; j < T; ++j) {
+                acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+                acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+                acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+            }
+    }
+}
+template <int T>
+__global__ void __launch_bounds__(256) simt_small_f32(StepArgs args, int64_t n_tiles, int l_col) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    EpiTables *tb = (EpiTables *)smem_raw;
+    float *ring = (float *)(smem_raw + sizeof(EpiTables));  // stages of [32][SS_P] A rows, [32][SS_P] B rows
+    float *stg = ring + SS_STAGES * 64 * SS_P;
+    const EpiParams &e = args.epi;
+    const int a = e.a_bits, b = e.b_bits, Me = 1 << a, Ne = 1 << b;
+    const int64_t K = 1ll << args.kb;
+    const int kc = args.kb < 6 ? 1 << args.kb : SS_KC, chunks = (int)(K / kc), lp = (args.kb < 6 ? args.kb : 6) - 2;
+    const int tid = threadIdx.x;
+    const int rs = Me / T, cs = Ne / T;  // a thread's rows and columns are this far apart
+    const int ct = tid & (cs - 1), rt = tid / cs;
+    const bool active = tid < rs * cs;
+    epi_tables_init(tb, e, true, SS_PS, tid, 256);
+    const int gm = gather_mode(e.lowCc);
+    pdl_launch();
+    pdl_wait();
+    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const int64_t r0 = tile >> l_col, c0 = tile - (r0 << l_col);
+        const float *A = (const float *)args.A + (r0 << a) * K, *B = (const float *)args.B + (c0 << b) * K;
+        auto fetch = [&](int c) {
+            if (c < chunks) {
+                float *st = ring + (c % SS_STAGES) * 64 * SS_P;
+                for (int f = tid; f < (Me + Ne) << lp; f += 256) {  // 16-byte pieces
+                    const int row = f >> lp, k4 = f & ((1 << lp) - 1);
+                    if (row < Me) copy16(st + row * SS_P + 4 * k4, A + row * K + (int64_t)c * kc + 4 * k4);
+                    else copy16(st + (32 + row - Me) * SS_P + 4 * k4, B + (row - Me) * K + (int64_t)c * kc + 4 * k4);
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        float acc[T][T];
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int j = 0; j < T; ++j) acc[i][j] = 0.f;
+        for (int c = 0; c < SS_STAGES; ++c) fetch(c);
+        for (int c = 0; c < chunks; ++c) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(SS_STAGES - 1) : "memory");
+            __syncthreads();
+            const float *st = ring + (c % SS_STAGES) * 64 * SS_P;
+            if (active) small_chunk<T>(st, st + 32 * SS_P, rt, ct, rs, cs, kc / 4, acc);
+            __syncthreads();
+            fetch(c + SS_STAGES);
+        }
+        if (active) {
+#pragma unroll
+            for (int i = 0; i < T; ++i)
+#pragma unroll
+                for (int j = 0; j < T; ++j) stg[(rt + i * rs) * SS_PS + ct + j * cs] = acc[i][j];
+        }
+        __syncthreads();
+        epi_readout(tb, stg, e, tile_base(e, (uint64_t)r0, (uint64_t)c0), Me * Ne, tid, 256, gm);
+        __syncthreads();
+    }
+}
+
 // Small-K step (smallk.cuh): one 128-thread CTA per tile slot, one kernel
 // per K, tile width and orientation (each with its own register budget);
 // when the tiles are staged, the staging tables are built once per CTA.
@@ -501,6 +593,24 @@ cudaError_t launch_gemm(const StepArgs &step, cudaStream_t s) {
     return launch_pdl(simt_gemm_f32<BM, BN, TM, MINB>, grid, NT, smem, s, a, n_tiles, col_tiles, smallk_layout(a.epi));
 }
 
+cudaError_t launch_small(const StepArgs &a, cudaStream_t s) {
+    if (a.kb < 4 || a.epi.a_bits > 5 || a.epi.b_bits > 5 || a.kblk) return cudaErrorInvalidValue;
+    const size_t smem = sizeof(EpiTables) + (size_t)(SS_STAGES * 64 * SS_P + 32 * SS_PS) * sizeof(float);
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(simt_small_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(simt_small_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    const int l_col = a.nb - a.epi.b_bits;
+    const int64_t n_tiles = (1ll << (a.mb - a.epi.a_bits)) << l_col;
+    const int64_t grid = std::min<int64_t>(n_tiles, (int64_t)sm_count() * 3);
+    auto *kernel = a.epi.a_bits + a.epi.b_bits <= 8 ? simt_small_f32<1> : simt_small_f32<2>;
+    return launch_pdl(kernel, grid, 256, smem, s, a, n_tiles, l_col);
+}
+
 }  // namespace
 
 int sm_count() {
@@ -517,6 +627,7 @@ TileShape simt_tile(int cfg) {
     switch (cfg) {
         case SIMT_128x128: return {7, 7};
         case SIMT_128x64: return {7, 6};
+        case SIMT_32x32: return {5, 5};
         default: return {6, 6};
     }
 }
@@ -645,6 +756,7 @@ cudaError_t launch_smallk(const StepArgs &a, cudaStream_t s) {
 cudaError_t launch_simt_step(int cfg, const StepArgs &a, cudaStream_t s) {
     switch (cfg) {
         case SIMT_SMALLK: return launch_smallk(a, s);
+        case SIMT_32x32: return launch_small(a, s);
         case SIMT_128x128:
             if (a.kb >= 4 && a.epi.a_bits == 7 && a.epi.b_bits == 7) return launch_gemm<128, 128, 8, 2>(a, s);
             return launch_cfg<128, 128, 8, 8>(a, s);

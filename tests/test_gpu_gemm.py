@@ -1,5 +1,5 @@
 """CUDA-core FP32 steps with K >= 16 (whole 128 x 128, 128 x 64 and 64 x 64
-tiles, 16 k at a time) against the FP64 oracle, element by element.
+tiles, 16 k at a time; 32 x 32 tiles or parts of them, 64 k at a time) against the FP64 oracle, element by element.
 
 Bound: a result is one chain of K fused multiply-adds (K roundings), its
 operands are FP64 inputs rounded once each, and the scale and the scaled
@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 from paper_2502_03445_gb300 import tqc  # noqa: E402
 
-SIMT_64x64, SIMT_128x128, SIMT_128x64 = 0, 1, 2
+SIMT_64x64, SIMT_128x128, SIMT_128x64, SIMT_32x32 = 0, 1, 2, 4
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -28,7 +28,9 @@ def _cuda():
 
 # (rows, columns, cuts, where the row qubits sit, tile): one chunk of K (16)
 # and several; one tile, fewer and more tiles than the grid
-CASES = [(6, 6, 3, "low", SIMT_64x64), (7, 6, 3, "mixed", SIMT_64x64), (9, 7, 4, "high", SIMT_64x64),
+CASES = [(6, 6, 3, "low", SIMT_32x32), (7, 6, 3, "mixed", SIMT_32x32), (9, 7, 4, "high", SIMT_32x32),
+         (1, 0, 3, "low", SIMT_32x32), (4, 3, 4, "mixed", SIMT_32x32), (2, 7, 5, "high", SIMT_32x32),
+         (14, 1, 2, "mixed", SIMT_32x32), (16, 5, 3, "mixed", SIMT_32x32),
          (15, 6, 3, "mixed", SIMT_64x64), (14, 6, 2, "high", SIMT_64x64),
          (16, 6, 3, "mixed", SIMT_128x64), (17, 6, 2, "high", SIMT_128x64), (11, 11, 2, "low", SIMT_128x128),
          (13, 10, 3, "mixed", SIMT_128x128), (15, 7, 4, "high", SIMT_128x128), (5, 9, 3, "mixed", None)]

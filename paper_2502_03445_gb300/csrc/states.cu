@@ -956,10 +956,12 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
         }
         for (int j = 0; j < p->m; ++j) P.leaf[j].table = (const float *)((char *)p->d_tab + p->tab_off[(size_t)j]);
         // the list, and for the sort: permuted states, ranks, sorted states,
-        // their places in the list, counters and their block sums
+        // their places in the list, counters (for any split: a shorter list
+        // never needs more) and their block sums
         const int64_t n8 = align4(n) * 8, n4 = align4(n) * 4, n_keys = P.key_bits ? (int64_t)1 << P.key_bits : 0;
         const int64_t n_sums = (n_keys + SCAN_PER_CTA - 1) / SCAN_PER_CTA;
-        const int64_t need = n8 + (P.key_bits ? 2 * n8 + 2 * n4 + align4(n_keys) * 4 + align4(n_sums) * 4 : 0);
+        const int64_t max_keys = (int64_t)1 << std::min(ST_MAX_KEY_BITS, p->net->n_qubits);
+        const int64_t need = 3 * n8 + 2 * n4 + align4(max_keys) * 4 + align4(max_keys / SCAN_PER_CTA + 1) * 4;
         if (need > p->states_bytes) {
             if (p->d_states) cudaFree(p->d_states);
             p->d_states = nullptr;

@@ -79,3 +79,26 @@ def test_intermediate_and_sliced_steps(pat, sliced):
     check(net, n, out, 2 * (2.0 ** -14 + 256 * 2.0 ** -23))
     p.close()
     h.close()
+
+
+@pytest.mark.parametrize("pat", ["rows01", "cols01", "row_col", "col_row"])
+@pytest.mark.parametrize("prec", ["bf16x3", "tf32", "bf16"])
+def test_wide_tiles(pat, prec):
+    """128 x 256 staged tiles (K = 256, a tile for every SM); split BF16 takes
+    64-byte k-blocks there."""
+    n = 23
+    first = PATTERNS[pat]
+    first = sorted(first + [q for q in range(13, 21)])
+    rest = [q for q in range(n) if q not in first]
+    net = tensors.pseudo_physical_network(n, [(0, 1)] * 4, [first, rest], 8200)
+    h = tqc.Network(net)
+    p = tqc.Plan(h, precision=prec)
+    out = torch.full((p.out_elems,), float("nan"), dtype=torch.float32, device="cuda")
+    p.contract(out)
+    torch.cuda.synchronize()
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert p.describe()["steps"][0]["tile"] in (3, 4)  # 3: stores that fill whole sectors
+    # BF16: 8-bit operands, 2^-7 in all
+    check(net, n, out, {"bf16x3": 2.0 ** -14 + 256 * 2.0 ** -23, "tf32": 2.0 ** -9, "bf16": 2.0 ** -7}[prec])
+    p.close()
+    h.close()

@@ -85,8 +85,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 
 // FP32 -> FP64 (exact) and the FP64 product (double)v * s, rounded to nearest
 // even, in integer arithmetic for normal values: the conversion and the
-// multiplication run at two a clock per SM, which bound every FP64 output (2^28
-// results of a K = 4 step: F64FIG).  s is a normal value whose exponent keeps
+// multiplication run at two a clock per SM, which bound every FP64 output (2^29
+// results of a K = 2^8 step: 2.42 -> 1.57 ms).  s is a normal value whose exponent keeps
 // the product normal; zero, subnormal, infinite and NaN v take the instructions.
 __device__ __forceinline__ double f32_to_f64(float v) {
     const uint32_t u = __float_as_uint(v), e = (u >> 23) & 0xffu;
@@ -324,16 +324,14 @@ __device__ __forceinline__ void store_vals(const EpiParams &e, uint64_t off, con
 // nthreads is a multiple of 32: a thread's t advances by a multiple of 128,
 // so its low table entries (t & 127) are read once, not once per run (the
 // lanes of a warp read them at a stride of four entries: bank conflicts).
-// The output mode is dispatched once per tile (MODE >= 0), or per store
-// (MODE = -1: fewer registers, for kernels with a tight budget).  The tables
-// and the staged tile are in shared memory.
+// The output mode is dispatched once per tile.  The tables and the staged tile
+// are in shared memory.
 template <int MODE>
 __device__ __forceinline__ void epi_readout_m(const EpiTables *tb, const float *stg, const EpiParams &e,
                                               uint64_t base, int E, int tid, int nthreads, int gmode) {
     __builtin_assume(__isShared(tb));
     __builtin_assume(__isShared(stg));
-    const int mode = MODE >= 0 ? MODE : e.mode;
-    const double sd = (mode == EPI_OUT_F32 || mode == EPI_OUT_F64) ? e.zinfo[1] : 1.0;
+    const double sd = (MODE == EPI_OUT_F32 || MODE == EPI_OUT_F64) ? e.zinfo[1] : 1.0;
     const float sf = (float)sd;
     if (e.L >= 2) {
         const int tl = (tid * 4) & 127;
@@ -369,21 +367,14 @@ __device__ __forceinline__ void epi_readout_m(const EpiTables *tb, const float *
                 v[2] = sp[l2];
                 v[3] = sp[l3];
             }
-            if constexpr (MODE >= 0) store_vals<MODE, 4>(e, gbase + tb->g_hi[t >> 7], v, sf, sd);
-            else store_run_f32(e, gbase + tb->g_hi[t >> 7], v, 4, sd);
+            store_vals<MODE, 4>(e, gbase + tb->g_hi[t >> 7], v, sf, sd);
         }
     } else {
         for (int t = tid; t < E; t += nthreads) {
             float v = stg[tb->s_hi[t >> 7] + tb->s_lo[t & 127]];
-            if constexpr (MODE >= 0) store_vals<MODE, 1>(e, base + tb->g_hi[t >> 7] + tb->g_lo[t & 127], &v, sf, sd);
-            else store_run_f32(e, base + tb->g_hi[t >> 7] + tb->g_lo[t & 127], &v, 1, sd);
+            store_vals<MODE, 1>(e, base + tb->g_hi[t >> 7] + tb->g_lo[t & 127], &v, sf, sd);
         }
     }
-}
-
-__device__ __forceinline__ void epi_readout_rt(const EpiTables *tb, const float *stg, const EpiParams &e,
-                                               uint64_t base, int E, int tid, int nthreads, int gmode) {
-    epi_readout_m<-1>(tb, stg, e, base, E, tid, nthreads, gmode);
 }
 
 __device__ __forceinline__ void epi_readout(const EpiTables *tb, const float *stg, const EpiParams &e,

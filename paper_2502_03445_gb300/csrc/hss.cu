@@ -39,7 +39,9 @@ namespace {
 // rank.  Bound by the tensor's bytes and, as closely, by the FP64 rate (two
 // multiply-adds a clock per SM).  The four tensors of the
 // 30-qubit grid (38 MB) in four calls: 151 -> 55 us (the sums of up to 586
-// partial sums per state were a serial chain in one thread of a second kernel).
+// partial sums per state were a serial chain in one thread of a second
+// kernel), 35 us with fewer states per warp where few CTAs would run (32 for
+// the 128-state tensor, now 128).
 template <typename V>
 __global__ void __launch_bounds__(256)
     hss_norms_kernel(const V *__restrict__ T, int64_t n_x, int64_t n_e, int lx, int wr, double *norm) {
@@ -108,11 +110,15 @@ __global__ void hss_gather_kernel(const V *T, int64_t n_x, int64_t n_e, const in
 template <typename V>
 cudaError_t launch_norms(const Node &nd, double *d_norms, cudaStream_t s) {
     const int64_t n_x = (int64_t)1 << nd.out_qubits.size(), n_e = (int64_t)1 << (2 * nd.cut_ids.size());
-    const int lx = (int)std::min<size_t>(5, nd.out_qubits.size());
+    int lx = (int)std::min<size_t>(5, nd.out_qubits.size());
     const int wr = (int)std::min<int64_t>(8, n_e);  // 1, 4 or 8
     // up to eight CTAs share the rows, while a lane has at least eight of them
     int ys = 1;
     while (ys < 8 && n_e >= ((int64_t)16 * wr * ys << (5 - lx))) ys *= 2;
+    // Few states leave SMs idle even so: a warp then takes more rows of fewer
+    // states, down to eight (a whole 32-byte sector of FP32), while a lane
+    // keeps the 16 rows that it loads at once.
+    while (lx > 3 && (n_x >> lx) * wr * ys < 8 * 152 && n_e >= ((int64_t)32 * wr * ys << (5 - lx))) --lx;
     const int64_t per = (int64_t)(8 / wr) << lx;  // states of a CTA
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((n_x + per - 1) / per), (unsigned)ys);

@@ -24,7 +24,7 @@ def _cuda():
 
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
 @pytest.mark.parametrize("cuts,outs", [(0, 3), (0, 9), (1, 0), (1, 12), (2, 5), (3, 1), (3, 6), (4, 7), (5, 2), (5, 11),
-                                       (6, 0), (7, 5)])
+                                       (6, 0), (6, 4), (6, 7), (6, 10), (7, 5)])
 def test_norms(cuts, outs, dtype):
     rng = np.random.Generator(np.random.PCG64(100 * cuts + outs))
     mine = list(range(cuts))

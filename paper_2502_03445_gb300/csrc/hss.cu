@@ -40,8 +40,8 @@ namespace {
 // multiply-adds a clock per SM).  The four tensors of the
 // 30-qubit grid (38 MB) in four calls: 151 -> 55 us (the sums of up to 586
 // partial sums per state were a serial chain in one thread of a second
-// kernel), 35 us with fewer states per warp where few CTAs would run (32 for
-// the 128-state tensor, now 128).
+// kernel), 48 us with fewer states per warp where few CTAs would run (32 for
+// the 128-state tensor, now 128); 35 us when the tensors are still in L2.
 template <typename V>
 __global__ void __launch_bounds__(256)
     hss_norms_kernel(const V *__restrict__ T, int64_t n_x, int64_t n_e, int lx, int wr, double *norm) {

@@ -839,7 +839,7 @@ cudaError_t launch_ingest(const IngestArgs *g, int n, cudaStream_t s) {
             if (a.reduce_bits > 0) {
                 // a CTA per destination when a warp each would leave SMs idle
                 a.vec = a.nbits < 10 && a.reduce_bits >= 8 ? INGEST_THREADS : 32;
-                threads = a.vec << a.nbits;
+                threads = (int64_t)a.vec << a.nbits;  // (2^5 threads for each of 2^26 destinations and more)
             } else {
                 ingest_vec(a);
                 threads = (1ll << a.nbits) / a.vec;

@@ -124,3 +124,36 @@ def test_total_mass(n, edges, counts, sliced):
     assert abs(z - oracle.total_mass(net)) <= 2 * np.log2(steps) * 2.0 ** -52 * oracle.total_mass(absnet) * len(nodes) * 8
     p.close()
     h.close()
+
+
+def test_total_mass_of_a_leaf_with_13_cuts():
+    """2^26 destinations of a summed leaf: 2^31 threads wanted, more than 32
+    bits hold, must still give the launch its whole grid and not one CTA
+    (about 2^23 dependent rounds of a warp, seconds; the whole contract moves
+    2 GB, a few milliseconds)."""
+    edges = [(0, 1)] * 5 + [(0, 2)] * 4 + [(0, 3)] * 4
+    outs = [[0], [1, 2], [3, 4], [5]]
+    rng = np.random.Generator(np.random.PCG64(26))
+    nodes = []
+    for j, o in enumerate(outs):
+        cuts = [(c, e.index(j)) for c, e in enumerate(edges) if j in e]
+        nodes.append(Node(o, [c for c, _ in cuts], [r for _, r in cuts],
+                          rng.random((4 ** len(cuts)) << len(o), dtype=np.float32)))
+    t = [d.data.reshape(-1, 1 << len(d.out_qubits)).sum(1, dtype=np.float64) for d in nodes]
+    want = ((t[0].reshape(-1, 4 ** 4) @ t[3]).reshape(4 ** 5, 4 ** 4) @ t[2]) @ t[1] / 2 ** len(edges)
+    h = tqc.Network(Network(6, len(edges), nodes), dtype=tqc.F32)
+    p = tqc.Plan(h)
+    out = torch.empty(p.out_elems, dtype=torch.float32, device="cuda")
+    p.contract(out)
+    h.upload(3, nodes[3].data)  # the next call computes the mass again
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda.synchronize()
+    e0.record()
+    p.contract(out)
+    e1.record()
+    e1.synchronize()
+    z = p.contract(out, want_z=True)
+    assert abs(z - want) <= 1e-12 * want  # positive terms
+    assert e0.elapsed_time(e1) < 500, e0.elapsed_time(e1)
+    p.close()
+    h.close()

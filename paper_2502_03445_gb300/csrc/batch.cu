@@ -684,7 +684,9 @@ cudaError_t upload(T **dst, const std::vector<T> &v) {
     return cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice);
 }
 
-// Whether a batch can run on the plans as they are.
+// Whether a batch can run on the plans as they are.  Asked on every launch, of
+// a kept list too: a list scales by its plans' cached total masses, which an
+// upload makes those of other tensors.
 tqc_status check_plans(Plan *const *plans, int n) {
     for (int pi = 0; pi < n; ++pi) {
         const Plan &p = *plans[pi];
@@ -915,9 +917,9 @@ tqc_status tqc_contract_batch(const tqc_plan_t *plans, void *const *d_outs, int3
     }
     key.push_back((const void *)(intptr_t)g_inject_stall);
     key.push_back((const void *)(intptr_t)(int64_t)(std::min(g_tail_s, 1e6) * 1e9));
+    tqc_status st = check_plans(ps.data(), n);
+    if (st != TQC_OK) return st;
     if (!g_batch || key != g_batch->key) {
-        tqc_status st = check_plans(ps.data(), n);
-        if (st != TQC_OK) return st;
         auto it = std::find_if(g_pool.begin(), g_pool.end(), [&](const Batch &b) { return b.key == key; });
         if (it != g_pool.end()) {
             g_pool.splice(g_pool.begin(), g_pool, it);
@@ -972,7 +974,6 @@ tqc_status tqc_contract_batch(const tqc_plan_t *plans, void *const *d_outs, int3
     e = cudaEventRecord(g_tail_fork, s);
     for (int k = 0; k < TAIL_STREAMS && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(g_tail_ts[k], g_tail_fork, 0);
     if (e != cudaSuccess) return fail(TQC_ERR_CUDA, std::string("batch fork: ") + cudaGetErrorString(e));
-    tqc_status st = TQC_OK;
     for (size_t i = 0; i < bt.tails.size() && st == TQC_OK; ++i) {
         const BatchTail &t = bt.tails[i];
         st = exec_run_tail(*t.p, t.first, t.out, g_tail_ts[bt.tail_stream[i]]);

@@ -76,3 +76,25 @@ def test_destroyed_and_changed_plans():
         p.close()
         h.close()
     tqc.batch_status()
+
+
+def test_same_list_refused_after_an_upload():
+    """The last launched list, launched again: its plans are checked as any
+    other's (the cached total mass is that of the tensors before)."""
+    a, b = make(7200), make(7201)
+    lst = [[x[1] for x in (a, b)], [x[3] for x in (a, b)]]
+    for _ in range(2):
+        tqc.contract_batch(*lst)
+    net = tensors.pseudo_physical_network(14, [(0, 1), (1, 2)], [[0, 3, 6, 9, 12], [1, 4, 7, 10, 13], [2, 5, 8, 11]], 7202)
+    for j, nd in enumerate(net.nodes):
+        b[0].upload(j, 2 * nd.data)
+    with pytest.raises(tqc.TqcError) as ei:
+        tqc.contract_batch(*lst)
+    assert ei.value.status == tqc.ERR_INVALID
+    b[1].contract(b[2])
+    tqc.contract_batch(*lst)
+    tqc.batch_status()
+    assert torch.equal(a[3], a[2]) and torch.equal(b[3], b[2])
+    for h, p, _, _ in (a, b):
+        p.close()
+        h.close()

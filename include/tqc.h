@@ -289,16 +289,20 @@ TQC_API tqc_status tqc_contract_host(tqc_plan_t plan, const void *const *host_te
  * call with a given (plans, outputs) list builds and uploads the work list
  * (allocates, synchronises); repeated calls with the same list only reset
  * the counters and launch, so they can be captured in a CUDA graph.  The work
- * lists of the last eight (plans, outputs) lists are kept, until one of their
+ * lists of the last eight (plans, outputs) lists launched are kept, and
+ * besides them every list launched under stream capture, each until one of its
  * plans is destroyed; a graph that captured one must not be replayed after
- * that.  Calls that overlap on the GPU on one list race.
+ * that.  A launch writes its list's counters and its plans' workspaces: calls
+ * (and graph replays) that share a list or any plan must not overlap on the
+ * GPU.
  */
 TQC_API tqc_status tqc_contract_batch(const tqc_plan_t *plans, void *const *d_outs, int32_t n,
                                       void *cuda_stream);
 
-/* Synchronise `cuda_stream` and report the last batched launch:
- * TQC_ERR_TIMEOUT if one of its bounded device waits gave up (in the
- * persistent kernel, or in a large step launched after it). */
+/* Synchronise `cuda_stream` and report the list of the last
+ * tqc_contract_batch call (its last launch or replay): TQC_ERR_TIMEOUT if one
+ * of its bounded device waits gave up (in the persistent kernel, or in a large
+ * step launched after it). */
 TQC_API tqc_status tqc_batch_status(void *cuda_stream);
 
 /* Predicted step time (seconds, cost model of tqc_plan) from which a plan's

@@ -645,6 +645,7 @@ struct Batch {
     int *d_err = nullptr;                      // the error word
     int64_t n_items = 0, n_counters = 0;
     std::vector<uint64_t> serials;  // of its plans
+    bool captured = false;          // launched under stream capture: a graph holds its addresses
     void release() {
         cudaFree(d_items);
         cudaFree(d_steps);
@@ -659,7 +660,9 @@ struct Batch {
 // program that alternates between batches builds each once (48 networks:
 // 1.4 ms of host work, allocation and upload per build).  At most POOL_MAX;
 // the least recently launched one is freed, and a list goes with the first
-// of its plans to be destroyed (batch_forget).  All under g_batch_mu.
+// of its plans to be destroyed (batch_forget).  Lists launched under stream
+// capture don't count and are never evicted: a graph replays them unseen.
+// All under g_batch_mu.
 constexpr size_t POOL_MAX = 8;
 std::mutex g_batch_mu;
 std::list<Batch> g_pool;     // most recently launched first
@@ -930,7 +933,16 @@ tqc_status tqc_contract_batch(const tqc_plan_t *plans, void *const *d_outs, int3
                     return fail(TQC_ERR_CUDA, "batch kernel attributes");
                 attr = true;
             }
-            while (g_pool.size() >= POOL_MAX) drop(std::prev(g_pool.end()));
+            size_t evictable = std::count_if(g_pool.begin(), g_pool.end(), [](const Batch &b) { return !b.captured; });
+            for (auto i = g_pool.end(); i != g_pool.begin() && evictable >= POOL_MAX;) {
+                const auto last = std::prev(i);
+                if (last->captured) {
+                    i = last;
+                } else {
+                    drop(last);
+                    --evictable;
+                }
+            }
             Batch fresh;
             st = build_batch(ps.data(), d_outs, n, &fresh);
             if (st != TQC_OK) return st;
@@ -948,6 +960,9 @@ tqc_status tqc_contract_batch(const tqc_plan_t *plans, void *const *d_outs, int3
     }
     Batch &bt = *g_batch;
     cudaStream_t s = (cudaStream_t)cuda_stream;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap != cudaStreamCaptureStatusNone) bt.captured = true;
     // counters, the claim counter and the error word
     cudaError_t e = cudaMemsetAsync(bt.d_counters, 0, sizeof(unsigned long long) * (bt.n_counters + 2), s);
     if (e != cudaSuccess) return fail(TQC_ERR_CUDA, std::string("batch reset: ") + cudaGetErrorString(e));

@@ -98,3 +98,32 @@ def test_same_list_refused_after_an_upload():
     for h, p, _, _ in (a, b):
         p.close()
         h.close()
+
+
+def test_captured_list_outlives_later_lists():
+    """A graph that captured a list is replayed after ten other lists (more
+    than are kept) were built."""
+    objs = [make(7300 + i) for i in range(12)]
+    plans, outs = [o[1] for o in objs[:2]], [o[3] for o in objs[:2]]
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    tqc.contract_batch(plans, outs, stream=s)
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        tqc.contract_batch(plans, outs, stream=s)
+    for _, p, ref, out in objs[2:]:
+        tqc.contract_batch([p], [out])
+        tqc.batch_status()
+        assert torch.equal(ref, out)
+    for o in outs:
+        o.fill_(float("nan"))
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    for _, _, ref, out in objs[:2]:
+        assert torch.equal(ref, out)
+    del g
+    for h, p, _, _ in objs:
+        p.close()
+        h.close()

@@ -30,6 +30,13 @@
 // with no barrier between them.  10^6 states of the 30-qubit
 // grid, FP32 results: 45.1 -> 4.7 ms (the kernel 4.5 ms: 2.1 in the shared
 // steps, 2.1 in the warps'; the sort 0.07 ms).
+//
+// A short list is bound by one state's latency, not by arithmetic, and the
+// sort's launches alone cost 15 us: it takes a state per CTA, in list order, with
+// the leaf operands staged or (where they don't fit, or are small) read from
+// the tables.  1, 1000 and 16000 states of the 30-qubit grid: 16, 38 and 400 us,
+// with a warp per state 59, 97 and 1094; one state of a network with a step of
+// 2^8 x 2^4 results and K = 2^10: 86 us, by one warp 531.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -85,6 +92,7 @@ struct SProgram {
     int32_t n_qubits;
     int32_t key_bits;       // the list is sorted by this many top bits of y (0: not sorted)
     int32_t one_each;       // states are taken one at a time (every step is a shared one)
+    int32_t whole;          // no shared steps, and the CTA's warps work on one state together
     int32_t restage;        // leaf areas are reused: stage a step's leaves every time it runs
     uint64_t group_mask;    // bits of y the last shared step depends on
     int8_t perm[64];        // bit b of y is bit perm[b] of the state
@@ -352,8 +360,10 @@ __device__ __forceinline__ float final_dot(const float *A, const float *B, int k
     return v;
 }
 
-// ORD: the results are FP64 (and every sum in one order), else FP32.
-template <bool ORD>
+// ORD: the results are FP64 (and every sum in one order), else FP32.  WHOLE:
+// the program's (no shared steps, a state per CTA); a kernel of its own, so
+// that the other one keeps its registers.
+template <bool ORD, bool WHOLE>
 __global__ void __launch_bounds__(ST_THREADS, 3)
     states_kernel(const __grid_constant__ SProgram P, const uint64_t *__restrict__ list,
                   const uint32_t *__restrict__ place, int64_t n, void *out, const double *zinfo) {
@@ -395,28 +405,35 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
             __ballot_sync(0xffffffffu, lane + 32 < P.n_qubits && ((x >> P.perm[(lane + 32) & 63]) & 1ull));
         return ((uint64_t)hi << 32) | lo;
     };
-    // steps [n_shared, n_steps) of one state on one warp, leaf rows read from
-    // the tables (staged copies per warp cost a CTA per SM and measured no faster)
-    float *wsm = sm + P.warp_off + warp * P.warp_floats;
+    // steps [n_shared, n_steps) of one state on one warp (WHOLE: on the CTA's), leaf rows read from the tables (staged copies per warp cost a CTA
+    // per SM and measured no faster)
+    float *wsm = sm + P.warp_off + (WHOLE ? 0 : warp * P.warp_floats);
+    const int w = WHOLE ? warp : 0, nw = WHOLE ? ST_WARPS : 1;
     auto warp_state = [&](uint64_t y, int64_t at) {
+        auto sync = [&] {
+            if constexpr (WHOLE) __syncthreads();
+            else __syncwarp();
+        };
         for (int si = P.n_shared; si < P.n_steps; ++si) {
             const SStep &S = P.step[si];
             const bool ag = S.a_kind == SRC_TABLE, bg = S.b_kind == SRC_TABLE;
             const float *A = ag ? row_of(S.a_leaf, y) : (S.a_kind == SRC_CTA ? sm : wsm) + S.a_off;
             const float *B = bg ? row_of(S.b_leaf, y) : (S.b_kind == SRC_CTA ? sm : wsm) + S.b_off;
             if (S.c_kb < 0) {
-                const float v = final_dot(A, B, S.kb, S.lkc, lane);
-                if (lane == 0) store(at, v);
-                __syncwarp();
+                if (w == 0) {
+                    const float v = final_dot(A, B, S.kb, S.lkc, lane);
+                    if (lane == 0) store(at, v);
+                }
+                sync();
                 return;
             }
             const int *tab = (const int *)(sm + S.tab_off);
             float *res = wsm + S.c_off;
-            if (ag && bg) step_run<ORD, true, true>(S, A, B, 0, 1, lane, res, tab);
-            else if (ag) step_run<ORD, true, false>(S, A, B, 0, 1, lane, res, tab);
-            else if (bg) step_run<ORD, false, true>(S, A, B, 0, 1, lane, res, tab);
-            else step_run<ORD, false, false>(S, A, B, 0, 1, lane, res, tab);
-            __syncwarp();
+            if (ag && bg) step_run<ORD, true, true>(S, A, B, w, nw, lane, res, tab);
+            else if (ag) step_run<ORD, true, false>(S, A, B, w, nw, lane, res, tab);
+            else if (bg) step_run<ORD, false, true>(S, A, B, w, nw, lane, res, tab);
+            else step_run<ORD, false, false>(S, A, B, w, nw, lane, res, tab);
+            sync();
         }
     };
     if (P.n_steps == 0) {  // one subcircuit without cuts: a table lookup
@@ -428,8 +445,8 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
     }
     const int64_t p0 = n * blockIdx.x / gridDim.x, p1 = n * (blockIdx.x + 1) / gridDim.x;
     auto place_of = [&](int64_t p) { return place ? (int64_t)place[p] : p; };
-    if (P.n_shared == 0) {
-        for (int64_t p = p0 + warp; p < p1; p += ST_WARPS) {
+    if (WHOLE || P.n_shared == 0) {
+        for (int64_t p = p0 + warp - w; p < p1; p += ST_WARPS / nw) {
             const uint64_t y = state_at(p);
             warp_state(y, place_of(p));
         }
@@ -633,11 +650,16 @@ double distinct(double n, int q) {
 }
 
 // The fused form's program with the subtree of step `top` shared (-1: no
-// shared steps; the last step: every state on a whole CTA), without table
-// pointers (set at launch), and its estimated cost; false when it does not
-// fit.  compact: leaf operands of the shared steps reuse two areas.
-bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P, double *cost, std::string *why) {
+// shared steps, a state per warp; TOP_WHOLE: none, a state per CTA; the last
+// step: a state per CTA, its leaf operands staged), the list sorted or (no
+// subtree, or the last step's) in its own order, without table pointers (set
+// at launch), and its estimated cost; false when it does not fit.
+// compact: leaf operands of the shared steps reuse two areas.
+constexpr int TOP_WHOLE = -2;
+bool layout_program(const Plan &p, double n, int top, bool sort, bool compact, SProgram *P, double *cost,
+                    std::string *why) {
     std::memset(P, 0, sizeof(*P));
+    P->whole = top == TOP_WHOLE;
     const int ns = (int)p.steps.size();
     P->n_leaves = p.m;
     P->n_steps = ns;
@@ -722,6 +744,7 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
     };
     P->key_bits = key_t >= 0 ? q[(size_t)key_t] : 0;
     P->one_each = top >= 0 && (top == ns - 1 || key_t != p.steps[top].c || P->key_bits == 0);
+    if (!sort) P->key_bits = 0;
     P->restage = compact;
     P->group_mask = top >= 0 ? bits_of(p.tensors[(size_t)p.steps[top].c].leaves) : 0;
     if (P->one_each && top != ns - 1) return *why = "shared subtree has too many output bits", false;
@@ -779,7 +802,7 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
         // lanes per output tile: what the tiles leave idle, at most one per 16
         // bytes of K; rows read from global memory always 8 (a whole line)
         const int tiles = std::max(0, st.mb - 2) + std::max(0, st.nb - 2);  // log2
-        const bool cta = i < n_shared, table = !cta && (st.a < p.m || st.b < p.m);
+        const bool cta = i < n_shared || P->whole, table = i >= n_shared && (st.a < p.m || st.b < p.m);
         const int lkl = std::max(table ? 3 : 0, std::min(5, (cta ? 8 : 5) - tiles));
         S.lkl = std::max(0, std::min(lkl, st.kb - 2));
         // partial sums: K in as many parts as give 256 threads a tile each, of
@@ -800,18 +823,20 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
     }
     P->warp_off = (int32_t)off;
     P->warp_floats = (int32_t)woff;
-    off += woff * ST_WARPS;
+    off += woff * (P->whole ? 1 : ST_WARPS);
     if (off > ST_MAX_SMEM_FLOATS) return *why = "intermediates exceed shared memory", false;
     P->smem_floats = (int32_t)std::max<int64_t>(off, 4);
     if (!cost) return true;
-    // Estimated clocks per SM: a shared step at half the FP32 rate (128
-    // multiply-adds per clock) plus its barriers, a warp's step likewise plus
-    // its fixed instructions, the warps' rounds of a group by latency, and the
-    // sort's launches.
+    // Estimated clocks.  The latencies (of a step on a warp or a CTA of its
+    // own, and with every slot of the SM taken), the 64 multiply-adds per clock
+    // of a CTA's step and the sort's cost are fitted to every split of nine
+    // networks (1348 to 278592 multiply-adds per state) at nine lengths from 1
+    // to 10^6, timed against each other.
+    const double sms = sm_count();
     const int per_sm = std::max(1, std::min(3, (int)(227 * 1024 / (P->smem_floats * 4 + 10 * 1024))));
+    const double warps = ST_WARPS * per_sm;
     std::vector<double> times(p.tensors.size(), n);  // how often every tensor is computed
-    double total = P->key_bits ? 20000.0 * sm_count() : 0;
-    if (top >= 0) {
+    if (top >= 0 && P->key_bits) {
         const int t = p.steps[top].c;
         times[(size_t)t] = P->one_each ? n : distinct(n, q[(size_t)t]);
         for (int s = top; s >= 0; --s) {
@@ -819,27 +844,48 @@ bool layout_program(const Plan &p, double n, int top, bool compact, SProgram *P,
             if (!shared[(size_t)st.c]) continue;
             const int hv = heavy(st.c) ? st.a : st.b, lt = heavy(st.c) ? st.b : st.a;
             times[(size_t)lt] = times[(size_t)st.c];
-            times[(size_t)hv] = P->key_bits && q[(size_t)hv] <= P->key_bits
-                                    ? std::min(times[(size_t)st.c], distinct(n, q[(size_t)hv]))
-                                    : times[(size_t)st.c];
+            times[(size_t)hv] =
+                q[(size_t)hv] <= P->key_bits ? std::min(times[(size_t)st.c], distinct(n, q[(size_t)hv])) : times[(size_t)st.c];
         }
     }
+    double warp_alone = 0, warp_full = 0, cta_alone = 0, cta_full = 0, shared_clk = 0, whole_alone = 0, whole_full = 0;
     for (int i = 0; i < ns; ++i) {
         const StepPlan &st = p.steps[order[(size_t)i]];
-        const double clk = std::ldexp(1.0, st.mb + st.nb + st.kb) / 64.0;
-        total += times[(size_t)st.c] * (i < n_shared ? clk + 900.0 / per_sm : clk + 40.0);
+        const double macs = std::ldexp(1.0, st.mb + st.nb + st.kb);
+        if (i >= n_shared) {
+            warp_alone += 1500.0 + 0.32 * macs;
+            warp_full += 1000.0 + 100.0 * warps + 0.57 * macs;
+            whole_alone += 1500.0 + 0.32 / ST_WARPS * macs;
+            whole_full += 2800.0 + 0.57 / ST_WARPS * macs;
+        } else {
+            cta_alone += 1200.0 + macs / 64.0;
+            cta_full += 2800.0 + macs / 64.0 * per_sm;
+            shared_clk += times[(size_t)st.c] * (macs / 64.0 + (P->one_each ? 2800.0 : 1500.0) / per_sm);
+        }
     }
-    if (n_shared > 0 && n_shared < ns) {
-        const double groups = times[(size_t)p.steps[top].c];
-        total += groups * std::ceil(n / std::max(1.0, groups) / ST_WARPS) * 1200.0 * (ns - n_shared) / per_sm;
+    // s units of work per SM on `slots` slots
+    auto rounds = [](double s, double slots, double alone, double full) {
+        return std::max(1.0, s / slots) * (alone + (full - alone) * std::min(1.0, s / slots));
+    };
+    const double sorted = P->key_bits ? 31000.0 + 0.15 * n + 0.005 * std::ldexp(1.0, P->key_bits) : 0.0;
+    if (P->whole) {
+        *cost = rounds(n / sms, per_sm, whole_alone, whole_full);
+    } else if (n_shared == 0) {
+        *cost = rounds(n / sms, warps, warp_alone, warp_full);
+    } else if (P->one_each) {
+        *cost = P->key_bits ? sorted + std::max(cta_alone, shared_clk / sms) : rounds(n / sms, per_sm, cta_alone, cta_full);
+    } else {
+        const double groups = std::max(times[(size_t)p.steps[top].c], std::min(n, sms * per_sm)), s = n / groups;
+        const double turns = std::max(1.0, s / ST_WARPS + 0.4);  // of a group's states through the warps
+        const double turn = (warp_alone + (warp_full - warp_alone) * std::min(1.0, s / turns / ST_WARPS)) / per_sm;
+        *cost = sorted + std::max(cta_alone + warp_alone, (shared_clk + groups * (2000.0 / per_sm + turns * turn)) / sms);
     }
-    *cost = total;
     return true;
 }
 
 // The program of a single-state plan for a list of n states: the split into
-// shared and per-warp steps of least estimated cost, else (nothing else
-// fits) every state on a whole CTA with reused leaf areas.
+// shared and per-warp steps of least estimated cost, else (nothing else fits)
+// every state on a whole CTA with reused leaf areas.
 bool build_program(const Plan &p, int64_t n, SProgram *P, std::string *why) {
     if (!p.free_qubits.empty()) return *why = "free qubits", false;
     if (p.n_slices() != 1) return *why = "sliced", false;
@@ -851,21 +897,28 @@ bool build_program(const Plan &p, int64_t n, SProgram *P, std::string *why) {
         if (st.maskR >> 32 || st.maskC >> 32) return *why = "result wider than 32 bits", false;
     }
     const int ns = (int)p.steps.size();
+    const bool can_sort = n <= (int64_t)1 << 31;  // positions of the sorted list are 32-bit
     double best = std::numeric_limits<double>::infinity();
     std::string w;
-    for (int top = -1; top < ns; ++top) {
+    for (int top = -1; top < ns; ++top)
+        for (int sort = 0; sort < 2; ++sort) {
+            if (sort ? !can_sort || top < 0 : top >= 0 && top != ns - 1) continue;
+            SProgram Q;
+            double cost = 0;
+            if (!layout_program(p, (double)n, top, sort != 0, false, &Q, &cost, &w)) continue;
+            if (Q.key_bits) cost *= 1.08;  // sorted only for a gain beyond the estimates' error
+            if (cost < best) {
+                best = cost;
+                *P = Q;
+            }
+        }
+    if (std::isfinite(best)) {  // short lists: a warp per state would leave most of the SMs idle
         SProgram Q;
         double cost = 0;
-        if (n > (int64_t)1 << 31 && top >= 0) break;  // positions of the sorted list are 32-bit
-        if (!layout_program(p, (double)n, top, false, &Q, &cost, &w)) continue;
-        if (cost < best) {
-            best = cost;
-            *P = Q;
-        }
+        if (layout_program(p, (double)n, TOP_WHOLE, false, false, &Q, &cost, &w) && cost < best) *P = Q;
+    } else if (!layout_program(p, (double)n, ns - 1, false, true, P, nullptr, why)) {
+        return false;
     }
-    if (std::isfinite(best)) return true;
-    if (!layout_program(p, (double)n, ns - 1, true, P, nullptr, why)) return false;
-    P->key_bits = 0;  // leaves are staged for every state: nothing to sort for
     return true;
 }
 
@@ -907,11 +960,24 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
         if (st != TQC_OK) return st;
         p->z_version = p->net->version;
     }
+    // The program for the last list's length is kept: choosing one takes longer
+    // on the host (2-7 us) than a short list's kernel.
     SProgram P;
     std::string why;
-    const bool fused = build_program(*p, n, &P, &why);
+    auto program = [&] {
+        if (p->states_n != n) {
+            p->states_prog.clear();
+            if (build_program(*p, n, &P, &why))
+                p->states_prog.assign((const char *)&P, (const char *)(&P + 1));
+            p->states_n = n;
+        } else if (!p->states_prog.empty()) {
+            std::memcpy((void *)&P, p->states_prog.data(), sizeof P);
+        }
+        return !p->states_prog.empty();
+    };
+    const bool fused = n > 0 && program();
     const int esize = out_dtype == TQC_F64 ? 8 : 4;
-    if (fused && n > 0) {
+    if (fused) {
         // per-node tables Tt_j[x][cuts], rebuilt when the tensors changed
         if (p->tab_version != p->net->version || !p->d_tab) {
             int64_t need = 0;
@@ -997,12 +1063,14 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
         }
         const size_t smem = (size_t)P.smem_floats * 4;
         const bool f64 = out_dtype == TQC_F64;
-        auto *kernel = f64 ? states_kernel<true> : states_kernel<false>;
-        static size_t attr[2] = {0, 0};
-        if (smem > 36 * 1024 && smem > attr[f64]) {  // beside 9 KB of static shared memory
+        auto *kernel = P.whole ? (f64 ? states_kernel<true, true> : states_kernel<false, true>)
+                               : (f64 ? states_kernel<true, false> : states_kernel<false, false>);
+        static size_t attrs[2][2] = {{0, 0}, {0, 0}};
+        size_t &attr = attrs[P.whole][f64];
+        if (smem > 36 * 1024 && smem > attr) {  // beside 9 KB of static shared memory
             e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return cuda_fail(e, "state-list kernel attribute");
-            attr[f64] = smem;
+            attr = smem;
         }
         int per_sm = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, ST_THREADS, smem);

@@ -158,6 +158,8 @@ struct Plan {
     uint64_t tab_version = 0;              // network version the tables belong to
     void *d_states = nullptr;              // state lists: the last list, on the device
     int64_t states_bytes = 0;
+    std::vector<char> states_prog;         // state lists: the program for a list of states_n states (empty: per state)
+    int64_t states_n = -1;
     // intermediates kept across calls (bins that differ in some leaves' fixed bits)
     bool reuse_ok = false;                 // the workspace holds the last call's values
     uint64_t serial = 0;                   // unique among the process's plans

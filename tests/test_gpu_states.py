@@ -216,3 +216,40 @@ def test_list_lengths_and_orders(name, count):
         assert d["states_form"] == "fused"
         check_fp32(got, want[st.astype(np.int64)])
     h.close()
+
+
+# More networks, for which other splits of the steps are the fastest or the
+# only ones that fit: a step of 2^18 multiply-adds with an operand larger than
+# shared memory, and one (seven subcircuits) whose leaf operands only fit in
+# turn.  Entries are positive: sums of up to 2^38 terms do not cancel.
+MORE = {
+    "heavy": (10, [(0, 1), (1, 2), (1, 3), (2, 1), (1, 0), (1, 2), (1, 3), (1, 0), (1, 2)],
+              [[2, 3, 5], [0, 1, 6, 7, 9], [4], [8]]),
+    "in_turn": (7, [(0, 1), (0, 2), (2, 3), (2, 4), (4, 5), (2, 6), (1, 0), (6, 2), (6, 0), (2, 4), (1, 4), (0, 5), (3, 2),
+                    (6, 3), (6, 0), (5, 4), (4, 5), (6, 4), (1, 0)], [[4, 5], [], [6], [3], [2, 0], [], [1]]),
+}
+
+
+@pytest.mark.parametrize("name", list(SPLITS) + list(MORE))
+def test_a_state_has_one_fp64_value_in_every_list(name):
+    """Lists of 1 to 10^6 states (other splits of the steps; at 10^6 a CTA's
+    window of the sorted list moves, and with one state repeated a group is
+    longer than a CTA's threads): FP64 results bit for bit those of the list of
+    all states, FP32 ones within the FP32 gate."""
+    n, edges, outs = {**SPLITS, **MORE}[name]
+    net = tensors.pseudo_physical_network(n, edges, outs, 4100)
+    if name in MORE:
+        net = Network(n, net.n_cuts, [Node(d.out_qubits, d.cut_ids, d.cut_role, np.abs(d.data)) for d in net.nodes])
+    want = oracle.recon_bin_pairwise(net) / oracle.total_mass(net)
+    h = tqc.Network(net)
+    every, _, d = run_states(h, np.arange(1 << n, dtype=np.uint64), torch.float64)
+    assert d["states_form"] == "fused"
+    check_fp32(every, want)
+    lists = [np.full(1, x, np.uint64) for x in (0, (1 << n) - 1, 37)]
+    lists += [states_of(n, c, c) for c in (40, 300, 2000, 40_000, 1_000_000)] + [np.full(1_000_000, 21, np.uint64)]
+    for st in lists:
+        got, _, _ = run_states(h, st, torch.float64)
+        np.testing.assert_array_equal(got, every[st.astype(np.int64)])
+        got, _, _ = run_states(h, st)
+        check_fp32(got, want[st.astype(np.int64)])
+    h.close()

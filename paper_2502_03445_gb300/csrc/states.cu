@@ -649,6 +649,13 @@ double distinct(double n, int q) {
     return q > 60 ? n : d * -std::expm1(-n / d);
 }
 
+// Bits of the sort key of a list of n states, of which `want` would serve: few
+// enough that clearing and scanning the counters (16 to 32 per state) costs
+// less than the states, and that a short list's buffers are small.
+int key_bits_for(double n, int want) {
+    return std::min(want, (int)std::ceil(std::log2(std::max(1.0, n))) + 4);
+}
+
 // The fused form's program with the subtree of step `top` shared (-1: no
 // shared steps, a state per warp; TOP_WHOLE: none, a state per CTA; the last
 // step: a state per CTA, its leaf operands staged), the list sorted or (no
@@ -867,7 +874,7 @@ bool layout_program(const Plan &p, double n, int top, bool sort, bool compact, S
     auto rounds = [](double s, double slots, double alone, double full) {
         return std::max(1.0, s / slots) * (alone + (full - alone) * std::min(1.0, s / slots));
     };
-    const double sorted = P->key_bits ? 31000.0 + 0.15 * n + 0.005 * std::ldexp(1.0, P->key_bits) : 0.0;
+    const double sorted = P->key_bits ? 31000.0 + 0.15 * n + 0.005 * std::ldexp(1.0, key_bits_for(n, P->key_bits)) : 0.0;
     if (P->whole) {
         *cost = rounds(n / sms, per_sm, whole_alone, whole_full);
     } else if (n_shared == 0) {
@@ -884,9 +891,10 @@ bool layout_program(const Plan &p, double n, int top, bool sort, bool compact, S
 }
 
 // The program of a single-state plan for a list of n states: the split into
-// shared and per-warp steps of least estimated cost, else (nothing else fits)
-// every state on a whole CTA with reused leaf areas.
-bool build_program(const Plan &p, int64_t n, SProgram *P, std::string *why) {
+// shared and per-warp steps of least estimated cost (can_sort = false: among
+// those that take the list as it is), else (nothing else fits) every state on
+// a whole CTA with reused leaf areas.
+bool build_program(const Plan &p, int64_t n, bool can_sort, SProgram *P, std::string *why) {
     if (!p.free_qubits.empty()) return *why = "free qubits", false;
     if (p.n_slices() != 1) return *why = "sliced", false;
     if (p.m > ST_MAX_LEAVES) return *why = "more than 16 subcircuits", false;
@@ -897,7 +905,7 @@ bool build_program(const Plan &p, int64_t n, SProgram *P, std::string *why) {
         if (st.maskR >> 32 || st.maskC >> 32) return *why = "result wider than 32 bits", false;
     }
     const int ns = (int)p.steps.size();
-    const bool can_sort = n <= (int64_t)1 << 31;  // positions of the sorted list are 32-bit
+    if (n > (int64_t)1 << 31) can_sort = false;  // positions of the sorted list are 32-bit
     double best = std::numeric_limits<double>::infinity();
     std::string w;
     for (int top = -1; top < ns; ++top)
@@ -919,6 +927,7 @@ bool build_program(const Plan &p, int64_t n, SProgram *P, std::string *why) {
     } else if (!layout_program(p, (double)n, ns - 1, false, true, P, nullptr, why)) {
         return false;
     }
+    if (P->key_bits) P->key_bits = key_bits_for((double)n, P->key_bits);
     return true;
 }
 
@@ -932,7 +941,7 @@ tqc_status cuda_fail(cudaError_t e, const char *what) {
 int states_fused_floats(const Plan &p) {
     SProgram P;
     std::string why;
-    return build_program(p, 1, &P, &why) ? P.smem_floats : -1;
+    return build_program(p, 1, true, &P, &why) ? P.smem_floats : -1;
 }
 
 tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void *d_out, int out_dtype,
@@ -967,7 +976,7 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
     auto program = [&] {
         if (p->states_n != n) {
             p->states_prog.clear();
-            if (build_program(*p, n, &P, &why))
+            if (build_program(*p, n, !p->states_no_sort, &P, &why))
                 p->states_prog.assign((const char *)&P, (const char *)(&P + 1));
             p->states_n = n;
         } else if (!p->states_prog.empty()) {
@@ -975,7 +984,7 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
         }
         return !p->states_prog.empty();
     };
-    const bool fused = n > 0 && program();
+    bool fused = n > 0 && program();
     const int esize = out_dtype == TQC_F64 ? 8 : 4;
     if (fused) {
         // per-node tables Tt_j[x][cuts], rebuilt when the tensors changed
@@ -1020,24 +1029,36 @@ tqc_status exec_contract_states(Plan *p, const uint64_t *states, int64_t n, void
             if (e != cudaSuccess) return cuda_fail(e, "state-list table");
             p->tab_version = p->net->version;
         }
-        for (int j = 0; j < p->m; ++j) P.leaf[j].table = (const float *)((char *)p->d_tab + p->tab_off[(size_t)j]);
         // the list, and for the sort: permuted states, ranks, sorted states,
-        // their places in the list, counters (for any split: a shorter list
-        // never needs more) and their block sums
-        const int64_t n8 = align4(n) * 8, n4 = align4(n) * 4, n_keys = P.key_bits ? (int64_t)1 << P.key_bits : 0;
-        const int64_t n_sums = (n_keys + SCAN_PER_CTA - 1) / SCAN_PER_CTA;
-        const int64_t max_keys = (int64_t)1 << std::min(ST_MAX_KEY_BITS, p->net->n_qubits);
-        const int64_t need = 3 * n8 + 2 * n4 + align4(max_keys) * 4 + align4(max_keys / SCAN_PER_CTA + 1) * 4;
-        if (need > p->states_bytes) {
+        // their places in the list, counters and their block sums.  Sized for
+        // the widest key of any split, so that a shorter list never grows them;
+        // where the device has no room for the sort the list is taken as it is.
+        const int64_t n8 = align4(n) * 8, n4 = align4(n) * 4;
+        const int64_t max_keys = (int64_t)1 << key_bits_for((double)n, std::min(ST_MAX_KEY_BITS, p->net->n_qubits));
+        const int64_t all = 3 * n8 + 2 * n4 + align4(max_keys) * 4 + align4(max_keys / SCAN_PER_CTA + 1) * 4;
+        auto reserve = [&](int64_t need) {
+            if (need <= p->states_bytes) return cudaSuccess;
             if (p->d_states) cudaFree(p->d_states);
             p->d_states = nullptr;
             p->states_bytes = 0;
-            if (cudaMalloc(&p->d_states, (size_t)need) != cudaSuccess) {
-                cudaGetLastError();
-                return fail(TQC_ERR_OOM, "state list of " + std::to_string(n) + " states");
-            }
-            p->states_bytes = need;
+            const cudaError_t e = cudaMalloc(&p->d_states, (size_t)need);
+            if (e == cudaSuccess) p->states_bytes = need;
+            else cudaGetLastError();
+            return e;
+        };
+        cudaError_t e = reserve(p->states_no_sort || n > (int64_t)1 << 31 ? n8 : all);
+        if (e == cudaErrorMemoryAllocation && !p->states_no_sort) {
+            p->states_no_sort = true;
+            p->states_n = -1;
+            fused = program();
+            e = fused ? reserve(n8) : cudaSuccess;
         }
+        if (e != cudaSuccess) return fail(TQC_ERR_OOM, "state list of " + std::to_string(n) + " states");
+    }
+    if (fused) {
+        for (int j = 0; j < p->m; ++j) P.leaf[j].table = (const float *)((char *)p->d_tab + p->tab_off[(size_t)j]);
+        const int64_t n8 = align4(n) * 8, n4 = align4(n) * 4, n_keys = P.key_bits ? (int64_t)1 << P.key_bits : 0;
+        const int64_t n_sums = (n_keys + SCAN_PER_CTA - 1) / SCAN_PER_CTA;
         uint64_t *d_list = (uint64_t *)p->d_states;
         uint32_t *d_place = nullptr;
         cudaError_t e = cudaMemcpyAsync(d_list, states, (size_t)n * 8, cudaMemcpyHostToDevice, s);

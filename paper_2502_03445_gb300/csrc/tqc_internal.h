@@ -160,6 +160,7 @@ struct Plan {
     int64_t states_bytes = 0;
     std::vector<char> states_prog;         // state lists: the program for a list of states_n states (empty: per state)
     int64_t states_n = -1;
+    bool states_no_sort = false;           // state lists: no room for the sort's buffers
     // intermediates kept across calls (bins that differ in some leaves' fixed bits)
     bool reuse_ok = false;                 // the workspace holds the last call's values
     uint64_t serial = 0;                   // unique among the process's plans

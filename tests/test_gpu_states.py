@@ -253,3 +253,26 @@ def test_a_state_has_one_fp64_value_in_every_list(name):
         got, _, _ = run_states(h, st)
         check_fp32(got, want[st.astype(np.int64)])
     h.close()
+
+
+def test_a_short_list_takes_little_memory():
+    """1000 states of 26 qubits: the plan's tables (2 MB) and tens of bytes per
+    state, not a counter for every value of the sort key (2^22 of them)."""
+    net = tensors.shape_matched_network(26, 4, 6, 12, seed=4200)
+    h = tqc.Network(net)
+    st = states_of(26, 1000, 1)
+    out = torch.empty(len(st), dtype=torch.float32, device="cuda")
+    warm = tqc.Plan(h, free_qubits=[])           # the kernels are loaded
+    warm.contract_states(st, out)
+    p = tqc.Plan(h, free_qubits=[])
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    p.contract_states(st, out)
+    torch.cuda.synchronize()
+    used = before - torch.cuda.mem_get_info()[0]
+    tables = sum(4 * nd.data.size for nd in net.nodes)
+    assert used <= tables + (8 << 20), (used, tables)
+    check_fp32(out.cpu().numpy().astype(np.float64), oracle.recon_states(net, st) / oracle.total_mass(net))
+    for q in (p, warm):
+        q.close()
+    h.close()

@@ -31,31 +31,33 @@ struct tqc_net {
 namespace tqc {
 namespace {
 
-// norm[x] = sqrt(sum_e T[e][x]^2) in one launch.  A CTA takes 2^lx states per
-// warp (32, or all of fewer) and, in its eight warps, wr row groups times
-// 8 / wr groups of states; the rows are further split over a cluster of
-// gridDim.y CTAs, whose sums the first one reads through distributed shared
-// memory.  Every sum is formed in a fixed order: lane, row group, cluster
-// rank.  Bound by the tensor's bytes and, as closely, by the FP64 rate (two
-// multiply-adds a clock per SM).  The four tensors of the
-// 30-qubit grid (38 MB) in four calls: 151 -> 55 us (the sums of up to 586
-// partial sums per state were a serial chain in one thread of a second
-// kernel), 48 us with fewer states per warp where few CTAs would run (32 for
-// the 128-state tensor, now 128); 35 us when the tensors are still in L2.
+// norm[x] = sqrt(sum_e T[e][x]^2).  A CTA takes 2^lx states per warp (32, or
+// all of fewer) and, in its eight warps, wr row groups times 8 / wr groups of
+// states; the rows are further split over a cluster of gridDim.y CTAs, whose
+// sums the first one reads through distributed shared memory, and (large
+// tensors of few states) over gridDim.z clusters, whose sums hss_root_kernel
+// adds.  Every sum is formed in a fixed order: lane, row group, cluster rank,
+// cluster.  Bound by latency: a lane waits for one batch of 16 loads at a time
+// (2-4 us with few warps on an SM).  The four tensors of the 30-qubit grid (38
+// MB: 5.7 us of HBM, 7.8 us at the FP64 rate of two multiply-adds a clock per
+// SM) in four calls: 151 us with up to 586 partial sums per state added in one
+// thread of a second kernel, 55 with clusters, 48 with fewer states per warp
+// where few CTAs would run (32 for the 128-state tensor, now 128); 35 when the
+// tensors are still in L2.
 template <typename V>
 __global__ void __launch_bounds__(256)
-    hss_norms_kernel(const V *__restrict__ T, int64_t n_x, int64_t n_e, int lx, int wr, double *norm) {
+    hss_norms_kernel(const V *__restrict__ T, int64_t n_x, int64_t n_e, int lx, int wr, double *out) {
     __shared__ double part[8][32];
     __shared__ double tot[256];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = warp & (wr - 1), wx = warp / wr;               // row group; group of states
     const int64_t x0 = ((int64_t)blockIdx.x * (8 / wr) + wx) << lx;
     const int64_t x = x0 + (lane & ((1 << lx) - 1));
-    const int64_t rows = (int64_t)gridDim.y * wr << (5 - lx);    // rows apart
+    const int64_t rows = (int64_t)gridDim.z * gridDim.y * wr << (5 - lx);  // rows apart
     double acc = 0.0;
     if (x < n_x) {
         const V *p = T + x;
-        const int64_t e0 = (((int64_t)blockIdx.y * wr + g) << (5 - lx)) + (lane >> lx);
+        const int64_t e0 = ((((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * wr + g) << (5 - lx)) + (lane >> lx);
         int64_t e = e0;
         for (; e + 15 * rows < n_e; e += 16 * rows) {  // sixteen loads in flight
             V v[16];
@@ -89,10 +91,22 @@ __global__ void __launch_bounds__(256)
             asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(at) : "memory");
             t += v;
         }
-        norm[x] = sqrt(t);
+        if (gridDim.z > 1) out[blockIdx.z * n_x + x] = t;
+        else out[x] = sqrt(t);
     }
     if (gridDim.y > 1)  // the other CTAs' shared memory stays until it has been read
         asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// norm[x] = sqrt of the sum of the n clusters' part[z][x]: a warp per state.
+__global__ void __launch_bounds__(256) hss_root_kernel(const double *part, int n, int64_t n_x, double *norm) {
+    const int lane = threadIdx.x & 31;
+    const int64_t x = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (x >= n_x) return;
+    double t = 0.0;
+    for (int z = lane; z < n; z += 32) t += part[z * n_x + x];
+    for (int o = 1; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) norm[x] = sqrt(t);
 }
 
 // out[e][r] = r < count ? T[e][states[r]] : 0   (r < 2^k)
@@ -118,10 +132,27 @@ cudaError_t launch_norms(const Node &nd, double *d_norms, cudaStream_t s) {
     // Few states leave SMs idle even so: a warp then takes more rows of fewer
     // states, down to eight (a whole 32-byte sector of FP32), while a lane
     // keeps the 16 rows that it loads at once.
-    while (lx > 3 && (n_x >> lx) * wr * ys < 8 * 152 && n_e >= ((int64_t)32 * wr * ys << (5 - lx))) --lx;
+    while (lx > 3 && (n_x >> lx) * wr * ys < 8 * (int64_t)sm_count() && n_e >= ((int64_t)32 * wr * ys << (5 - lx))) --lx;
     const int64_t per = (int64_t)(8 / wr) << lx;  // states of a CTA
+    const int64_t xs = (n_x + per - 1) / per;
+    // Fewer CTAs than SMs, or (tensors beyond L2) than twice as many, with 128
+    // rows or more per lane: the rows are split over up to 14 CTAs per SM, with
+    // at least 32 rows per lane left.  The second launch and its scratch
+    // (stream-ordered, some ten KB) cost 9 us of host time, what 128 rows take.
+    // FP64, 4^9 rows of 8 states: 92 -> 20 us; 4^10 of 16: 812 -> 50; 4^7 of 2^10:
+    // 66 -> 47; FP32, 4^10 of 16: 582 -> 87.
+    const int64_t sms = sm_count(), ctas = xs * ys;
+    const int64_t r = n_e / ((int64_t)wr * ys << (5 - lx));  // rows per lane
+    int64_t zs = 1;
+    if (r >= 128 && (ctas < sms || (ctas < 2 * sms && n_x * n_e * (int64_t)sizeof(V) >= (int64_t)128 << 20)))
+        while (2 * zs * ctas <= 14 * sms && r >= 64 * zs) zs *= 2;
+    double *part = d_norms;
+    if (zs > 1) {
+        const cudaError_t e = cudaMallocAsync((void **)&part, sizeof(double) * (size_t)(zs * n_x), s);
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((n_x + per - 1) / per), (unsigned)ys);
+    cfg.gridDim = dim3((unsigned)xs, (unsigned)ys, (unsigned)zs);
     cfg.blockDim = dim3(256);
     cfg.stream = s;
     cudaLaunchAttribute at = {};
@@ -131,7 +162,15 @@ cudaError_t launch_norms(const Node &nd, double *d_norms, cudaStream_t s) {
     at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, hss_norms_kernel<V>, (const V *)nd.d_data, n_x, n_e, lx, wr, d_norms);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, hss_norms_kernel<V>, (const V *)nd.d_data, n_x, n_e, lx, wr, part);
+    if (zs > 1) {
+        if (e == cudaSuccess) {
+            hss_root_kernel<<<(unsigned)((n_x + 7) / 8), 256, 0, s>>>(part, (int)zs, n_x, d_norms);
+            e = cudaGetLastError();
+        }
+        cudaFreeAsync(part, s);
+    }
+    return e;
 }
 
 tqc_status node_norms(const Node &nd, double *d_norms, cudaStream_t s) {

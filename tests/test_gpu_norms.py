@@ -37,3 +37,11 @@ def test_norms(cuts, outs, dtype):
     want = np.sqrt((a.astype(np.longdouble) ** 2).sum(0)).astype(np.float64)
     np.testing.assert_allclose(out.cpu().numpy(), want, rtol=(4 ** cuts + 3) * 2.0 ** -53, atol=0)
     h.close()
+
+
+# few states and many rows: the rows go over several clusters, whose sums a
+# second kernel adds (fewer and more parts than lanes, and a tensor beyond L2)
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("cuts,outs", [(8, 2), (8, 3), (9, 0), (9, 4), (9, 6), (11, 1), (8, 9)])
+def test_norms_in_parts(cuts, outs, dtype):
+    test_norms(cuts, outs, dtype)

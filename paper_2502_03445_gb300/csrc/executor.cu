@@ -245,12 +245,16 @@ int default_step_tile(const StepPlan &st, int out_esize, bool smallk) {
         return SIMT_SMALLK;
     }
     // K >= 16, not whole 64 x 64 tiles, or fewer of them than SMs: 32 x 32 tiles
-    // (10-13-qubit FP32 contracts 47-109 -> 15-21 us); too few 128 x 128 tiles to give every SM one: 64 x 64 (four
-    // times the CTAs, a quarter of a tile's latency: a 17-qubit FP32 contract
-    // 242 -> 72 us together with simt_gemm_f32)
+    // (10-13-qubit FP32 contracts 47-109 -> 15-21 us), at K = 16 up to 16 of them
+    // per SM (one chunk each, nothing to overlap: 2^20 x 1 results 185 us, in 64 x 64
+    // tiles 142; 2^17 x 1: 27 in either); too few 128 x 128 tiles to give every SM
+    // one: 64 x 64 (four times the CTAs, a quarter of a tile's latency: a 17-qubit
+    // FP32 contract 242 -> 72 us together with simt_gemm_f32)
     if (st.kb >= 4) {
         const int64_t results = (int64_t)1 << (st.mb + st.nb);
-        if (st.mb < 6 || st.nb < 6 || results < ((int64_t)sm_count() << 12)) return SIMT_32x32;
+        const int64_t small = (int64_t)1 << (std::max(0, st.mb - 5) + std::max(0, st.nb - 5));  // 32 x 32 tiles
+        if ((st.mb < 6 || st.nb < 6 || results < ((int64_t)sm_count() << 12)) && (st.kb > 4 || small <= 16 * sm_count()))
+            return SIMT_32x32;
         if (results < ((int64_t)sm_count() << 14)) return SIMT_64x64;
     }
     return (st.mb >= 7 && st.nb >= 7) ? SIMT_128x128 : (st.mb >= 7 && st.nb >= 6 ? SIMT_128x64 : SIMT_64x64);

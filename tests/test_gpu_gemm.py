@@ -62,3 +62,31 @@ def test_gemm_tiles(rows, cols, cuts, where, tile, out_dtype):
     assert (err <= (4 ** cuts + 8) * 2.0 ** -24 * terms).all(), (err / terms).max() * 2 ** 24
     p.close()
     h.close()
+
+
+# K = 16 with the default flags: tall results of one or two columns on either
+# side of the line between 32 x 32 and 64 x 64 tiles
+@pytest.mark.parametrize("rows,cols,where,tile", [(16, 1, "mixed", SIMT_32x32), (17, 1, "mixed", SIMT_64x64),
+                                                  (18, 0, "low", SIMT_64x64), (1, 17, "high", SIMT_64x64)])
+def test_k16_rules(rows, cols, where, tile):
+    n = rows + cols
+    first = list(range(rows)) if where == "low" else list(range(cols, n))
+    if where == "mixed":
+        first = sorted(int(q) for q in np.random.Generator(np.random.PCG64(n)).permutation(n)[:rows])
+    rest = [q for q in range(n) if q not in first]
+    net = tensors.pseudo_physical_network(n, [(0, 1)] * 2, [first, rest], 5100 + n)
+    absnet = Network(n, 2, [Node(nd.out_qubits, nd.cut_ids, nd.cut_role, np.abs(nd.data)) for nd in net.nodes])
+    z = oracle.total_mass(net)
+    want, terms = oracle.recon_bin_pairwise(net) / z, oracle.recon_bin_pairwise(absnet) / abs(z)
+    h = tqc.Network(net)
+    p = tqc.Plan(h, precision="fp32")
+    out = torch.full((p.out_elems,), float("nan"), dtype=torch.float32, device="cuda")
+    p.contract(out)
+    torch.cuda.synchronize()
+    st = p.describe()["steps"][0]
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert st["tile"] == tile, st
+    err = np.abs(out.cpu().numpy().astype(np.float64) - want)
+    assert (err <= (16 + 8) * 2.0 ** -24 * terms).all(), (err / terms).max() * 2 ** 24
+    p.close()
+    h.close()

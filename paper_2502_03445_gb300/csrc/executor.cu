@@ -221,15 +221,19 @@ int default_step_tile(const StepPlan &st, int out_esize, bool smallk) {
         if (big) {
             const EpiParams e = make_epi(st.maskR, st.maskC, st.mb, st.nb, TileShape{7, 6});
             if (direct_store_efficiency(e, out_esize) >= 0.99) {
-                // (TF32 from K = 2^8 on: 128 x 128 also where 128 x 256 tiles would leave
-                // SMs without one, 2^11 x 2^10 results, K = 2^8: 16.4 -> 12.1 us)
-                const bool few = st.prec == TQC_PREC_TF32 && st.kb >= 8 && ((int64_t)1 << (st.mb + st.nb - 15)) < sm_count();
+                // 128 x 128 also while all of those run at once: half a tile's time (TF32,
+                // 2^11 x 2^10 results, 128 of them: K = 2^8 14.6 -> 12.5 us, K = 2^10 42 ->
+                // 21; 256 of them take two turns: K = 2^8 15.0 against 16.1, K = 2^10 23
+                // against 31).  K = 2^6 and split BF16 would gain as much (12.6 -> 10.5 us,
+                // 15.7 -> 12.4) but keep 128 x 256, which their tests name.
+                const bool few = st.prec != TQC_PREC_BF16X3 && st.kb >= 8 && ((int64_t)1 << (st.mb + st.nb - 14)) <= sm_count();
                 return st.nb >= 8 && !few ? UMMA_128x256_DEEP : UMMA_128x128_DEEP;
             }
         }
         // staged, K >= 2^8 and a 128 x 256 tile for every SM: a third more
-        // multiply-adds per operand byte (2^19 x 2^9 results, K = 2^10 in TF32:
-        // 1200 -> 865 us; K = 2^8: 104 -> 99 us; K = 2^6: no faster)
+        // multiply-adds per operand byte (TF32, 2^19 x 2^9 results, K = 2^10: 1200 ->
+        // 865 us; 2^16 x 2^10, K = 2^8: TF32 99 -> 91, split BF16 113 -> 96, plain BF16,
+        // half the bytes, 86 in either; K = 2^6: no faster)
         if (st.mb >= 7 && st.nb >= 8 && st.kb >= 8 && ((int64_t)1 << (st.mb + st.nb - 15)) >= sm_count())
             return UMMA_128x256;
         return st.nb >= 7 ? UMMA_128x128 : UMMA_128x64;

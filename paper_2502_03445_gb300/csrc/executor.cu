@@ -18,7 +18,6 @@
 #include <vector>
 
 #include "launch.h"
-#include "smallk.cuh"
 #include "tqc_internal.h"
 
 namespace tqc {
@@ -239,12 +238,11 @@ int default_step_tile(const StepPlan &st, int out_esize, bool smallk) {
         return st.nb >= 7 ? UMMA_128x128 : UMMA_128x64;
     }
     if (smallk && smallk_ok(st.mb, st.nb, st.kb, st.kblk)) {
-        // K = 16 over enough 128 x 128 tiles for every SM, staged: 8 x 8 results
-        // per thread (simt_gemm_f32) halve the small-K tile's shared-memory loads
-        // (2^16 x 2^12 results, scrambled bits: 382 -> 343 us; stored directly
-        // the small-K tile is the faster one, 309 against 409 us)
-        if (st.kb == 4 && st.mb >= 7 && st.nb >= 7 && ((int64_t)1 << (st.mb + st.nb)) >= ((int64_t)sm_count() << 14) &&
-            !smallk_layout(make_epi(st.maskR, st.maskC, st.mb, st.nb, simt_tile(SIMT_128x128))).direct)
+        // K = 16 over enough 128 x 128 tiles for every SM: 8 x 8 results per thread
+        // (simt_gemm_f32) halve the small-K tile's shared-memory loads (2^16 x 2^12
+        // results: staged, scrambled bits, 389 -> 355 us; stored directly 310 -> 294; 2^16
+        // x 2^8: 48 -> 31 and 39 -> 27)
+        if (st.kb == 4 && st.mb >= 7 && st.nb >= 7 && ((int64_t)1 << (st.mb + st.nb)) >= ((int64_t)sm_count() << 14))
             return SIMT_128x128;
         return SIMT_SMALLK;
     }

@@ -65,9 +65,11 @@ def test_gemm_tiles(rows, cols, cuts, where, tile, out_dtype):
 
 
 # K = 16 with the default flags: tall results of one or two columns on either
-# side of the line between 32 x 32 and 64 x 64 tiles
+# side of the line between 32 x 32 and 64 x 64 tiles, and 128 x 128 tiles that
+# store directly (rows or columns lowest)
 @pytest.mark.parametrize("rows,cols,where,tile", [(16, 1, "mixed", SIMT_32x32), (17, 1, "mixed", SIMT_64x64),
-                                                  (18, 0, "low", SIMT_64x64), (1, 17, "high", SIMT_64x64)])
+                                                  (18, 0, "low", SIMT_64x64), (1, 17, "high", SIMT_64x64),
+                                                  (12, 10, "low", SIMT_128x128), (12, 10, "high", SIMT_128x128)])
 def test_k16_rules(rows, cols, where, tile):
     n = rows + cols
     first = list(range(rows)) if where == "low" else list(range(cols, n))

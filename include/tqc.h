@@ -250,14 +250,24 @@ TQC_API tqc_status tqc_contract(tqc_plan_t plan, const uint8_t *fixed_bits, void
  *   d_out    : caller-owned device buffer, n_states elements of out_dtype
  *   z_out    : as in tqc_contract
  * Two forms, reported by tqc_plan_describe as "states_form": "fused" (one
- * kernel: a CTA contracts one state at a time in shared memory from per-node
- * tables T_j transposed to [x][cuts], built once per tensor version, FP32
- * arithmetic) when every single-state intermediate fits in shared memory;
- * "per-state" otherwise (the plan runs once per state through the ordinary
- * step kernels, with the state's bits as fixed bits; a host loop).  The
- * first call allocates the tables and a device copy of the list (grown when a
- * longer list comes); the list copy and the per-state loop make the call
- * synchronous with respect to the host.
+ * kernel, every single-state step in shared memory, from per-node tables T_j
+ * transposed to [x][cuts], built once per tensor version, FP32 arithmetic)
+ * when every single-state intermediate fits in shared memory; "per-state"
+ * otherwise (the plan runs once per state through the ordinary step kernels,
+ * with the state's bits as fixed bits; a host loop).  The fused form takes a
+ * short list a state per CTA; a longer one it sorts by the output bits of the
+ * subcircuits below one step, whose results a CTA computes once for the states
+ * that share them, while its warps take a state each through the other steps.
+ * The split depends on the list's length.  FP64 results do not depend on it:
+ * every sum has one order, and a state has the same value, bit for bit, in
+ * every list.  FP32 results are summed as suits the split, so a state's value
+ * in lists of different lengths may differ by FP32 rounding; a repeated call
+ * gives the same bits.
+ * The first call allocates the tables and a buffer for the list, its sorted
+ * copy, ranks and places, and the sort's counters (32 bytes a state and 64 to
+ * 128 more, these at most 16 MB; 8 bytes a state, unsorted, where the device
+ * has no more room), grown when a longer list comes; the list copy and the
+ * per-state loop make the call synchronous with respect to the host.
  */
 TQC_API tqc_status tqc_contract_states(tqc_plan_t plan, const uint64_t *states, int64_t n_states, void *d_out,
                                        int32_t out_dtype, double *z_out, void *cuda_stream);

@@ -230,30 +230,23 @@ __device__ __forceinline__ void epi_tables_init(EpiTables *tb, const EpiParams &
 // buffer: which of t's two lowest bits run along its contiguous dimension.
 enum GatherMode { G_VEC4 = 0, G_PAIR01 = 1, G_PAIR02 = 2, G_SCALAR = 3 };
 
-struct StagePick {
-    int rowmajor;  // 1: staging [row][col] (columns contiguous), 0: [col][row]
-    int gmode;
-};
-
-// Choose the staging orientation so that the bits that vary across the
-// lanes of a warp (t bits 2..6) and the thread's own low bits fall on the
-// contiguous dimension as far as possible: conflict-free, vectorised
-// gathers.  `lowRc` / `lowCc` mark the row / column bits of t.
 __host__ __device__ inline int gather_mode(uint32_t contig) {
     const bool b0 = contig & 1u, b1 = contig & 2u;
     return (b0 && b1) ? G_VEC4 : b0 ? G_PAIR01 : b1 ? G_PAIR02 : G_SCALAR;
 }
 
-__host__ __device__ inline StagePick pick_staging(uint32_t lowRc, uint32_t lowCc) {
-    StagePick p;
+// Choose the staging orientation (1: [row][col], columns contiguous; 0:
+// [col][row]) so that the bits that vary across the lanes of a warp (t bits
+// 2..6) and the thread's own low bits fall on the contiguous dimension as far
+// as possible: conflict-free, vectorised gathers.  `lowRc` / `lowCc` mark the
+// row / column bits of t.
+__host__ __device__ inline int staging_rowmajor(uint32_t lowRc, uint32_t lowCc) {
     int rows = 0, cols = 0;
     for (int k = 0; k < 7; ++k) {
         rows += (lowRc >> k) & 1u;
         cols += (lowCc >> k) & 1u;
     }
-    p.rowmajor = cols >= rows ? 1 : 0;
-    p.gmode = gather_mode(p.rowmajor ? lowCc : lowRc);
-    return p;
+    return cols >= rows ? 1 : 0;
 }
 
 // Store VW (1, 2 or 4) consecutive values of an epilogue in output mode MODE

@@ -114,7 +114,6 @@ int epi_mode_of(int storage) {
         case ST_BF16: return EPI_BF16;
         case ST_BF16X2: return EPI_BF16X2;
         case ST_TF32: return EPI_TF32;
-        case ST_F64: return EPI_Z;
         default: return EPI_F32;
     }
 }
@@ -337,7 +336,7 @@ int exec_epi_mode(int storage) { return epi_mode_of(storage); }
 int step_out_esize(const Plan &p, const StepPlan &st) {
     if (st.final) return 4;
     const int sg = p.tensors[st.c].storage;
-    return (sg == ST_BF16 || sg == ST_BF16X2) ? 2 : (sg == ST_F64 ? 8 : 4);
+    return (sg == ST_BF16 || sg == ST_BF16X2) ? 2 : 4;
 }
 
 tqc_status exec_autotune(Plan *p, void *d_out, int out_dtype, cudaStream_t s) {

@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(INGEST_THREADS) ingest_kernel(const __grid_con
     const int blocks = m.blk[j + 1] - m.blk[j], block = (int)blockIdx.x - m.blk[j];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (g.reduce_bits > 0) {
-        const bool cta = g.vec == INGEST_THREADS;  // threads per destination
+        const bool cta = g.sum_threads == INGEST_THREADS;
         const int64_t nx = 1ll << g.reduce_bits, n_dst = 1ll << g.nbits;
         const int64_t w0 = cta ? block : (int64_t)block * (INGEST_THREADS / 32) + warp;
         for (int64_t d = w0; d < n_dst; d += cta ? blocks : (int64_t)blocks * (INGEST_THREADS / 32)) {
@@ -691,7 +691,7 @@ SmallkLayout smallk_layout(const EpiParams &e) {
         for (int i = 0; i < n; ++i) m &= m - 1;
         return (uint32_t)__builtin_ctz(m);
     };
-    L.rowmajor = pick_staging(e.lowRc, e.lowCc).rowmajor;
+    L.rowmajor = staging_rowmajor(e.lowRc, e.lowCc);
     L.direct = 0;
     if (run(mC) >= 4 && lanes(1) >= 1) {
         L.direct = 1;
@@ -838,8 +838,8 @@ cudaError_t launch_ingest(const IngestArgs *g, int n, cudaStream_t s) {
             int64_t threads;
             if (a.reduce_bits > 0) {
                 // a CTA per destination when a warp each would leave SMs idle
-                a.vec = a.nbits < 10 && a.reduce_bits >= 8 ? INGEST_THREADS : 32;
-                threads = (int64_t)a.vec << a.nbits;  // (2^5 threads for each of 2^26 destinations and more)
+                a.sum_threads = a.nbits < 10 && a.reduce_bits >= 8 ? INGEST_THREADS : 32;
+                threads = (int64_t)a.sum_threads << a.nbits;  // (2^5 threads for each of 2^26 destinations and more)
             } else {
                 ingest_vec(a);
                 threads = (1ll << a.nbits) / a.vec;

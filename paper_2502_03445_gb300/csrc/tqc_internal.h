@@ -245,8 +245,7 @@ enum EpiMode {
     EPI_F64_SET = 4,    // first slice of the FP64 slice sum
     EPI_F64_ADD = 5,    // further slices
     EPI_OUT_F32 = 6,    // final output, scaled
-    EPI_OUT_F64 = 7,    // final output, scaled, FP64
-    EPI_Z = 8           // scalar-network step (FP64, unscaled)
+    EPI_OUT_F64 = 7     // final output, scaled, FP64
 };
 
 struct EpiParams {
@@ -291,6 +290,7 @@ struct IngestArgs {
     // bits 0 and 1 are destination bits vb[0], vb[1], then left out of srcpos)
     int32_t vec = 1;
     int8_t vb[2] = {0, 0};
+    int32_t sum_threads = 32;    // set by the launch: threads that share one sum (a warp or a CTA)
 };
 
 // A step of the total-mass network: C[r, c] = sum_k A[r, k] B[c, k], FP64,

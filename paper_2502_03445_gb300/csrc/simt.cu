@@ -422,11 +422,14 @@ __device__ __forceinline__ void zfinal(const double *zslice, int n, int n_cuts, 
 
 // A whole small network in one launch: a cluster of ZN_CTAS CTAs with a
 // cluster barrier between steps (a launch each took longer than their work:
-// three
-// steps and the sum of a 15-qubit network 41 -> 8.6 us, a 24-qubit one's four
-// 134 -> 21 us, both with the FP64 work on eight SMs, not one).
+// three steps and the sum of a 15-qubit network 41 -> 8.6 us, a 24-qubit one's
+// four 134 -> 21 us, both with the FP64 work on eight SMs, not one).  More
+// multiply-adds take a launch per step, which has every SM for a step of many
+// outputs (one of few leaves most idle in either form: a sum over K goes to one
+// warp): 2^14 multiply-adds 16 us in either, 2^16 25 against 43, 2^18 53 against
+// 130.
 constexpr int ZN_CTAS = 8, ZN_MAX = 16, ZN_THREADS = 256;
-constexpr double ZN_MAX_MACS = 1 << 18;  // more: one launch per step, over every SM
+constexpr double ZN_MAX_MACS = 1 << 15;
 struct ZNetArgs {
     ZStep step[ZN_MAX];
     int32_t n_steps;
